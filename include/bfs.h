@@ -114,7 +114,7 @@ typedef struct bfs_tuning {
   int32_t warp_degree;   /* TD_BINNED: degree from which a vertex gets a warp (default 32) */
   int32_t cta_degree;    /* TD_BINNED: degree from which a vertex gets a CTA (default 256) */
   int32_t pull_thread_degree; /* PULL: top entries of a row each lane tests alone before the warp-wide scan
-                                 (1..4, larger values act as 4; default 4) */
+                                 (1..4, larger values act as 4; default 4; a row's probe record holds three, so 4 acts as 3) */
   int32_t chunk_degree;  /* top-down: vertices above this degree are split into grid-wide chunks of 1024
                             edges (>= 1024, default 1024) */
   float alpha;           /* heuristic: go PULL when frontier edges * alpha' > unvisited edges and the

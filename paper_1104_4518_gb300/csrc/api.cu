@@ -286,6 +286,8 @@ static int make_graph_from_device_csr(int64_t* d_off, int32_t* d_adj, int32_t n,
   // no arc enters a dead vertex; the big-row chunks serve the batched pull, which scans in-rows
   if (!rc) rc = compute_dead_bits(g->d_toff, n, g->d_dead, nullptr);
   if (!rc) rc = build_big_chunks(g->d_toff, n, nnz, nullptr, &g->d_big, &g->nbig);
+  // the pull works without probe records, only slower: a graph that leaves no room for them does without
+  if (!rc) rc = build_probe_records(g->d_toff, g->d_tadj, n, g->d_dead, nullptr, &g->d_probe, &g->d_rank);
   if (!rc) {
     err = cudaDeviceSynchronize();
     if (err != cudaSuccess) rc = cuda_fail(err, "edgeless-vertex bitmap");
@@ -293,6 +295,8 @@ static int make_graph_from_device_csr(int64_t* d_off, int32_t* d_adj, int32_t n,
   if (rc) {
     if (g->d_dead) cudaFree(g->d_dead);
     if (g->d_big) cudaFree(g->d_big);
+    if (g->d_probe) cudaFree(g->d_probe);
+    if (g->d_rank) cudaFree(g->d_rank);
     cudaFree(g->d_part_base);
     delete g;
     return rc;
@@ -531,6 +535,8 @@ void bfs_graph_destroy(bfs_graph* g) {
   if (g->d_part_base) cudaFree(g->d_part_base);
   if (g->d_dead) cudaFree(g->d_dead);
   if (g->d_big) cudaFree(g->d_big);
+  if (g->d_probe) cudaFree(g->d_probe);
+  if (g->d_rank) cudaFree(g->d_rank);
   free_tiles(g->tiles);
   free_half(g);
   delete g;

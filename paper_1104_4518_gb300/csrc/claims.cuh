@@ -24,9 +24,10 @@ namespace bfsint {
 
 constexpr int kClaimBlock = 512;
 constexpr int kClaimWarps = kClaimBlock / 32;
-constexpr int kQBuf = 6144;               // per-CTA buffer of next-frontier vertices (top-down claims)
+constexpr int kQBuf = 4352;               // per-CTA buffer of next-frontier vertices (top-down claims)
+// The buffers are sized so that two CTAs of the level loop leave 124 KB of L1.
 constexpr int kWQBuf = 256;               // per-warp buffer of next-frontier vertices (pull claims)
-constexpr int kBigBuf = 2 * kClaimBlock;  // per-CTA buffer of claimed vertices above the chunk degree
+constexpr int kBigBuf = kClaimBlock;      // per-CTA buffer of claimed vertices above the chunk degree
 static_assert(kQBuf >= 2 * 64 * 33, "the batched transpose tiles live in the CTA buffer");
 
 struct Claims {

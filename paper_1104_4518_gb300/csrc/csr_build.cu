@@ -13,6 +13,7 @@
 //      "first of its value" flags gives every kept key its slot, the low b
 //      bits are the column, and the row changes between consecutive kept keys
 //      give the int64 row offsets.
+#include <algorithm>
 #include <cstdio>
 
 #include "device_common.cuh"
@@ -384,6 +385,30 @@ __global__ void big_chunks_kernel(const int64_t* __restrict__ off, int32_t n, in
   }
 }
 
+// cnt[w] = vertices of bitmap word w with entries.
+__global__ void live_count_kernel(const uint32_t* __restrict__ dead, long long nwords, uint32_t* __restrict__ cnt) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x; w < nwords; w += stride) cnt[w] = __popc(~dead[w]);
+}
+
+// One warp per bitmap word: the records of its vertices, packed, and the word's rank.
+__global__ void probe_records_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
+                                     const uint32_t* __restrict__ dead, const int64_t* __restrict__ pos,
+                                     long long nwords, int4* __restrict__ out, uint32_t* __restrict__ rank) {
+  const int lane = threadIdx.x & 31;
+  const long long stride = (long long)gridDim.x * blockDim.x / 32;
+  for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32; w < nwords; w += stride) {
+    const uint32_t live = ~dead[w];  // the bits past n are dead
+    const int64_t base = pos[w];
+    if (lane == 0) rank[w] = (uint32_t)base;
+    if ((live >> lane) & 1u) {
+      const long long v = w * 32 + lane, b = off[v], e = off[v + 1], d = e - b;
+      out[base + __popc(live & bfsdev::lanemask_lt())] =
+          make_int4((int)d, adj[e - 1], d > 1 ? adj[e - 2] : 0, d > 2 ? adj[e - 3] : 0);
+    }
+  }
+}
+
 int bits_for(int32_t n) {
   int b = 1;
   while (b < 31 && ((int64_t)1 << b) < (int64_t)n) ++b;
@@ -552,6 +577,38 @@ int compute_dead_bits(const int64_t* d_off, int32_t n, uint32_t* d_dead, cudaStr
   if (int e = current_device_info(&di)) return e;
   dead_bits_kernel<<<di.sm_count * 4, 256, 0, s>>>(d_off, n, ((long long)n + 31) / 32, d_dead);
   BFS_CUDA_TRY(cudaGetLastError());
+  return BFS_OK;
+}
+
+int build_probe_records(const int64_t* d_off, const int32_t* d_adj, int32_t n, const uint32_t* d_dead, cudaStream_t s,
+                        int4** d_probe, uint32_t** d_rank) {
+  *d_probe = nullptr;
+  *d_rank = nullptr;
+  DeviceInfo di;
+  if (int e = current_device_info(&di)) return e;
+  const long long nwords = ((long long)n + 31) / 32;
+  uint32_t* rank = nullptr;
+  int64_t* pos = nullptr;
+  int4* rec = nullptr;
+  if (dev_alloc((void**)&rank, sizeof(uint32_t) * nwords, "record ranks")) return BFS_OK;
+  if (dev_alloc((void**)&pos, sizeof(int64_t) * nwords, "record positions")) return cudaFree(rank), BFS_OK;
+  live_count_kernel<<<di.sm_count * 4, 256, 0, s>>>(d_dead, nwords, rank);
+  long long total = 0;
+  int rc = exclusive_scan_u32(rank, nwords, pos, s, &total);
+  if (!rc && !dev_alloc((void**)&rec, sizeof(int4) * (size_t)std::max(total, 1ll), "probe records")) {
+    probe_records_kernel<<<di.sm_count * 8, 256, 0, s>>>(d_off, d_adj, d_dead, pos, nwords, rec, rank);
+    cudaError_t err = cudaGetLastError();
+    if (err == cudaSuccess) err = cudaStreamSynchronize(s);
+    if (err != cudaSuccess) rc = cuda_fail(err, "probe records");
+  }
+  cudaFree(pos);
+  if (rc || !rec) {
+    cudaFree(rank);
+    if (rec) cudaFree(rec);
+    return rc;
+  }
+  *d_probe = rec;
+  *d_rank = rank;
   return BFS_OK;
 }
 

@@ -136,6 +136,10 @@ struct bfs_graph {
   int64_t* d_toff = nullptr;  // rows of in-neighbours: the transpose when directed, else d_off
   int32_t* d_tadj = nullptr;
   uint32_t* d_dead = nullptr;  // bitmap of vertices no arc enters (tail bits set)
+  // probe records, or null: per vertex that an arc enters (in id order) its in-degree, then its in-row's largest
+  // three ids (0 past the row); d_rank[w] = records of the vertices before bitmap word w
+  int4* d_probe = nullptr;
+  uint32_t* d_rank = nullptr;
   int64_t* d_big = nullptr;    // (v << 32 | c) for every kChunkEdges-entry chunk c of rows longer than kChunkEdges
   int64_t nbig = 0;
   int32_t parts = 1;
@@ -191,6 +195,10 @@ int build_transpose(const int64_t* d_off, const int32_t* d_adj, int32_t n, int64
                     int64_t** d_toff, int32_t** d_tadj);
 // Bitmap of the vertices without edges (bits beyond n set), one word per 32 vertices.
 int compute_dead_bits(const int64_t* d_off, int32_t n, uint32_t* d_dead, cudaStream_t s);
+// Probe record of every non-empty row: its length and its last three entries (the largest ids), 0 past the row.
+// d_dead is the bitmap of the empty rows.  Without room for them *d_probe and *d_rank stay null.  Synchronises s.
+int build_probe_records(const int64_t* d_off, const int32_t* d_adj, int32_t n, const uint32_t* d_dead, cudaStream_t s,
+                        int4** d_probe, uint32_t** d_rank);
 // Chunk items of every row longer than kChunkEdges (order unspecified); *count receives their number.
 int build_big_chunks(const int64_t* d_off, int32_t n, int64_t nnz, cudaStream_t s, int64_t** items, int64_t* count);
 // Adds off_shift to n_part offsets and id_shift to nnz_part ids (union building).

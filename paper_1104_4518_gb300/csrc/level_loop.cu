@@ -26,13 +26,11 @@
 //     kChunkEdges edges, one CTA each.
 //   pull: for every vertex v not yet reached, scan its sorted row from the
 //     largest id down; the first neighbour in f_k is the max-id parent.  One
-//     warp owns a chunk of 32 bitmap words (1,024 vertices) at a time, so nxt /
-//     vis words are written by their owner lane without atomics; the chunk's
-//     live rows are dealt to the lanes, two per lane.  Each lane first probes
-//     the top entries of its rows; rows still open are then scanned by the
-//     whole warp, 32 entries per step, packed across rows by a warp prefix sum
-//     (per-row early exit is kept).  Vertices without edges are marked visited
-//     at init, so pull levels never touch them.
+//     warp owns a chunk of bitmap words at a time; the chunk's live rows are
+//     dealt to the lanes, two per lane, and first tested against their probe
+//     record (the row's largest ids); rows still open are collected per warp and
+//     scanned one per lane.  Vertices without edges are marked
+//     visited at init, so pull levels never touch them.
 #include <cooperative_groups.h>
 #include <cooperative_groups/scan.h>
 
@@ -128,12 +126,18 @@ struct LoopParams {
   const int64_t* __restrict__ t_dir_jc;
   const int64_t* __restrict__ t_dir_ir;
   int32_t t_rb_bits, t_cb_bits, t_nrb, t_ncb;
-  int32_t tile_smem_off;  // byte offset of the tiled phase's slices in dynamic shared memory
+  int32_t phase_smem_off;  // byte offset of the pull / tiled phase's area in dynamic shared memory
+  const int4* __restrict__ probe;  // per vertex an arc enters: in-degree and its row's largest three ids, or null
+  const uint32_t* __restrict__ rank;  // per bitmap word: the records before it
+  int32_t pull_words;              // bitmap words per pull chunk
+  int32_t fr_shift;                // pull: log2 of the vertices per shared-memory frontier bit
+  unsigned fr_limit;               // pull: largest frontier summarised in shared memory when fr_shift > 0
 };
 
 // Per-thread accumulation of the next frontier's counters.
 struct Acc {
-  unsigned long long edges = 0, b0 = 0, b1 = 0, b2 = 0;
+  unsigned long long edges = 0;
+  unsigned b0 = 0, b1 = 0, b2 = 0;  // one thread claims fewer than 2^32 vertices
 };
 
 __device__ __forceinline__ void acc_vertex(Acc& a, long long deg) {
@@ -168,85 +172,6 @@ __device__ __forceinline__ void td_visit(const LoopParams& p, const uint32_t* cu
   claim_topdown(p, k + 1, w, we - wb, acc, cl);
 }
 
-// Warp-cooperative descending scan of the rows still open in a warp: lane r
-// owns row r with entries [b, t) not yet examined (t exclusive, scanned from
-// t-1 down).  Every step the open rows' next entries (at most kCoopRow per
-// row) are packed into kCoopSteps x 32 slots by a prefix sum; slot g is
-// examined by lane g % 32 in sub-step g / 32, so every lane has kCoopSteps
-// adjacency loads and bitmap loads in flight.  A row whose slots hold a hit
-// takes the hit in its lowest slot (its highest position, i.e. its largest
-// id) and closes.  All lanes call it; returns the row's hit or -1.  status and
-// n serve the bounds-checking build's check of every id the scan loads.
-#ifndef BFS_COOP_STEPS
-#define BFS_COOP_STEPS 1
-#endif
-constexpr int kCoopSteps = BFS_COOP_STEPS;
-constexpr int kCoopRow = 32 * kCoopSteps;
-
-__device__ __forceinline__ int scan_desc_coop(const int32_t* __restrict__ adj, const uint32_t* bm, long long b,
-                                              long long t, bool open, int hit, int lane, int* status, int n) {
-  unsigned pm = __ballot_sync(kFull, open);
-  while (pm) {
-    const int rc = open ? (int)min(t - b, (long long)kCoopRow) : 0;
-    int incl = rc;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += y;
-    }
-    const int excl = incl - rc;
-    const int total = __shfl_sync(kFull, incl, 31);
-    int u[kCoopSteps];
-    bool h[kCoopSteps];
-#pragma unroll
-    for (int sstep = 0; sstep < kCoopSteps; ++sstep) {
-      const int slot = sstep * 32 + lane;
-      // owner row of this slot: the last row whose prefix is <= slot
-      int r = 0;
-#pragma unroll
-      for (int st = 16; st >= 1; st >>= 1) {
-        const int c = r + st;
-        const int ec = __shfl_sync(kFull, excl, c & 31);
-        if (c < 32 && ec <= slot) r = c;
-      }
-      const long long tr = __shfl_sync(kFull, t, r);
-      const int er = __shfl_sync(kFull, excl, r);
-      u[sstep] = slot < total ? __ldg(&adj[tr - 1 - (slot - er)]) : -1;
-    }
-#pragma unroll
-    for (int sstep = 0; sstep < kCoopSteps; ++sstep) {
-      const bool live = bfsdev::kBoundsCheck
-                            ? sstep * 32 + lane < total && bfsdev::in_range(status, bfsdev::kSitePull, u[sstep], n)
-                            : u[sstep] >= 0;
-      h[sstep] = live && ((bm[u[sstep] >> 5] >> (u[sstep] & 31)) & 1u);
-    }
-    // this lane's row takes slots [excl, excl + cons) of the kCoopRow slots
-    const int cons = max(0, min(rc, kCoopRow - excl));
-    int found = -1;
-#pragma unroll
-    for (int sstep = 0; sstep < kCoopSteps; ++sstep) {
-      const unsigned hm = __ballot_sync(kFull, h[sstep]);
-      const int lo = max(excl - sstep * 32, 0), hi = min(excl + cons - sstep * 32, 32);
-      unsigned seg = 0u;
-      if (hi > lo) seg = (hi - lo == 32 ? kFull : ((1u << (hi - lo)) - 1u)) << lo;
-      const unsigned mine = hm & seg;
-      const int hv = __shfl_sync(kFull, u[sstep], mine ? __ffs(mine) - 1 : 0);
-      if (found < 0 && mine) found = hv;
-    }
-    if (open) {
-      if (found >= 0) {
-        hit = found;
-        open = false;
-      } else {
-        t -= cons;
-        if (t <= b) open = false;
-      }
-    }
-    pm = __ballot_sync(kFull, open);
-  }
-  return hit;
-}
-
 // 64-bit warp sum.
 __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
 #pragma unroll
@@ -261,15 +186,17 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
 // and its buffered chunk items go to level knext with one atomic each.
 template <typename S>
 __device__ __forceinline__ void end_phase(const LoopParams& p, int knext, Acc& acc, S& sm) {
-  const bool mine = (acc.edges | acc.b0 | acc.b1 | acc.b2) != 0;
+  const bool mine = (acc.b0 | acc.b1 | acc.b2) != 0;
   if (__syncthreads_or(mine)) {
-    const unsigned long long e = warp_sum_u64(acc.edges), b0 = warp_sum_u64(acc.b0), b1 = warp_sum_u64(acc.b1),
-                             b2 = warp_sum_u64(acc.b2);
+    // n < 2^31 vertices in all: a warp's counts fit 32 bits
+    const unsigned long long e = warp_sum_u64(acc.edges);
+    const unsigned b0 = __reduce_add_sync(kFull, acc.b0), b1 = __reduce_add_sync(kFull, acc.b1),
+                   b2 = __reduce_add_sync(kFull, acc.b2);
     if ((threadIdx.x & 31) == 0 && (e | b0 | b1 | b2)) {
       atomicAdd(&sm.acc[0], e);
-      atomicAdd(&sm.acc[1], b0);
-      atomicAdd(&sm.acc[2], b1);
-      atomicAdd(&sm.acc[3], b2);
+      atomicAdd(&sm.acc[1], (unsigned long long)b0);
+      atomicAdd(&sm.acc[2], (unsigned long long)b1);
+      atomicAdd(&sm.acc[3], (unsigned long long)b2);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -291,19 +218,23 @@ struct Smem {
   long long cb, ce;
   int warp_tmp[kWarps + 1];
   unsigned long long acc[4];
-  int tu[kBlock];
-  long long tb[kBlock];
-  int tpref[kBlock + 1];
   Claims cl;
-  uint32_t pull_hits[kWarps][32];  // pull: hit bits of each warp's 32 bitmap words
   __align__(16) float h1[64];  // selector network: hidden layer 1, choice
   int choice;
   unsigned long long next_item;  // top-down: the next chunk item of this CTA
 };
 
 // ---------------- top-down phase ----------------
+// Dynamic shared memory of the top-down and tiled phases: frontier rows of a
+// CTA with the prefix sums of their lengths.
+struct FlatSmem {
+  long long tb[kBlock];
+  int tu[kBlock];
+  int tpref[kBlock + 1];
+};
+
 __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned count, unsigned nchunks, Smem& sm,
-                              Acc& acc, unsigned G) {
+                              FlatSmem& fl, Acc& acc, unsigned G) {
   const uint32_t* cur = p.bits[k % 3];
   uint32_t* nxt = p.bits[(k + 1) % 3];
   const int32_t* Q = p.queue[k % 3];
@@ -390,10 +321,10 @@ __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned 
       const int sdeg = u >= 0 ? (int)deg : 0;
       int excl = 0;
       const int total = block_exclusive_scan(sdeg, sm.warp_tmp, excl);
-      sm.tu[tid] = u;
-      sm.tb[tid] = b;
-      sm.tpref[tid] = excl;
-      if (tid == 0) sm.tpref[kBlock] = total;
+      fl.tu[tid] = u;
+      fl.tb[tid] = b;
+      fl.tpref[tid] = excl;
+      if (tid == 0) fl.tpref[kBlock] = total;
       __syncthreads();
       for (int base = 0; base < total; base += kBlock) {
         const int idx = base + tid;
@@ -401,11 +332,11 @@ __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned 
           int lo = 0, hi = kBlock;  // largest slot with tpref <= idx (and a non-empty row)
           while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
-            if (sm.tpref[mid] <= idx) lo = mid;
+            if (fl.tpref[mid] <= idx) lo = mid;
             else hi = mid;
           }
-          const int ou = sm.tu[lo];
-          td_visit(p, cur, nxt, k, ou, __ldg(&p.adj[sm.tb[lo] + (idx - sm.tpref[lo])]), acc, sm.cl);
+          const int ou = fl.tu[lo];
+          td_visit(p, cur, nxt, k, ou, __ldg(&p.adj[fl.tb[lo] + (idx - fl.tpref[lo])]), acc, sm.cl);
         }
       }
       __syncthreads();
@@ -414,8 +345,26 @@ __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned 
 }
 
 // ---------------- pull phase ----------------
-constexpr int kPullRows = 2;    // live rows per lane in flight
-constexpr int kPullProbes = 4;  // at most this many top entries of each row are probed before the warp scan
+constexpr int kPullRows = 2;       // live rows per lane in flight
+constexpr int kPullProbes = 3;     // top entries of a row tested from its probe record
+constexpr int kFrWords = 2048;     // frontier test in shared memory: 65,536 bits.  8,192 words left the top-down
+                                   // levels' bitmap loads too little L1 (77 K-vertex level: 37 -> 63 us)
+static_assert(kPullProbes == 3, "the unpacking of the probe records below");
+constexpr int kDefer = 112;        // deferred rows a warp can hold; scanned once fewer than 64 more would fit
+constexpr int kScanRefill = 24;    // a deferred scan with this many open rows or fewer takes new ones
+constexpr int kScanOpen = 8;       // a deferred scan with fewer open rows and none left to take hands them back
+constexpr int kWarpRow = 128;      // remaining entries from which a row left open is scanned by the whole warp
+
+// Dynamic shared memory of the pull phase.
+struct __align__(16) PullSmem {
+  uint32_t fr[kFrWords];
+  uint32_t hits[kWarps][32];   // hit bits of each warp's bitmap words
+  uint2 entry[kWarps][32];     // of each warp's bitmap words: the vertices with a record, the records before
+  int4 defer[kWarps][kDefer];  // rows still open after their probe: vertex, entries not yet examined, row start (64 bits)
+};
+
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
 // Position of the r-th (0-based) set bit of m; r < popc(m).
 __device__ __forceinline__ int select_bit(uint32_t m, int r) {
   int pos = 0;
@@ -431,11 +380,11 @@ __device__ __forceinline__ int select_bit(uint32_t m, int r) {
   return pos;
 }
 
-// The idx-th live vertex of a warp's chunk of 32 bitmap words (all lanes call
-// it; lane l holds word l's live bits `live` and the inclusive prefix `incl` of
-// their counts).  Returns the vertex, the owner lane of its word and its bit.
-__device__ __forceinline__ int live_vertex(long long chunk, uint32_t live, int incl, int idx, int& owner,
-                                           uint32_t& bit) {
+// The idx-th live vertex of a warp's chunk of bitmap words that starts at word
+// w0 (all lanes call it; lane l holds word l's live bits `live` and the
+// inclusive prefix `incl` of their counts).  Returns the vertex, the owner lane
+// of its word and its bit.
+__device__ __forceinline__ int live_vertex(int w0, uint32_t live, int incl, int idx, int& owner, uint32_t& bit) {
   int o = 0;  // number of lanes whose inclusive prefix is <= idx: the owner
 #pragma unroll
   for (int st = 16; st >= 1; st >>= 1) {
@@ -448,65 +397,105 @@ __device__ __forceinline__ int live_vertex(long long chunk, uint32_t live, int i
   const int b = select_bit(lo, max(idx - excl_o, 0));
   owner = o;
   bit = 1u << b;
-  return (int)((chunk * 32 + o) * 32 + b);
+  return (w0 + o) * 32 + b;
 }
 
-// The max-id frontier neighbour of R rows per lane (v[r] < 0: no row): the
-// rows' bounds, then a probe of the top `probe` (<= P) entries of every row with all their
-// adjacency loads and then all their frontier-word loads in flight together,
-// then the warp's cooperative descending scan of the rows still open.  R = 2,
-// P = 4 is what the 64-register budget holds without spills (R = 3 or 4 with
-// P = 2 spilled and ran 5 % and 16 % slower on R-MAT scale 26).
-template <int R, int P>
-__device__ __forceinline__ void pull_rows(const LoopParams& p, const uint32_t* cur, int lane, int probe,
-                                          const int (&v)[R], int (&h)[R], long long (&d)[R]) {
-  long long b[R], e[R];
+// Where a pull level tests "is u in f_k".
+enum FrontierMode : int {
+  kFrGlobal = 0,   // the bitmap in global memory (L2)
+  kFrExact = 1,    // a copy of the whole bitmap in shared memory (n <= 32 * kFrWords)
+  kFrSummary = 2,  // shared memory holds one bit per 2^fr_shift vertices; a set one is confirmed in the bitmap
+};
+
+struct FrontierTest {
+  const uint32_t* cur;
+  const uint32_t* fr;
+  int shift;
+  FrontierMode mode;
+};
+
+// Which of the N ids u (those with their bit in `valid`) are in f_k, as a bit
+// mask; the loads of one call are in flight together.
+template <int N>
+__device__ __forceinline__ unsigned in_frontier(const LoopParams& p, const FrontierTest& f, const int (&u)[N],
+                                                unsigned valid) {
+  if constexpr (bfsdev::kBoundsCheck) {
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    b[r] = e[r] = 0;
-    if (v[r] >= 0) {
-      b[r] = __ldg(&p.toff[v[r]]);
-      e[r] = __ldg(&p.toff[v[r] + 1]);
+    for (int q = 0; q < N; ++q)
+      if (((valid >> q) & 1u) && !bfsdev::in_range(p.status, bfsdev::kSitePull, u[q], p.n)) valid &= ~(1u << q);
+  }
+  unsigned m = valid;
+  if (f.mode != kFrGlobal) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const unsigned y = (unsigned)u[q] >> f.shift;
+      const unsigned t = (f.fr[(y >> 5) & (kFrWords - 1)] >> (y & 31)) & 1u;
+      m &= ~((t ^ 1u) << q);
     }
+    if (f.mode == kFrExact) return m;
   }
-  int np[R];
-  int u[R][P];
-  uint32_t x[R][P];
+  uint32_t x[N];
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    np[r] = v[r] >= 0 ? (int)min((long long)probe, e[r] - b[r]) : 0;
+  for (int q = 0; q < N; ++q) x[q] = ((m >> q) & 1u) ? f.cur[u[q] >> 5] : 0u;
+  unsigned h = 0;
 #pragma unroll
-    for (int q = 0; q < P; ++q) u[r][q] = q < np[r] ? __ldg(&p.tadj[e[r] - 1 - q]) : 0;
-  }
-#pragma unroll
-  for (int r = 0; r < R; ++r)
-#pragma unroll
-    for (int q = 0; q < P; ++q)
-      x[r][q] = q < np[r] && bfsdev::in_range(p.status, bfsdev::kSitePull, u[r][q], p.n) ? cur[u[r][q] >> 5] : 0u;
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    h[r] = -1;
-#pragma unroll
-    for (int q = 0; q < P; ++q)
-      if (q < np[r] && h[r] < 0 && ((x[r][q] >> (u[r][q] & 31)) & 1u)) h[r] = u[r][q];
-  }
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const long long t = e[r] - np[r];
-    h[r] = scan_desc_coop(p.tadj, cur, b[r], t, v[r] >= 0 && h[r] < 0 && t > b[r], h[r], lane, p.status, p.n);
-    d[r] = e[r] - b[r];
-  }
+  for (int q = 0; q < N; ++q) h |= ((x[q] >> (u[q] & 31)) & 1u) << q;
+  return h;
 }
 
-// Bookkeeping of a vertex v reached by the pull (hit = its parent): outputs,
-// counters, chunk items, the owner word's hit bit and the warp's queue buffer.
-__device__ __forceinline__ void pull_claim(const LoopParams& p, int knext, int v, int hit, long long deg_in,
-                                           uint32_t* hitw, int owner, uint32_t bit, Acc& acc, Claims& cl, int* wq,
-                                           int& nbuf, int lane) {
+// Four consecutive entries of the in-adjacency from index i, which is a
+// multiple of four entries from a 16-byte boundary; entries outside the array
+// read as 0.
+__device__ __forceinline__ int4 load_entries4(const LoopParams& p, long long i) {
+  if (i >= 0 && i + 4 <= p.nnz) return __ldg(reinterpret_cast<const int4*>(p.tadj + i));
+  int4 r = make_int4(0, 0, 0, 0);
+  if (i >= 0 && i < p.nnz) r.x = __ldg(p.tadj + i);
+  if (i + 1 >= 0 && i + 1 < p.nnz) r.y = __ldg(p.tadj + i + 1);
+  if (i + 2 >= 0 && i + 2 < p.nnz) r.z = __ldg(p.tadj + i + 2);
+  if (i + 3 >= 0 && i + 3 < p.nnz) r.w = __ldg(p.tadj + i + 3);
+  return r;
+}
+
+// Start of the aligned group of four entries that holds entry i.
+__device__ __forceinline__ long long group_start(const LoopParams& p, long long i) {
+  const int a = (int)((reinterpret_cast<uintptr_t>(p.tadj) >> 2) & 3u);
+  return ((i + a) & ~3ll) - a;
+}
+
+// The whole warp scans entries [b, t) of one row from the top, 128 per step;
+// returns the first frontier neighbour (the largest id) or -1.
+__device__ __forceinline__ int scan_row_warp(const LoopParams& p, const FrontierTest& f, long long b, long long t,
+                                             int lane) {
+  while (t > b) {
+    const long long top = group_start(p, t - 1), g = top - 4 * lane;
+    int u[4] = {0, 0, 0, 0};
+    unsigned valid = 0;
+    if (g + 3 >= b) {
+      const int4 e = load_entries4(p, g);
+      u[0] = e.w, u[1] = e.z, u[2] = e.y, u[3] = e.x;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) valid |= (g + 3 - q >= b && g + 3 - q < t) ? 1u << q : 0u;
+    }
+    const unsigned h = in_frontier<4>(p, f, u, valid);
+    const unsigned any = __ballot_sync(kFull, h != 0);
+    if (any) {
+      const int q = __ffs(h) - 1;
+      const int mine = q == 0 ? u[0] : q == 1 ? u[1] : q == 2 ? u[2] : u[3];
+      return __shfl_sync(kFull, mine, __ffs(any) - 1);
+    }
+    t = top - 124;
+  }
+  return -1;
+}
+
+// Bookkeeping of vertices reached by the pull (one per lane where hit >= 0, its
+// parent): outputs, counters, chunk items and the warp's queue buffer.  deg_in
+// is the in-degree.
+__device__ __forceinline__ void pull_claim(const LoopParams& p, int knext, int v, int hit, long long deg_in, Acc& acc,
+                                           Claims& cl, int* wq, int& nbuf, int lane) {
   if (hit >= 0) {
     p.parent[v] = hit;
     p.level[v] = knext;
-    atomicOr(&hitw[owner], bit);
     // out-degree: the next level expands v's out-row (the row scanned here when undirected)
     const long long deg = p.directed ? __ldg(&p.off[v + 1]) - __ldg(&p.off[v]) : deg_in;
     acc_vertex(acc, deg);
@@ -515,45 +504,171 @@ __device__ __forceinline__ void pull_claim(const LoopParams& p, int knext, int v
   warp_enqueue(p, knext, wq, nbuf, hit >= 0, v, lane, false);
 }
 
-// Dense-frontier SpMV over the unvisited rows.  A warp takes a chunk of 32
-// bitmap words (1,024 vertices) at a time: lane l loads word l of `vis` and of
-// `cur`, and the chunk's live vertices (not reached, not edgeless) are dealt to
-// the lanes 64 at a time, two rows per lane, so that every lane carries an open
-// row however sparse the live vertices are (in the last pull levels of a
-// scale-26 R-MAT graph most words hold one live vertex).  Each word's hits are
-// gathered in shared memory and its owner lane writes the word's `nxt` and
-// `vis` (no global atomics on the bitmaps).  Rows without a frontier
-// neighbour near their top make some chunks far dearer than others, so the
-// second half of a large level's chunks is handed out dynamically: with an
-// all-static deal the level waited on its slowest warps (R-MAT scale 26: 126.4
-// ms for the 64 bench roots, 121.8 with the dynamic tail), and with an
-// all-dynamic one the cursor's atomics, all at once at the start of every
-// level, made the 2^27-edge edgefactor-16 and -64 graphs 11 % and 15 % slower.
-__device__ void pull_phase(const LoopParams& p, int k, Smem& sm, Acc& acc, unsigned G) {
-  const uint32_t* cur = p.bits[k % 3];
+// Scans the warp's deferred rows, one per lane: eight entries (two aligned
+// 16-byte loads) per step and row, from the top.  A lane whose row is done
+// takes the next of the list, so that the lanes stay busy however different
+// the rows' lengths are.  Once the list is empty and fewer than kScanOpen rows
+// are open, those go back to the list (with `flush`: are scanned to their
+// end), except that one with kWarpRow or more entries left is scanned by the
+// whole warp.
+__device__ __forceinline__ void scan_deferred(const LoopParams& p, const FrontierTest& f, int knext, uint32_t* nxt,
+                                              int4* defer, int& nd, bool flush, Acc& acc, Claims& cl, int* wq,
+                                              int& nbuf, int lane) {
+  asm volatile("cp.async.wait_all;" ::: "memory");  // the row starts of the list
+  __syncwarp();
+  int v = -1, hit = -1;
+  long long b = 0, t = 0;
+  bool open = false;
+  for (;;) {
+    unsigned m = __ballot_sync(kFull, open);
+    if (__popc(m) <= kScanRefill) {
+      if (nd == 0 && __popc(m) < kScanOpen) {
+        for (unsigned big = __ballot_sync(kFull, open && t - b >= kWarpRow); big; big &= big - 1u) {
+          const int l = __ffs(big) - 1;
+          const int r = scan_row_warp(p, f, __shfl_sync(kFull, b, l), __shfl_sync(kFull, t, l), lane);
+          if (lane == l) {
+            hit = r;
+            open = false;
+          }
+        }
+      }
+      if (__any_sync(kFull, hit >= 0)) {
+        long long deg = 0;
+        if (hit >= 0) {
+          atomicOr(&nxt[v >> 5], 1u << (v & 31));
+          if (!p.directed) deg = __ldg(&p.toff[v + 1]) - b;
+        }
+        pull_claim(p, knext, v, hit, deg, acc, cl, wq, nbuf, lane);
+        hit = -1;
+      }
+      m = __ballot_sync(kFull, open);
+      if (nd > 0) {
+        const int i = nd - 1 - __popc(~m & bfsdev::lanemask_lt());
+        if (!open && i >= 0) {
+          const int4 d = defer[i];
+          v = d.x;
+          b = (long long)(((unsigned long long)(unsigned)d.w << 32) | (unsigned)d.z);
+          t = b + d.y;
+          open = true;
+        }
+        nd = max(0, nd - __popc(~m));
+      } else if (m == 0) {
+        break;
+      } else if (!flush && __popc(m) < kScanOpen) {
+        __syncwarp();  // every lane has read its entry
+        if (open)
+          defer[__popc(m & bfsdev::lanemask_lt())] = make_int4(v, (int)(t - b), (int)b, (int)(b >> 32));
+        nd = __popc(m);
+        break;
+      }
+    }
+    if (open) {
+      const long long g1 = group_start(p, t - 1), g0 = g1 - 4;
+      const int4 e1 = load_entries4(p, g1);
+      int4 e0 = make_int4(0, 0, 0, 0);
+      if (g1 > b) e0 = load_entries4(p, g0);
+      const int u[8] = {e1.w, e1.z, e1.y, e1.x, e0.w, e0.z, e0.y, e0.x};
+      const int skip = (int)(g1 + 4 - t);  // entries of the top group at or above t
+      const int cnt = (int)min((long long)(8 - skip), t - b);
+      const unsigned h = in_frontier<8>(p, f, u, ((1u << cnt) - 1u) << skip);
+      if (h) {
+        const unsigned first = h & (0u - h);
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (first == 1u << q) hit = u[q];
+        open = false;
+      } else {
+        t -= cnt;
+        open = t > b;
+      }
+    }
+  }
+  __syncwarp();
+}
+
+// Dense-frontier SpMV over the unvisited rows.  A warp takes a chunk of
+// pull_words bitmap words (32 vertices each) at a time: lane l loads word l of
+// `vis` and of `cur`, and the chunk's live vertices (not reached, not
+// edgeless) are dealt to the lanes 64 at a time, two rows per lane, so that
+// every lane carries a row however sparse the live vertices are.
+//
+// The top entries of a row come from its probe record (degree and largest
+// three ids, 16 bytes per vertex that an arc enters, built with the graph): on an R-MAT graph's
+// dense level nearly every row ends there, and the records of a chunk are
+// read in order, where the rows' own ends are one DRAM sector each at random.
+// Rows still open go to a list of the warp, their starts fetched into it with
+// cp.async; once it fills, they are scanned one per lane, eight entries per
+// step (scan_deferred), so that a warp has 256 entries in flight instead of
+// the 32 of a scan that packs the open rows into one load per lane.
+//
+// The frontier test reads shared memory where it can: an exact copy of the
+// bitmap up to 65,536 vertices, and above that, for a frontier of at most
+// fr_limit vertices, one bit per 2^fr_shift vertices, which rejects all but a
+// few percent of the entries (the first pull level of a traversal led by hubs
+// tests half a billion entries at scale 26 against a few thousand vertices).
+//
+// Chunk size and deal: a chunk costs its warp about 3.5 us of dependent loads
+// however few live rows it holds, so a graph of up to 32 words per resident
+// warp gives every warp one chunk (32-word chunks for all sizes left 64 of
+// 4,864 warps with work at scale 16), and larger graphs use 32-word chunks.
+// Rows without a frontier neighbour near their top make some chunks far dearer
+// than others, so the second half of a large level's chunks is handed out
+// dynamically (with an all-dynamic deal the cursor's atomics, all at once at
+// the start of a level, cost more than they save).
+//
+// What bounds it: the latency of the chain bitmap words -> record -> frontier
+// test -> row, with 8 warps per scheduler to hide it, and on a dense level
+// at scale 26 DRAM (records, outputs written over their -1 fill).  Measured
+// against a pull that read the rows' bounds and top entries and packed the open
+// rows into one load per lane (level times, R-MAT edgefactor 16): scale 26, f_k
+// of 5,328 vertices 2,341 -> 1,270 us, of 9.6 M 615 -> 373 us, of 2.9 M 713 ->
+// 455 us; scale 22, f_k of 3,946 vertices 162 -> 80 us; scale 16, f_k of 4,525
+// vertices 33 -> 13 us.
+__device__ void pull_phase(const LoopParams& p, int k, unsigned count, Smem& sm, PullSmem& ps, Acc& acc, unsigned G) {
   uint32_t* nxt = p.bits[(k + 1) % 3];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const long long gwarps = (long long)G * kWarps;
   const int knext = k + 1;
   const int probe = min(p.pull_thread_deg, kPullProbes);  // the tuning knob, at most kPullProbes
+  FrontierTest f{p.bits[k % 3], ps.fr, p.fr_shift, kFrGlobal};
+  if (p.fr_shift == 0) {
+    f.mode = kFrExact;
+    for (int i = threadIdx.x; i < p.nwords; i += kBlock) ps.fr[i] = f.cur[i];
+    __syncthreads();
+  } else if (count <= p.fr_limit) {
+    f.mode = kFrSummary;
+    for (int i = threadIdx.x; i < kFrWords / 4; i += kBlock) reinterpret_cast<uint4*>(ps.fr)[i] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    const int32_t* Q = p.queue[k % 3];
+#pragma unroll 4
+    for (unsigned i = threadIdx.x; i < count; i += kBlock) {
+      const unsigned y = (unsigned)Q[i] >> p.fr_shift;
+      atomicOr(&ps.fr[(y >> 5) & (kFrWords - 1)], 1u << (y & 31));
+    }
+    __syncthreads();
+  }
   int* wq = sm.cl.wq[wid];
-  uint32_t* hitw = sm.pull_hits[wid];
-  int nbuf = 0;
+  uint32_t* hitw = ps.hits[wid];
+  uint2* entry = ps.entry[wid];
+  int4* defer = ps.defer[wid];
+  int nbuf = 0, nd = 0;
   // chunk indices fit 32 bits: nwords < 2^26
-  const int nchunks = (p.nwords + 31) / 32, gw = (int)gwarps;
+  const int W = p.pull_words, nchunks = (p.nwords + W - 1) / W, gw = (int)gwarps;
   // Chunks [0, S) are dealt statically (warp i takes i, i + gw, ...), the
   // rest from the level's cursor, each fetch issued one chunk ahead.  With
   // fewer than two chunks per warp the level is all static (S past every chunk).
   const int S = nchunks > 2 * gw ? gw * max(1, (nchunks / 2) / gw) : INT_MAX;
-  for (int c = wid * (int)G + (int)blockIdx.x; c < nchunks;) {
+  for (int c = wid * (int)G + (int)blockIdx.x;;) {
+    const bool more = c < nchunks;  // after the last chunk one more turn scans what is left deferred
     unsigned taken = 0;
-    if (c + gw >= S && lane == 0) taken = (unsigned)atomicAdd(&p.ctr[k % kCtrRing].pad, 1ull);  // used after the chunk
-    const int w = c * 32 + lane;
-    const bool has = w < p.nwords;
+    if (more && c + gw >= S && lane == 0) taken = (unsigned)atomicAdd(&p.ctr[k % kCtrRing].pad, 1ull);  // used after the chunk
+    const int w0 = c * W, w = w0 + lane;
+    const bool has = more && lane < W && w < p.nwords;
     const uint32_t vw = has ? p.vis[w] : 0xffffffffu;
-    const uint32_t cw = has ? cur[w] : 0u;
+    const uint32_t cw = has ? f.cur[w] : 0u;
     const uint32_t visw = vw | cw;
     const uint32_t live = ~visw;
+    if (p.probe != nullptr && has) entry[lane] = make_uint2(~__ldg(&p.dead[w]), __ldg(&p.rank[w]));
     const int cnt = __popc(live);
     int incl = cnt;
 #pragma unroll
@@ -564,25 +679,63 @@ __device__ void pull_phase(const LoopParams& p, int k, Smem& sm, Acc& acc, unsig
     const int total = __shfl_sync(kFull, incl, 31);
     hitw[lane] = 0u;
     __syncwarp();
-    for (int base = 0; base < total; base += 32 * kPullRows) {
-      int v[kPullRows], o[kPullRows], h[kPullRows];
+    for (int base = 0;; base += 32 * kPullRows) {
+      if (nd > kDefer - 32 * kPullRows || !more)
+        scan_deferred(p, f, knext, nxt, defer, nd, !more, acc, sm.cl, wq, nbuf, lane);
+      if (base >= total) break;
+      int v[kPullRows], o[kPullRows], deg[kPullRows], u[kPullRows * kPullProbes];
       uint32_t bit[kPullRows];
-      long long d[kPullRows];
 #pragma unroll
       for (int r = 0; r < kPullRows; ++r) {
         const int i = base + r * 32 + lane;
-        const int lv = live_vertex(c, live, incl, min(i, total - 1), o[r], bit[r]);
+        const int lv = live_vertex(w0, live, incl, min(i, total - 1), o[r], bit[r]);
         v[r] = i < total ? lv : -1;
       }
-      pull_rows<kPullRows, kPullProbes>(p, cur, lane, probe, v, h, d);
+      if (p.probe != nullptr) {
 #pragma unroll
-      for (int r = 0; r < kPullRows; ++r)
-        pull_claim(p, knext, v[r], v[r] >= 0 ? h[r] : -1, d[r], hitw, o[r], bit[r], acc, sm.cl, wq, nbuf, lane);
+        for (int r = 0; r < kPullRows; ++r) {
+          const uint2 en = entry[o[r]];
+          const uint32_t at = en.y + __popc(en.x & (bit[r] - 1u));
+          const int4 rec = v[r] >= 0 ? __ldg(&p.probe[at]) : make_int4(0, 0, 0, 0);
+          deg[r] = rec.x;
+          u[3 * r] = rec.y, u[3 * r + 1] = rec.z, u[3 * r + 2] = rec.w;
+        }
+      } else {  // no records (the static entry point): the same from the row itself
+#pragma unroll
+        for (int r = 0; r < kPullRows; ++r) {
+          const long long b = v[r] >= 0 ? __ldg(&p.toff[v[r]]) : 0, e = v[r] >= 0 ? __ldg(&p.toff[v[r] + 1]) : 0;
+          deg[r] = (int)(e - b);
+#pragma unroll
+          for (int q = 0; q < kPullProbes; ++q) u[3 * r + q] = q < deg[r] ? __ldg(&p.tadj[e - 1 - q]) : 0;
+        }
+      }
+      unsigned valid = 0;  // one test of both rows: all its loads are in flight together
+#pragma unroll
+      for (int r = 0; r < kPullRows; ++r) valid |= ((1u << min(probe, deg[r])) - 1u) << (3 * r);
+      const unsigned found = in_frontier<kPullRows * kPullProbes>(p, f, u, valid);
+#pragma unroll
+      for (int r = 0; r < kPullRows; ++r) {
+        const unsigned h = found >> (3 * r) & 7u;
+        const int hit = h == 0 ? -1 : (h & 1u) ? u[3 * r] : (h & 2u) ? u[3 * r + 1] : u[3 * r + 2];
+        const bool later = hit < 0 && deg[r] > probe;
+        const unsigned m = __ballot_sync(kFull, later);
+        if (later) {
+          int4* d = &defer[nd + __popc(m & bfsdev::lanemask_lt())];
+          *reinterpret_cast<int2*>(d) = make_int2(v[r], deg[r] - probe);
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(d) + 8), "l"(p.toff + v[r]) : "memory");
+        }
+        nd += __popc(m);
+        if (hit >= 0) atomicOr(&hitw[o[r]], bit[r]);
+        pull_claim(p, knext, v[r], hit, deg[r], acc, sm.cl, wq, nbuf, lane);
+      }
+      __syncwarp();
     }
-    __syncwarp();
+    if (!more) break;
     const uint32_t hits = hitw[lane];
     if (has) {
-      if (hits) nxt[w] = hits;
+      // the deferred rows of this word OR their hits in as they are found; the
+      // next level's pull folds nxt into vis, so vis need not hold them yet
+      if (hits) atomicOr(&nxt[w], hits);
       if ((visw | hits) != vw) p.vis[w] = visw | hits;
     }
     __syncwarp();
@@ -608,7 +761,8 @@ __device__ void pull_phase(const LoopParams& p, int k, Smem& sm, Acc& acc, unsig
 // words, levels, counters and the warp queue buffers.
 constexpr int kTileWordsMax = 2048;  // 2^16 rows or columns per tile
 
-__device__ void tiled_phase(const LoopParams& p, int k, Smem& sm, uint32_t* tsm, Acc& acc, unsigned G) {
+__device__ void tiled_phase(const LoopParams& p, int k, Smem& sm, FlatSmem& fl, uint32_t* tsm, Acc& acc,
+                            unsigned G) {
   const uint32_t* cur = p.bits[k % 3];
   uint32_t* nxt = p.bits[(k + 1) % 3];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -654,10 +808,10 @@ __device__ void tiled_phase(const LoopParams& p, int k, Smem& sm, uint32_t* tsm,
         }
         int excl = 0;
         const int total = block_exclusive_scan((int)rlen, sm.warp_tmp, excl);
-        sm.tu[tid] = ul;
-        sm.tb[tid] = rbeg;
-        sm.tpref[tid] = excl;
-        if (tid == 0) sm.tpref[kBlock] = total;
+        fl.tu[tid] = ul;
+        fl.tb[tid] = rbeg;
+        fl.tpref[tid] = excl;
+        if (tid == 0) fl.tpref[kBlock] = total;
         __syncthreads();
         for (int base = 0; base < total; base += kBlock) {
           const int idx = base + tid;
@@ -665,12 +819,12 @@ __device__ void tiled_phase(const LoopParams& p, int k, Smem& sm, uint32_t* tsm,
             int lo = 0, hi = kBlock;  // largest slot with tpref <= idx (a frontier column with rows)
             while (hi - lo > 1) {
               const int mid = (lo + hi) >> 1;
-              if (sm.tpref[mid] <= idx) lo = mid;
+              if (fl.tpref[mid] <= idx) lo = mid;
               else hi = mid;
             }
-            const int r = p.t_ir[sm.tb[lo] + (idx - sm.tpref[lo])];
+            const int r = p.t_ir[fl.tb[lo] + (idx - fl.tpref[lo])];
             if (!((done[r >> 5] >> (r & 31)) & 1u)) {
-              atomicMax(&p.parent[(rb << p.t_rb_bits) + r], (cb << p.t_cb_bits) + sm.tu[lo]);
+              atomicMax(&p.parent[(rb << p.t_rb_bits) + r], (cb << p.t_cb_bits) + fl.tu[lo]);
               atomicOr(&newf[r >> 5], 1u << (r & 31));
               tile_hit = true;
             }
@@ -747,6 +901,10 @@ __device__ __forceinline__ int heuristic_variant(const LoopParams& p, int prev_v
   return (count <= p.small_frontier && small_rows) ? BFS_VARIANT_TD_WARP : BFS_VARIANT_TD_BINNED;
 }
 
+constexpr size_t kFlatBytes = (sizeof(FlatSmem) + 15) / 16 * 16;
+constexpr size_t kPhaseBytes = sizeof(PullSmem);  // the largest phase's area
+static_assert(kPhaseBytes >= kFlatBytes + sizeof(uint32_t) * 3 * kTileWordsMax, "the tiled phase fits the pull's area");
+
 // kTiles: the kernel can run the tiled phase.  Runs that cannot pick the tiled
 // variant launch the instance without it: on R-MAT scale 26 the tiled phase's
 // code alone made the other phases 5 % slower.
@@ -754,11 +912,13 @@ template <bool kTiles>
 __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
   __shared__ Smem sm;
   // dynamic shared memory: the selector network's parameters (BFS_MLP_PARAMS
-  // floats) when the learned selector is on, then the tiled phase's slices
-  // (3 * kTileWordsMax words) when tiles are present
+  // floats) when the learned selector is on, then one area that the phases use
+  // in turn: PullSmem, or FlatSmem and the tiled phase's 3 * kTileWordsMax words
   extern __shared__ __align__(16) unsigned char s_dyn[];
   float* s_mlp = reinterpret_cast<float*>(s_dyn);
-  uint32_t* s_tile = reinterpret_cast<uint32_t*>(s_dyn + p.tile_smem_off);
+  FlatSmem& s_flat = *reinterpret_cast<FlatSmem*>(s_dyn + p.phase_smem_off);
+  uint32_t* s_tile = reinterpret_cast<uint32_t*>(s_dyn + p.phase_smem_off + kFlatBytes);
+  PullSmem& s_pull = *reinterpret_cast<PullSmem*>(s_dyn + p.phase_smem_off);
   const int tid = threadIdx.x;
   unsigned long long bar_target = 0;
   if (tid == 0) {
@@ -935,9 +1095,9 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
     if (variant == BFS_VARIANT_TILED && (!kTiles || p.t_jc == nullptr)) variant = BFS_VARIANT_PULL;  // the SpMV untiled
     PHASE_TS(k, 2);
     if (part) {
-      if (variant == BFS_VARIANT_PULL) pull_phase(p, k, sm, acc, G);
-      else if (kTiles && variant == BFS_VARIANT_TILED) tiled_phase(p, k, sm, s_tile, acc, G);
-      else topdown_phase(p, k, variant, count, nchunks, sm, acc, G);
+      if (variant == BFS_VARIANT_PULL) pull_phase(p, k, count, sm, s_pull, acc, G);
+      else if (kTiles && variant == BFS_VARIANT_TILED) tiled_phase(p, k, sm, s_flat, s_tile, acc, G);
+      else topdown_phase(p, k, variant, count, nchunks, sm, s_flat, acc, G);
       PHASE_TS(k, 3);
       end_phase(p, k + 1, acc, sm);
     }
@@ -1093,11 +1253,10 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
     p.t_ncb = ts->ncb;
   }
 
-  // the tiled variant's slices follow the network's parameters in dynamic shared memory
+  // the pull / tiled phase's area follows the network's parameters in dynamic shared memory
   const size_t mlp_bytes = p.mlp ? (sizeof(float) * BFS_MLP_PARAMS + 15) / 16 * 16 : 0;
-  const size_t tile_bytes = p.t_jc ? sizeof(uint32_t) * 3 * kTileWordsMax : 0;
-  p.tile_smem_off = (int32_t)mlp_bytes;
-  const size_t dyn_smem = mlp_bytes + tile_bytes;
+  p.phase_smem_off = (int32_t)mlp_bytes;
+  const size_t dyn_smem = mlp_bytes + kPhaseBytes;
   const void* kernel = p.t_jc ? (const void*)level_loop_kernel<true> : (const void*)level_loop_kernel<false>;
   {  // the attribute belongs to the current device: set it once per device
     static std::mutex mu;
@@ -1105,7 +1264,7 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
     std::lock_guard<std::mutex> lk(mu);
     if (di.device < 0 || di.device >= 64) return fail(BFS_ERR_UNSUPPORTED, "device ordinal out of range");
     if (!configured[di.device]) {
-      const int max_dyn = (int)((sizeof(float) * BFS_MLP_PARAMS + 15) / 16 * 16 + sizeof(uint32_t) * 3 * kTileWordsMax);
+      const int max_dyn = (int)((sizeof(float) * BFS_MLP_PARAMS + 15) / 16 * 16 + kPhaseBytes);
       BFS_CUDA_TRY(cudaFuncSetAttribute((const void*)level_loop_kernel<false>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn));
       BFS_CUDA_TRY(cudaFuncSetAttribute((const void*)level_loop_kernel<true>,
@@ -1119,6 +1278,15 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
   const int grid = (t.ctas_per_sm > 0 ? std::min(per_sm, t.ctas_per_sm) : per_sm) * di.sm_count;
   if (int e = prepare_barrier(w, 0, grid, s, &p.bar)) return e;
   p.small_frontier = t.small_frontier > 0 ? t.small_frontier : (t.small_frontier == 0 ? (long long)grid * kWarps : 0);
+  p.probe = g->d_probe;
+  p.rank = g->d_rank;
+  // one chunk per resident warp while a lane per word allows it (see pull_phase)
+  const long long grid_warps = (long long)grid * kWarps;
+  p.pull_words = (int)std::min<long long>(32, std::max<long long>(1, (w->nwords + grid_warps - 1) / grid_warps));
+  while (((long long)g->n - 1) >> p.fr_shift >= 32ll * kFrWords) ++p.fr_shift;
+  // every CTA reads the whole queue to build the summary: at most 8,192 vertices (12 % of its bits set; a
+  // limit of 32,768 measured the same), and few against n so that the rows' scans pay for it
+  p.fr_limit = (unsigned)std::min<long long>(8192, g->n / 128);
   p.narrow_edges = t.narrow_edges > 0 ? t.narrow_edges : (t.narrow_edges == 0 ? (1ll << 14) : -1);
 #ifdef BFS_PHASE_TIMING
   fprintf(stderr, "level loop: %d CTAs (%d per SM), %zu bytes dynamic shared memory\n", grid, per_sm, dyn_smem);
