@@ -125,7 +125,7 @@ typedef struct bfs_tuning {
                              degree above 32, runs TD_WARP instead of TD_BINNED (0 = default: the warps resident
                              in the traversal's grid; negative = never) */
   int32_t batch_width;   /* batched: roots per traversal, the bits of a frontier word: 8, 16, 32 or 64
-                            (default 64) */
+                            (default 64); a traversal of fewer roots takes the narrowest word that holds them */
   int32_t narrow_edges;  /* a level whose frontier has at most this many edges runs on half the CTAs of the
                             traversal's grid, which also halves its barrier's arrivals (0 = default 16384;
                             negative = never) */

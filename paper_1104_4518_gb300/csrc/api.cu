@@ -697,7 +697,8 @@ int bfs_run_batch(bfs_graph* g, const int32_t* sources, int32_t k, int32_t* pare
     br.w = w;
     br.h_sources = sources + c;
     br.k = std::min(width, k - c);
-    br.width = width;
+    br.width = 8;  // the narrowest word that holds the roots: its arrays and scratch rows shrink with it
+    while (br.width < br.k) br.width *= 2;
     br.level = host ? dl : level_out + (size_t)c * n;
     br.parent = host ? dp : parent_out + (size_t)c * n;
     br.spin_limit = opts ? opts->spin_limit : 0;

@@ -12,10 +12,12 @@
 // "Reached before level k+1" is tested as V | F_k, so V only has to absorb a
 // frontier's bits during the level that expands it, and every level is one
 // phase.  Two ways to expand a level (identical results):
-//   pull     : every vertex not yet reached by all roots scans its row; short
-//              rows lane by lane, rows up to kChunkEdges entries by the whole
-//              warp, longer rows in kChunkEdges-entry chunks (a static table
-//              built with the graph), one CTA per chunk, the chunks combining
+//   pull     : every vertex not yet reached by all roots scans its row, first
+//              the top eight entries of eight rows at a time, then row by row
+//              with the whole warp; lane r owns root r (and r + 32) and takes
+//              its parent from a bit transpose of the entries' words; rows above
+//              kChunkEdges entries go in kChunkEdges-entry chunks (a static table
+//              built with the graph), one warp per chunk, the chunks combining
 //              through atomicMax on the parents and atomicOr on F_{k+1};
 //   top-down : every frontier row ORs its bits into F_{k+1} of unreached
 //              neighbours and offers itself as their parent with atomicMax
@@ -24,10 +26,14 @@
 //              level, the first writer of any bit enqueues the neighbour.
 //              Rows above kChunkEdges entries are split into chunk items.
 // Output rows are root-major: level[r * n + v], parent[r * n + v].  During
-// the traversal the results go to vertex-major scratch (sl / sp [v][r], one
-// row of `stride` ints per vertex), so that the results of one vertex share a
-// few sectors instead of landing 4 * n bytes apart; a last phase transposes the
-// scratch into the outputs through shared-memory tiles, coalesced both ways.
+// the traversal the parents go to vertex-major scratch (sp[v][r], one row of
+// `stride` ints per vertex), so that the results of one vertex share a few
+// sectors instead of landing 4 * n bytes apart, and the levels to bit planes:
+// bit r of plane[j][v] is bit j of root r's level of v, so that a level costs
+// a vertex one word per set bit of its number and an R-MAT traversal three
+// words per vertex in all, where 64 ints would be 256 bytes.  The planes take
+// F_k's level when level k expands it (by the vertex's owner, without atomics).
+// A last phase turns both into the outputs, coalesced.
 //
 // The words are 8, 16, 32 or 64 bits wide (one bit per root of the
 // traversal; bit arithmetic is done in 64-bit registers whatever the word).
@@ -48,10 +54,25 @@ namespace {
 
 using bfsdev::kFull;
 
+// What bounds the kernel and why it is split this way (R-MAT scale 24, 64
+// roots, level times): the pull levels look up one frontier word per row entry
+// in an array that just exceeds L2, with 32 warps per SM to hide the latency
+// (halving them makes the levels 1.4 times slower), and spend as many
+// instructions on recording parents as on finding them.  Recording was the
+// larger part when a lane or a warp wrote one root's level and parent at a
+// time (4-byte stores 256 bytes apart): with a lane per root the two dense
+// levels went from 9.4 and 5.9 ms to 4.0 and 2.9 ms.  The loads in flight
+// below are the best of 1 to 4 each; deeper ones cost registers that spill.
 constexpr int kBBlock = 512;
 static_assert(kBBlock == kClaimBlock, "the claim buffers assume 512-thread CTAs");
 constexpr int kBWarps = kBBlock / 32;
-constexpr int kShortRow = 32;  // rows up to this length are scanned by one lane
+constexpr int kTop = 8;        // entries of a row examined in the first packed step, 32 / kTop rows per load
+constexpr int kNext = 32;      // entries of a row examined in the second, one row per load
+constexpr int kTopLoads = 2, kNextLoads = 2;  // loads per lane in flight in these steps
+constexpr int kRowLoads = 4;   // loads per lane in flight when the warp scans the rest of one row
+constexpr int kFewBits = 6;    // up to this many new roots are resolved one by one instead of by a transpose
+constexpr int kPlanes = 31;    // level bit planes: levels are below 2^31
+static_assert(8 * kPlanes <= 64 * sizeof(int32_t), "the planes fit the second half of the scratch");
 
 struct BatchParams {
   const int64_t* __restrict__ off;   // out-rows: top-down
@@ -66,9 +87,10 @@ struct BatchParams {
   int32_t src[64];
   int32_t* level;   // [k][n]
   int32_t* parent;  // [k][n]
-  int32_t* sl;      // scratch levels [n][stride]
+  void* planes;     // level bit planes, Word[kPlanes][n]
   int32_t* sp;      // scratch parents [n][stride]
   int32_t stride;   // roots per scratch row (the word width)
+  const uint32_t* __restrict__ dead;  // bitmap of the vertices no arc enters
   void* F[3];  // Word[n] each
   void* V;     // Word[n]
   int32_t* queue[3];
@@ -114,116 +136,171 @@ __device__ __forceinline__ Bits warp_or(Bits v) {
   }
 }
 
-// Writes level / parent of the roots in `bits` for vertex v.
-__device__ __forceinline__ void write_hits(const BatchParams& p, uint64_t bits, int v, int u, int lvl) {
-  while (bits) {
-    const int r = __ffsll((long long)bits) - 1;
-    bits &= bits - 1;
-    const long long o = (long long)v * p.stride + r;
-    p.sl[o] = lvl;
-    p.sp[o] = u;
+// 32 x 32 bit transpose over the warp: bit s of lane r's result is bit r of lane s's x.
+__device__ __forceinline__ unsigned transpose32(unsigned x, int lane) {
+#pragma unroll
+  for (int s = 16; s >= 1; s >>= 1) {
+    const unsigned lo = s == 16 ? 0x0000ffffu : s == 8 ? 0x00ff00ffu : s == 4 ? 0x0f0f0f0fu : s == 2 ? 0x33333333u : 0x55555555u;
+    const unsigned y = __shfl_xor_sync(kFull, x, s);
+    x = (lane & s) ? ((x & ~lo) | ((y & ~lo) >> s)) : ((x & lo) | ((y & lo) << s));
   }
+  return x;
 }
 
-// One lane scans rows [b, e) of v from the top, four loads at a time, and
-// resolves the roots in `need`; returns the bits found.
-template <typename Word>
-__device__ __forceinline__ uint64_t resolve_lane(const BatchParams& p, const Word* F, int v, long long b,
-                                                 long long e, uint64_t need, int lvl) {
-  uint64_t found = 0;
-  long long j = e - 1;
-  while (j >= b && need) {
-    int u[4];
-    uint64_t f[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) u[q] = (j - q >= b) ? __ldg(&p.tadj[j - q]) : -1;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const bool live = bfsdev::kBoundsCheck
-                            ? j - q >= b && bfsdev::in_range(p.status, bfsdev::kSiteBatchPull, u[q], p.n)
-                            : u[q] >= 0;
-      f[q] = live ? (Bits)F[u[q]] : 0ull;
+// Records the parents of the roots found in one row: m0 (m1) has a bit for
+// every slot of the row whose word holds root `lane` (`lane` + 32), the lowest
+// slot being the largest id, and lane s holds slot s's id u.  kOffer: the ids
+// are candidates of one chunk of the row, so they are offered with atomicMax.
+// Returns the roots found (the same in every lane).
+template <typename Word, bool kOffer>
+__device__ __forceinline__ Bits store_parents(const BatchParams& p, int v, unsigned m0, unsigned m1, int u, int lane) {
+  int32_t* row = p.sp + (long long)v * p.stride;
+  const int u0 = __shfl_sync(kFull, u, m0 ? __ffs(m0) - 1 : 0);
+  if (m0) {
+    if (kOffer) bfsdev::red_max_i32(row + lane, u0);
+    else row[lane] = u0;
+  }
+  Bits found = __ballot_sync(kFull, m0 != 0);
+  if constexpr (sizeof(Word) == 8) {
+    const int u1 = __shfl_sync(kFull, u, m1 ? __ffs(m1) - 1 : 0);
+    if (m1) {
+      if (kOffer) bfsdev::red_max_i32(row + lane + 32, u1);
+      else row[lane + 32] = u1;
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const uint64_t h = f[q] & need;
-      if (h) {
-        write_hits(p, h, v, u[q], lvl);
-        need &= ~h;
-        found |= h;
-      }
-    }
-    j -= 4;
+    found |= (Bits)__ballot_sync(kFull, m1 != 0) << 32;
   }
   return found;
 }
 
-// The whole warp scans entries [b, e) of v's row from the top, 128 entries per
-// step (four loads per lane in flight, examined in descending position order);
-// returns the bits found (same value in every lane).  kChunk: the range is one
-// chunk of a longer row, so the first hit of a root is only this chunk's
-// candidate: it is offered with atomicMax and the level is left to the claim.
-template <typename Word, bool kChunk>
-__device__ __forceinline__ uint64_t resolve_warp(const BatchParams& p, const Word* F, int v, long long b,
-                                                 long long e, uint64_t need, int lvl, int lane) {
-  uint64_t found = 0;
-  for (long long top = e; top > b && need; top -= 128) {
-    int u[4];
-    uint64_t f[4];
+// The whole warp scans entries [b, t) of v's row from the top, 32 * kRowLoads
+// per step, and resolves the roots in `need`; returns the bits found (the same
+// value in every lane).  kOffer: see store_parents.
+template <typename Word, bool kOffer>
+__device__ __forceinline__ Bits resolve_row(const BatchParams& p, const Word* F, int v, long long b, long long t,
+                                            Bits need, int lane) {
+  Bits found = 0;
+  for (; t > b && need; t -= 32 * kRowLoads) {
+    int u[kRowLoads];
+    Bits f[kRowLoads];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const long long j = top - 1 - lane - 32 * q;
+    for (int q = 0; q < kRowLoads; ++q) {
+      const long long j = t - 1 - lane - 32 * q;
       u[q] = j >= b ? __ldg(&p.tadj[j]) : 0;
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      f[q] = (top - 1 - lane - 32 * q >= b && bfsdev::in_range(p.status, bfsdev::kSiteBatchPull, u[q], p.n))
-                 ? ((Bits)F[u[q]] & need)
-                 : 0ull;
+    for (int q = 0; q < kRowLoads; ++q)
+      f[q] = (t - 1 - lane - 32 * q >= b && bfsdev::in_range(p.status, bfsdev::kSiteBatchPull, u[q], p.n)) ? (Bits)__ldcg(&F[u[q]])
+                                                                                                         : 0ull;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      uint64_t nb = warp_or<Word>(f[q]) & need;
+    for (int q = 0; q < kRowLoads; ++q) {
+      const Bits mine = f[q] & need;
+      Bits nb = warp_or<Word>(mine);
+      if (!nb) continue;
       found |= nb;
       need &= ~nb;
-      while (nb) {  // each new root takes the lowest lane holding its bit (the highest position)
-        const int r = __ffsll((long long)nb) - 1;
-        nb &= nb - 1;
-        const unsigned who = __ballot_sync(kFull, (f[q] >> r) & 1ull);
-        const int pu = __shfl_sync(kFull, u[q], __ffs(who) - 1);
-        if (lane == 0) {
-          const long long o = (long long)v * p.stride + r;
-          if (kChunk) {
-            atomicMax(&p.sp[o], pu);
-          } else {
-            p.sl[o] = lvl;
-            p.sp[o] = pu;
+      if (__popcll(nb) <= kFewBits) {
+        for (; nb; nb &= nb - 1) {  // each new root takes the lowest lane holding its bit (the largest id)
+          const int r = __ffsll((long long)nb) - 1;
+          const unsigned who = __ballot_sync(kFull, (mine >> r) & 1ull);
+          if (lane == __ffs(who) - 1) {
+            int32_t* o = p.sp + (long long)v * p.stride + r;
+            if (kOffer) bfsdev::red_max_i32(o, u[q]);
+            else *o = u[q];
           }
         }
+      } else {
+        const unsigned m0 = transpose32((unsigned)mine, lane);
+        const unsigned m1 = sizeof(Word) == 8 ? transpose32((unsigned)(mine >> 32), lane) : 0u;
+        store_parents<Word, kOffer>(p, v, m0, m1, u[q], lane);
       }
     }
   }
   return found;
 }
 
-// Resolves the parents of 32 vertices (one per lane, need = roots to find)
-// against frontier F; lanes with short rows scan alone, long rows get the warp.
+// Examines kSlots entries of every row with roots to find, below its first
+// `skip`, 32 / kSlots rows per load and kLoads loads in flight: lane l's row
+// has deg entries ending at e and `need` roots to find.  Adds the roots found
+// to `found` and takes them from `need`.  list: 32 ints of the warp.
+template <typename Word, int kSlots, int kLoads>
+__device__ __forceinline__ void resolve_packed(const BatchParams& p, const Word* F, int v0, int skip, int deg,
+                                               long long e, Bits& need, Bits& found, int lane, int* list) {
+  constexpr int kRows = 32 / kSlots;  // rows per load
+  const bool open = need != 0 && deg > skip;
+  const unsigned pm = __ballot_sync(kFull, open);
+  if (!pm) return;
+  const int rows = __popc(pm);
+  if (open) list[__popc(pm & bfsdev::lanemask_lt())] = lane;
+  __syncwarp();
+  Bits got = 0;
+  const int sub = lane / kSlots, slot = skip + lane % kSlots;
+  for (int base = 0; base < rows; base += kRows * kLoads) {
+    int u[kLoads], own[kLoads];
+    Bits f[kLoads];
+    bool has[kLoads];
+#pragma unroll
+    for (int q = 0; q < kLoads; ++q) {
+      const int i = base + q * kRows + sub;
+      own[q] = list[min(i, rows - 1)];
+      const int d = __shfl_sync(kFull, deg, own[q]);
+      const long long eo = __shfl_sync(kFull, e, own[q]);
+      has[q] = i < rows && slot < d;
+      u[q] = has[q] ? __ldg(&p.tadj[eo - 1 - slot]) : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < kLoads; ++q)
+      f[q] = (has[q] && bfsdev::in_range(p.status, bfsdev::kSiteBatchPull, u[q], p.n)) ? (Bits)__ldcg(&F[u[q]]) : 0ull;
+#pragma unroll
+    for (int q = 0; q < kLoads; ++q) {
+      const Bits mine = f[q] & __shfl_sync(kFull, need, own[q]);
+      const unsigned any = __ballot_sync(kFull, mine != 0);
+      if (!any) continue;
+      const unsigned m0 = transpose32((unsigned)mine, lane);
+      const unsigned m1 = sizeof(Word) == 8 ? transpose32((unsigned)(mine >> 32), lane) : 0u;
+#pragma unroll
+      for (int j = 0; j < kRows; ++j) {
+        const unsigned seg = (kSlots == 32 ? kFull : (1u << kSlots) - 1u) << (j * kSlots);
+        if (!(any & seg)) continue;
+        const int o = __shfl_sync(kFull, own[q], j * kSlots);
+        const Bits fr = store_parents<Word, false>(p, v0 + o, m0 & seg, m1 & seg, u[q], lane);
+        if (lane == o) got = fr;
+      }
+    }
+  }
+  need &= ~got;
+  found |= got;
+  __syncwarp();  // the list is free again
+}
+
+// Resolves 32 vertices v0 .. v0 + 31 against frontier F: lane l's row has deg
+// entries ending at e and `need` roots to find.  First the top kTop entries of
+// every row, 32 / kTop rows per load: a dense level ends most rows there, and
+// short rows fill the lanes that a row each would leave idle; then the next
+// kNext entries, four rows in flight; then row by row.  Returns the lane's bits found.
 template <typename Word>
-__device__ __forceinline__ uint64_t resolve_group(const BatchParams& p, const Word* F, int v, long long b,
-                                                  long long e, uint64_t need, int lvl, int lane) {
-  uint64_t found = 0;
-  const bool longrow = need && (e - b) > kShortRow;
-  if (need && !longrow) found = resolve_lane(p, F, v, b, e, need, lvl);
-  unsigned lm = __ballot_sync(kFull, longrow);
-  while (lm) {
+__device__ __forceinline__ Bits resolve_group(const BatchParams& p, const Word* F, int v0, int deg, long long e,
+                                              Bits need, int lane, int* list) {
+  Bits found = 0;
+  resolve_packed<Word, kTop, kTopLoads>(p, F, v0, 0, deg, e, need, found, lane, list);
+  resolve_packed<Word, kNext, kNextLoads>(p, F, v0, kTop, deg, e, need, found, lane, list);
+  for (unsigned lm = __ballot_sync(kFull, need != 0 && deg > kTop + kNext); lm; lm &= lm - 1u) {
     const int l = __ffs(lm) - 1;
-    lm &= lm - 1;
-    const int lv = __shfl_sync(kFull, v, l);
-    const long long lb = __shfl_sync(kFull, b, l), le = __shfl_sync(kFull, e, l);
-    const uint64_t ln = __shfl_sync(kFull, need, l);
-    const uint64_t fw = resolve_warp<Word, false>(p, F, lv, lb, le, ln, lvl, lane);
-    if (lane == l) found = fw;
+    const long long el = __shfl_sync(kFull, e, l);
+    const Bits fr = resolve_row<Word, false>(p, F, v0 + l, el - __shfl_sync(kFull, deg, l), el - kTop - kNext,
+                                             __shfl_sync(kFull, need, l), lane);
+    if (lane == l) found |= fr;
   }
   return found;
+}
+
+// Adds level k of the roots in F_k[v] = bits to the bit planes; called once per
+// level and vertex, by the vertex's owner in that level.
+template <typename Word>
+__device__ __forceinline__ void add_level(const BatchParams& p, int v, Bits bits, int k) {
+  for (unsigned m = (unsigned)k; m; m &= m - 1u) {
+    Word* a = static_cast<Word*>(p.planes) + (long long)(__ffs(m) - 1) * p.n + v;
+    *a = (Word)((Bits)*a | bits);
+  }
 }
 
 // Top-down visit of edge (u -> w) with frontier bits f of u at level knext - 1.
@@ -233,22 +310,11 @@ __device__ __forceinline__ void td_visit(const BatchParams& p, const Word* Fc, W
   if (!bfsdev::in_range(p.status, bfsdev::kSiteBatchTopDown, w, p.n)) return;
   const uint64_t nb = f & ~((Bits)V[w] | (Bits)Fc[w]);
   if (!nb) return;
-  // u is a parent candidate of w for every new root bit; an offer no larger than
-  // the current one is dropped without an atomic (the row of w is one 256-byte
-  // line, read once)
-  for (uint64_t b = nb; b;) {
-    const int r = __ffsll((long long)b) - 1;
-    b &= b - 1;
-    int32_t* o = &p.sp[(long long)w * p.stride + r];
-    if (__ldcg(o) < u) atomicMax(o, u);
-  }
+  // u is a parent candidate of w for every new root bit (the offers return
+  // nothing, so none of them is waited for)
+  for (uint64_t b = nb; b; b &= b - 1) bfsdev::red_max_i32(&p.sp[(long long)w * p.stride + __ffsll((long long)b) - 1], u);
   if (((Bits)Fn[w] & nb) == nb) return;
   const Bits old = atomic_or_word(&Fn[w], nb);
-  for (uint64_t b = nb & ~old; b;) {
-    const int r = __ffsll((long long)b) - 1;
-    b &= b - 1;
-    p.sl[(long long)w * p.stride + r] = knext;
-  }
   if (old == 0) {
     cta_enqueue(p, knext, cl, w);
     const long long deg = __ldg(&p.off[w + 1]) - __ldg(&p.off[w]);
@@ -264,15 +330,10 @@ template <typename Word>
 __device__ __forceinline__ void pull_chunk(const BatchParams& p, const Word* Fc, Word* Fn, int knext, int v,
                                            long long rb, long long re, uint64_t need, int lane, Claims& cl,
                                            int* wq, int& nbuf) {
-  const uint64_t found = resolve_warp<Word, true>(p, Fc, v, rb, re, need, knext, lane);
+  const Bits found = resolve_row<Word, true>(p, Fc, v, rb, re, need, lane);
   bool claimed = false;
   if (lane == 0 && found) {
     const Bits old = atomic_or_word(&Fn[v], found);
-    for (uint64_t bb = found & ~old; bb;) {
-      const int r = __ffsll((long long)bb) - 1;
-      bb &= bb - 1;
-      p.sl[(long long)v * p.stride + r] = knext;
-    }
     if (old == 0) {
       claimed = true;
       push_chunks_cta(p, knext, cl, v, __ldg(&p.off[v + 1]) - __ldg(&p.off[v]));
@@ -286,6 +347,7 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
   Word* F[3] = {static_cast<Word*>(p.F[0]), static_cast<Word*>(p.F[1]), static_cast<Word*>(p.F[2])};
   Word* V = static_cast<Word*>(p.V);
   __shared__ Claims cl;
+  __shared__ int row_list[kBWarps][32];  // pull: the lanes of a word with roots to find
   const int tid = threadIdx.x, lane = tid & 31;
   unsigned long long bar_target = 0;
   if (tid == 0) {
@@ -299,11 +361,16 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
   const long long gwarp = blockIdx.x + (long long)(tid >> 5) * G;  // round-robin over CTAs
   const unsigned nblocks = gridDim.x;
 
-  // init: scratch parents to -1 (atomicMax offers need a floor; scratch levels
-  // are only read where V says the root reached the vertex), bitsets to 0,
-  // counters to 0
-  const long long total = (long long)p.n * p.stride;
-  for (long long i = gtid; i < total; i += gthreads) p.sp[i] = -1;
+  // init: scratch parents of the vertices that an arc enters to -1 (atomicMax
+  // offers need a floor; entries are only read where V says the root reached the
+  // vertex), bitsets to 0, counters to 0
+  const int S4 = p.stride / 4;  // 2 to 16, a power of two
+  const int s4 = __ffs(S4) - 1;
+  const long long total = (long long)p.n << s4;
+  for (long long i = gtid; i < total; i += gthreads) {
+    const long long v = i >> s4;
+    if (!((__ldg(&p.dead[v >> 5]) >> (v & 31)) & 1u)) reinterpret_cast<int4*>(p.sp)[i] = make_int4(-1, -1, -1, -1);
+  }
   for (long long v = gtid; v < p.n; v += gthreads) {
     F[0][v] = 0;
     F[1][v] = 0;
@@ -318,9 +385,7 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
   if (blockIdx.x == 0 && tid < p.k) {
     const int s = p.src[tid];
     const uint64_t bit = 1ull << tid;
-    const long long o = (long long)s * p.stride + tid;
-    p.sl[o] = 0;
-    p.sp[o] = s;
+    p.sp[(long long)s * p.stride + tid] = s;  // level 0 has no plane bits
     atomic_or_word(&V[s], bit);
     const Bits old = atomic_or_word(&F[0][s], bit);
     if (old == 0) {
@@ -356,6 +421,12 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
       }
     }
 
+    // the first level with bit j is 2^j: its plane is cleared one phase earlier
+    if (((k + 1) & k) == 0) {
+      Word* fresh = static_cast<Word*>(p.planes) + (long long)(31 - __clz(k + 1)) * p.n;
+      for (long long v = gtid; v < p.n; v += gthreads) fresh[v] = 0;
+    }
+
     const bool topdown = (long long)count <= p.td_limit;
     const int wid = tid >> 5;
     if (topdown) {
@@ -375,7 +446,10 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
       for (long long i = gwarp; i < count; i += gwarps) {
         const int u = Q[i];
         const uint64_t f = (Bits)Fc[u];
-        if (lane == 0) V[u] = (Word)((Bits)V[u] | f);
+        if (lane == 0) {
+          V[u] = (Word)((Bits)V[u] | f);
+          add_level<Word>(p, u, f, k);
+        }
         const long long b = __ldg(&p.off[u]), e = __ldg(&p.off[u + 1]);
         if (e - b > kChunkEdges) continue;
         for (long long j = b + lane; j < e; j += 32) td_visit(p, Fc, Fn, V, knext, f, u, __ldg(&p.adj[j]), cl);
@@ -406,44 +480,50 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
       // edgefactor-16 and -64 graphs (16 roots: 3 % and 4 % slower).
       const int S = nw > 64 * gw ? gw * ((nw / 2) / gw) : nw;
       const int ngroups = (nw - S + kGroupWords - 1) / kGroupWords;
-      auto pull_word = [&](int ww) {
-        const long long v0 = (long long)ww * 32 + lane;
-        const int v = (int)v0;
-        uint64_t need = 0, vv = 0, fv = 0;
-        long long b = 0, e = 0;
-        if (v0 < p.n) {
+      int* list = row_list[wid];
+      // the warp's words in turn: ww, then next_word(ww), until nw
+      unsigned fetched = 0;  // lane 0: the next group, fetched while the one before is worked on
+      int wend = 0;
+      if (ngroups > 0 && lane == 0) fetched = (unsigned)atomicAdd(&p.ctr[k % kCtrRing].pad, 1ull);
+      auto take_group = [&]() {
+        const int grp = (int)__shfl_sync(kFull, fetched, 0);
+        if (grp >= ngroups) return nw;
+        if (lane == 0) fetched = (unsigned)atomicAdd(&p.ctr[k % kCtrRing].pad, 1ull);
+        wend = min(nw, S + (grp + 1) * kGroupWords);
+        return S + grp * kGroupWords;
+      };
+      auto next_word = [&](int ww) {
+        const int w1 = ww < S ? ww + gw : ww + 1;
+        return w1 < (ww < S ? S : wend) ? w1 : take_group();
+      };
+      for (int ww = (int)gwarp < S ? (int)gwarp : take_group(); ww < nw; ww = next_word(ww)) {
+        const int v = ww * 32 + lane;
+        const bool in = v < p.n;  // (n rounded up to 32 fits: n < 2^31 - 1)
+        Bits need = 0, vv = 0, fv = 0;
+        int deg = 0;
+        long long e = 0;
+        if (in) {
           vv = (Bits)V[v];
           fv = (Bits)Fc[v];
-          need = ~(vv | fv) & p.mask;
-          if (need) {
-            b = __ldg(&p.toff[v]);
-            e = __ldg(&p.toff[v + 1]);
-            if (e == b || e - b > kChunkEdges) need = 0;
-          }
+          e = __ldg(&p.toff[v + 1]);
+          const long long d = e - __ldg(&p.toff[v]);
+          need = d == 0 || d > kChunkEdges ? 0ull : ~(vv | fv) & p.mask;
+          deg = (int)d;
         }
-        const uint64_t found = resolve_group(p, Fc, v, b, e, need, knext, lane);
-        if (v0 < p.n) {
-          const uint64_t nv = vv | fv | found;
+        const Bits found = resolve_group(p, Fc, v - lane, deg, e, need, lane, list);
+        if (in) {
+          const Bits nv = vv | fv | found;
           if (nv != vv) V[v] = (Word)nv;
+          if (fv) add_level<Word>(p, v, fv, k);
           if (found) {
             Fn[v] = (Word)found;
             if (p.directed) {  // the next level's top-down expansion needs the chunks of a long out-row
-              const long long deg = __ldg(&p.off[v + 1]) - __ldg(&p.off[v]);
-              if (deg > kChunkEdges) push_chunks_cta(p, knext, cl, v, deg);
+              const long long dout = __ldg(&p.off[v + 1]) - __ldg(&p.off[v]);
+              if (dout > kChunkEdges) push_chunks_cta(p, knext, cl, v, dout);
             }
           }
         }
         warp_enqueue(p, knext, wq, nbuf, found != 0, v, lane, false);
-      };
-      for (int ww = (int)gwarp; ww < S; ww += gw) pull_word(ww);
-      if (ngroups > 0) {
-        unsigned next = 0;
-        if (lane == 0) next = (unsigned)atomicAdd(&p.ctr[k % kCtrRing].pad, 1ull);
-        for (int grp = (int)__shfl_sync(kFull, next, 0); grp < ngroups; grp = (int)__shfl_sync(kFull, next, 0)) {
-          if (lane == 0) next = (unsigned)atomicAdd(&p.ctr[k % kCtrRing].pad, 1ull);  // fetched one group ahead
-          const int w0 = S + grp * kGroupWords, w1 = min(nw, w0 + kGroupWords);
-          for (int ww = w0; ww < w1; ++ww) pull_word(ww);
-        }
       }
       warp_enqueue(p, knext, wq, nbuf, false, 0, lane, true);
     }
@@ -461,55 +541,57 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
   }
   if (gtid == 0) p.misc[1] = k;
 
-  // transpose the scratch rows of 32 vertices into the root-major outputs
-  // (the loop ended right after a grid barrier, so the scratch is final, and V
-  // holds every root bit of every vertex reached).  Scratch rows are read as
-  // int4 (S is a multiple of 4 and the scratch 16-byte aligned); output rows
-  // are written as int4 when n is a multiple of 4 and both outputs start on a
-  // 16-byte boundary (every row then does), else one int at a time.
-  int* tl = cl.cq;            // [S][33] levels
-  int* tp = cl.cq + 64 * 33;  // [S][33] parents
-  const int S = p.stride, S4 = S / 4;
-  const bool vec_out = (p.n & 3) == 0 &&
-                       ((reinterpret_cast<uintptr_t>(p.level) | reinterpret_cast<uintptr_t>(p.parent)) & 15u) == 0;
+  // Outputs, root-major, from the scratch rows and planes (the loop ended right
+  // after a grid barrier, so both are final, and V holds every root bit of every
+  // vertex reached).  A warp takes 32 vertices, lane i the i-th: it reads its
+  // scratch row 16 bytes at a time (skipped where none of the four roots reached
+  // it), puts the levels together from the planes, and each root's 32 results
+  // leave as one 128-byte store.  No CTA barrier, and four row loads in flight
+  // per lane: through shared-memory tiles of 32 vertices per CTA the phase took
+  // 5.4 ms for 64 roots at R-MAT scale 24.
+  const int nplanes = k > 1 ? 32 - __clz(k - 1) : 0;  // levels 0 .. k - 1
+  const Word* planes = static_cast<const Word*>(p.planes);
+  constexpr int kRegPlanes = 3;
+  const int ngroups = (p.k + 3) / 4;
   const long long ntiles = ((long long)p.n + 31) / 32;
-  for (long long t = blockIdx.x; t < ntiles; t += G) {
-    const long long v0 = t * 32;
-    const int nv = (int)min(32ll, (long long)p.n - v0);
-    for (int e = tid; e < 32 * S4; e += kBBlock) {
-      const int i = e / S4, c = e - i * S4;
-      if (i < nv) {
-        const long long o = (v0 + i) * S + 4 * c;
-        const int4 lv = *reinterpret_cast<const int4*>(p.sl + o);
-        const int4 pv = *reinterpret_cast<const int4*>(p.sp + o);
-        const Bits vv = (Bits)V[v0 + i] >> (4 * c);
-        tl[(4 * c + 0) * 33 + i] = (vv & 1ull) ? lv.x : -1;
-        tl[(4 * c + 1) * 33 + i] = (vv & 2ull) ? lv.y : -1;
-        tl[(4 * c + 2) * 33 + i] = (vv & 4ull) ? lv.z : -1;
-        tl[(4 * c + 3) * 33 + i] = (vv & 8ull) ? lv.w : -1;
-        tp[(4 * c + 0) * 33 + i] = pv.x;
-        tp[(4 * c + 1) * 33 + i] = pv.y;
-        tp[(4 * c + 2) * 33 + i] = pv.z;
-        tp[(4 * c + 3) * 33 + i] = pv.w;
+  for (long long t = gwarp; t < ntiles; t += gwarps) {
+    const long long v = t * 32 + lane;
+    const bool in = v < p.n;
+    const Bits vv = in ? (Bits)V[v] : 0ull;
+    Bits pl[kRegPlanes];
+#pragma unroll
+    for (int j = 0; j < kRegPlanes; ++j) pl[j] = vv && j < nplanes ? (Bits)planes[(long long)j * p.n + v] : 0ull;
+    const int4* row = reinterpret_cast<const int4*>(p.sp) + (v << s4);
+#pragma unroll 4
+    for (int c = 0; c < ngroups; ++c) {
+      const unsigned on = (unsigned)(vv >> (4 * c)) & 15u;
+      int4 pv = make_int4(-1, -1, -1, -1);
+      if (on) pv = __ldg(row + c);
+      unsigned lb[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) lb[q] = 0;
+#pragma unroll
+      for (int j = 0; j < kRegPlanes; ++j) {
+        const unsigned b = (unsigned)(pl[j] >> (4 * c));
+#pragma unroll
+        for (int q = 0; q < 4; ++q) lb[q] |= (b >> q & 1u) << j;
       }
-    }
-    __syncthreads();
-    for (int e = tid; e < 8 * p.k; e += kBBlock) {
-      const int r = e >> 3, i = 4 * (e & 7);
-      const long long o = (long long)r * p.n + v0 + i;
-      const int* L = tl + r * 33 + i;
-      const int* P = tp + r * 33 + i;
-      if (vec_out && i + 4 <= nv) {
-        *reinterpret_cast<int4*>(p.level + o) = make_int4(L[0], L[1], L[2], L[3]);
-        *reinterpret_cast<int4*>(p.parent + o) = make_int4(P[0], P[1], P[2], P[3]);
-      } else {
-        for (int m = 0; m < 4 && i + m < nv; ++m) {
-          p.level[o + m] = L[m];
-          p.parent[o + m] = P[m];
+      for (int j = kRegPlanes; j < nplanes; ++j) {
+        const unsigned b = on ? (unsigned)((Bits)planes[(long long)j * p.n + v] >> (4 * c)) : 0u;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) lb[q] |= (b >> q & 1u) << j;
+      }
+      const int pq[4] = {pv.x, pv.y, pv.z, pv.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = 4 * c + q;
+        if (r < p.k && in) {
+          const bool reached = (on >> q) & 1u;
+          p.level[(long long)r * p.n + v] = reached ? (int)lb[q] : -1;
+          p.parent[(long long)r * p.n + v] = reached ? pq[q] : -1;
         }
       }
     }
-    __syncthreads();
   }
 }
 
@@ -541,8 +623,9 @@ int launch_batch(const BatchRequest& r, cudaStream_t s) {
   p.level = r.level;
   p.parent = r.parent;
   p.stride = r.width;
-  p.sl = w->bscr;
-  p.sp = w->bscr + (size_t)g->n * 64;
+  p.sp = w->bscr;
+  p.planes = w->bscr + (size_t)g->n * 64;
+  p.dead = g->d_dead;
   for (int i = 0; i < 3; ++i) {
     p.F[i] = w->bset[i];
     p.queue[i] = w->queue[i];

@@ -89,7 +89,7 @@ struct Workspace {
   // batched (64-root bitset) state, lazily
   uint64_t* bset[3] = {nullptr, nullptr, nullptr};
   uint64_t* bvis = nullptr;
-  int32_t* bscr = nullptr;  // batched: vertex-major scratch results, levels then parents, int32[2][n][64]
+  int32_t* bscr = nullptr;  // batched: vertex-major parents, int32[n][64], then level bit planes, up to 64 bits [31][n]
   // pinned host staging for schedules and multi-source seeds; `stage_ev` is
   // recorded after each copy out of it and waited on before it is rewritten
   int32_t* h_stage = nullptr;
