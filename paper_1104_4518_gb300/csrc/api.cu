@@ -282,25 +282,18 @@ static int make_graph_from_device_csr(int64_t* d_off, int32_t* d_adj, int32_t n,
     delete g;
     return cuda_fail(err, "part table copy");
   }
-  int rc = dev_alloc((void**)&g->d_dead, sizeof(uint32_t) * (((size_t)n + 31) / 32), "edgeless-vertex bitmap");
   // no arc enters a dead vertex; the big-row chunks serve the batched pull, which scans in-rows
-  if (!rc) rc = compute_dead_bits(g->d_toff, n, g->d_dead, nullptr);
-  if (!rc) rc = build_big_chunks(g->d_toff, n, nnz, nullptr, &g->d_big, &g->nbig);
-  // the pull works without probe records, only slower: a graph that leaves no room for them does without
-  if (!rc) rc = build_probe_records(g->d_toff, g->d_tadj, n, g->d_dead, nullptr, &g->d_probe, &g->d_rank);
-  if (!rc) {
-    err = cudaDeviceSynchronize();
-    if (err != cudaSuccess) rc = cuda_fail(err, "edgeless-vertex bitmap");
-  }
-  if (rc) {
-    if (g->d_dead) cudaFree(g->d_dead);
-    if (g->d_big) cudaFree(g->d_big);
-    if (g->d_probe) cudaFree(g->d_probe);
-    if (g->d_rank) cudaFree(g->d_rank);
+  RowTables t;
+  if (int rc = build_row_tables(g->d_toff, g->d_tadj, n, nnz, nullptr, &t)) {
     cudaFree(g->d_part_base);
     delete g;
     return rc;
   }
+  g->d_dead = t.dead;
+  g->d_rank = t.rank;
+  g->d_probe = t.probe;
+  g->d_big = t.big;
+  g->nbig = t.nbig;
   *out = g;
   return BFS_OK;
 }
@@ -536,7 +529,6 @@ void bfs_graph_destroy(bfs_graph* g) {
   if (g->d_dead) cudaFree(g->d_dead);
   if (g->d_big) cudaFree(g->d_big);
   if (g->d_probe) cudaFree(g->d_probe);
-  if (g->d_rank) cudaFree(g->d_rank);
   free_tiles(g->tiles);
   free_half(g);
   delete g;

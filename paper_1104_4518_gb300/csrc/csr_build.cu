@@ -1,83 +1,135 @@
-// Edge list -> symmetric, deduplicated, row-sorted CSR on the device, and the
-// CSR validation used by bfs_graph_create(BFS_VALIDATE).
+// Edge list -> symmetric, deduplicated, row-sorted CSR on the device, the row
+// tables that a graph keeps beside it, and the CSR validation used by
+// bfs_graph_create(BFS_VALIDATE).
 //
 // The paper stores each undirected edge in both rows with every row sorted
 // (Sec. 4.1) and its benchmark symmetrises the generated edges (Sec. 6).  Here:
 //   1. every non-loop edge (u, v) emits the keys (u << b) | v and (v << b) | u,
-//      b = bits of n - 1 (warp-aggregated append);
-//   2. the keys are sorted by a least-significant-digit radix sort over their
-//      2b significant bits, 8 bits per pass; each pass is a tile histogram, an
-//      exclusive scan of the digit-major histogram and a stable scatter whose
-//      in-tile ranks come from __match_any_sync on the digit;
-//   3. a key equal to its predecessor is a repeat; an exclusive scan of the
-//      "first of its value" flags gives every kept key its slot, the low b
-//      bits are the column, and the row changes between consecutive kept keys
-//      give the int64 row offsets.
+//      b = bits of n - 1, appended a tile at a time, and the digit histograms of
+//      all sort passes are counted on the way;
+//   2. the keys are sorted on their 2b significant bits (radix_sort.cu);
+//   3. a key equal to its predecessor is a repeat; one pass with a chained scan
+//      of the "first of its value" flags gives every kept key its slot and
+//      writes its column (the low b bits), and the row changes between
+//      consecutive keys give the int64 row offsets.
+// Nothing is read back before step 3 is enqueued: the number of keys stays on
+// the device.  The host waits twice, for the entry count and at the end.
 #include <algorithm>
 #include <cstdio>
 
 #include "device_common.cuh"
 #include "internal.h"
+#include "radix_sort.cuh"
 
 namespace bfsint {
 namespace {
 
 using bfsdev::kFull;
 
-constexpr int kSortThreads = 256;
-constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kKeysPerThread = 16;
-constexpr int kTile = kSortThreads * kKeysPerThread;  // 4096 keys
-constexpr int kRadix = 256;
-
 constexpr int kScanThreads = 512;
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kScanThreads * kScanItems;
 
+// What the construction kernels report; one block, cleared before them and read back after.
+struct BuildReport {
+  unsigned long long nkeys;  // keys emitted
+  unsigned long long nnz;    // keys kept
+  unsigned long long nlive;  // rows with entries
+  unsigned long long nbig;   // chunks of rows longer than kChunkEdges
+  int status[4];             // device status (BFS_ERR_TIMEOUT of a chained scan)
+  int bad;                   // an edge endpoint outside [0, n)
+  unsigned ticket;           // tiles handed out by the chained scan of this block's kernel
+};
+
 // ---------------- key emission ----------------
+constexpr int kKeyThreads = 256;
+constexpr int kKeyWarps = kKeyThreads / 32;
+constexpr int kKeyItems = 8;
+constexpr int kKeyTile = kKeyThreads * kKeyItems;  // 2,048 edges
+
 // Keys of the arcs of edge e = (u, v): mode 0 (undirected) emits u -> v and
-// v -> u, mode 1 u -> v only, mode 2 v -> u only (the transpose).
-__global__ void make_keys_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t m,
-                                 int32_t n, int vbits, int mode, uint64_t* __restrict__ keys,
-                                 unsigned long long* __restrict__ count, int* __restrict__ bad) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long mr = (m + 31) / 32 * 32;
-  const int lane = threadIdx.x & 31;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < mr; e += stride) {
-    int u = 0, v = 0;
-    bool ok = false;
-    if (e < m) {
-      u = src[e];
-      v = dst[e];
-      if (u < 0 || u >= n || v < 0 || v >= n) atomicExch(bad, 1);
-      else ok = (u != v);
+// v -> u, mode 1 u -> v only, mode 2 v -> u only (the transpose).  A tile's
+// keys take their places with one atomic (one per warp and step on the same
+// word made this kernel 1.48 ms for 67 M edges), in any order: the sort orders
+// them, and equal keys are alike.
+__global__ void __launch_bounds__(kKeyThreads) make_keys_kernel(const int32_t* __restrict__ src,
+                                                                const int32_t* __restrict__ dst, int64_t m, int32_t n,
+                                                                int vbits, int mode, SortPlan plan,
+                                                                uint64_t* __restrict__ keys,
+                                                                unsigned long long* __restrict__ hist,
+                                                                BuildReport* __restrict__ rep) {
+  __shared__ unsigned s_h[kSortMaxPasses * kSortBins];
+  __shared__ int s_cnt[kKeyItems * kKeyWarps];  // valid edges of each step and warp, then their exclusive sums
+  __shared__ unsigned long long s_at;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int per = mode == 0 ? 2 : 1;
+  for (int i = tid; i < plan.passes * kSortBins; i += kKeyThreads) s_h[i] = 0;
+  __syncthreads();
+  auto count = [&](uint64_t k) {
+    for (int q = 0; q < plan.passes; ++q)
+      atomicAdd(&s_h[q * kSortBins + (int)(k >> plan.shift[q] & ((1u << plan.bits[q]) - 1u))], 1u);
+  };
+  for (long long base = (long long)blockIdx.x * kKeyTile; base < m; base += (long long)gridDim.x * kKeyTile) {
+    int u[kKeyItems], v[kKeyItems];
+    unsigned bm[kKeyItems];
+    bool out = false;
+#pragma unroll
+    for (int i = 0; i < kKeyItems; ++i) {
+      const long long e = base + i * kKeyThreads + tid;
+      u[i] = e < m ? __ldg(&src[e]) : 0;
+      v[i] = e < m ? __ldg(&dst[e]) : 0;
     }
-    const unsigned bm = __ballot_sync(kFull, ok);
-    if (!bm) continue;
-    const unsigned long long per = mode == 0 ? 2ull : 1ull;
-    unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(count, per * __popc(bm));
-    base = __shfl_sync(kFull, base, 0);
-    if (ok) {
-      const unsigned long long at = base + per * __popc(bm & bfsdev::lanemask_lt());
-      if (mode != 2) keys[at] = ((uint64_t)u << vbits) | (uint64_t)v;
-      if (mode != 1) keys[at + (mode == 0 ? 1 : 0)] = ((uint64_t)v << vbits) | (uint64_t)u;
+#pragma unroll
+    for (int i = 0; i < kKeyItems; ++i) {
+      const bool in = (unsigned)u[i] < (unsigned)n && (unsigned)v[i] < (unsigned)n;
+      out |= !in;
+      bm[i] = __ballot_sync(kFull, in && u[i] != v[i]);  // an edge past m reads as the loop (0, 0)
+      if (lane == 0) s_cnt[i * kKeyWarps + wid] = __popc(bm[i]);
     }
+    if (out) atomicExch(&rep->bad, 1);
+    __syncthreads();
+    if (wid == 0) {  // exclusive sums over the 64 counts, two per lane
+      const int c0 = s_cnt[2 * lane], c1 = s_cnt[2 * lane + 1];
+      int incl = c0 + c1;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+      }
+      s_cnt[2 * lane] = incl - c0 - c1;
+      s_cnt[2 * lane + 1] = incl - c1;
+      if (lane == 31) s_at = incl ? atomicAdd(&rep->nkeys, (unsigned long long)(per * incl)) : 0ull;
+    }
+    __syncthreads();
+    const unsigned long long at = s_at;
+#pragma unroll
+    for (int i = 0; i < kKeyItems; ++i) {
+      if (!((bm[i] >> lane) & 1u)) continue;
+      const long long pos = (long long)at + (long long)per * (s_cnt[i * kKeyWarps + wid] + __popc(bm[i] & bfsdev::lanemask_lt()));
+      const uint64_t fwd = ((uint64_t)u[i] << vbits) | (uint64_t)v[i], rev = ((uint64_t)v[i] << vbits) | (uint64_t)u[i];
+      if (mode == 0) {
+        reinterpret_cast<ulonglong2*>(keys)[pos >> 1] = make_ulonglong2(fwd, rev);  // pos is even
+        count(fwd);
+        count(rev);
+      } else {
+        keys[pos] = mode == 1 ? fwd : rev;
+        count(mode == 1 ? fwd : rev);
+      }
+    }
+    __syncthreads();
   }
+  __syncthreads();
+  for (int i = tid; i < plan.passes * kSortBins; i += kKeyThreads)
+    if (s_h[i]) atomicAdd(&hist[i], (unsigned long long)s_h[i]);
 }
+static_assert(kKeyItems * kKeyWarps == 64, "the scan of the counts covers two per lane");
 
 // ---------------- exclusive scan (int64 output) ----------------
-// Input element i is in[i] (uint32 or int64 source) or, for the dedup flags,
-// "keys[i] differs from keys[i-1]".
+// Input element i is in[i] (uint32 or int64 source).
 struct ScanInput {
   const uint32_t* u32 = nullptr;
   const int64_t* i64 = nullptr;
-  const uint64_t* keys = nullptr;  // dedup flags
-  __device__ __forceinline__ long long at(long long i) const {
-    if (u32) return u32[i];
-    if (i64) return i64[i];
-    return (i == 0 || keys[i] != keys[i - 1]) ? 1 : 0;
-  }
+  __device__ __forceinline__ long long at(long long i) const { return u32 ? (long long)u32[i] : (long long)i64[i]; }
 };
 
 __device__ __forceinline__ long long block_scan_ll(long long x, long long* s_warp, long long& total) {
@@ -183,14 +235,9 @@ int exclusive_scan(const ScanInput& in, long long N, int64_t* out, cudaStream_t 
       err = cudaMemcpyAsync(&v, in.u32 + (N - 1), sizeof(v), cudaMemcpyDeviceToHost, s);
       if (err == cudaSuccess) err = cudaStreamSynchronize(s);
       last_in = v;
-    } else if (in.i64) {
+    } else {
       err = cudaMemcpyAsync(&last_in, in.i64 + (N - 1), sizeof(long long), cudaMemcpyDeviceToHost, s);
       if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-    } else {
-      uint64_t kk[2] = {0, 0};
-      if (N >= 2) err = cudaMemcpyAsync(kk, in.keys + (N - 2), 2 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s);
-      if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-      last_in = (N == 1 || kk[0] != kk[1]) ? 1 : 0;
     }
   }
   if (sums) cudaFree(sums);
@@ -200,94 +247,89 @@ int exclusive_scan(const ScanInput& in, long long N, int64_t* out, cudaStream_t 
   return BFS_OK;
 }
 
-// ---------------- radix sort passes ----------------
-__global__ void __launch_bounds__(kSortThreads) radix_hist_kernel(const uint64_t* __restrict__ keys, long long N,
-                                                                  int shift, uint32_t* __restrict__ hist,
-                                                                  long long ntiles) {
-  __shared__ uint32_t s_h[kRadix];
-  for (int i = threadIdx.x; i < kRadix; i += kSortThreads) s_h[i] = 0;
-  __syncthreads();
-  const long long base = (long long)blockIdx.x * kTile;
-  for (int i = threadIdx.x; i < kTile; i += kSortThreads) {
-    const long long idx = base + i;
-    if (idx < N) atomicAdd(&s_h[(keys[idx] >> shift) & (kRadix - 1)], 1u);
-  }
-  __syncthreads();
-  for (int d = threadIdx.x; d < kRadix; d += kSortThreads) hist[(long long)d * ntiles + blockIdx.x] = s_h[d];
-}
+// ---------------- dedup + CSR emission ----------------
+constexpr int kEmitThreads = 512;
+constexpr int kEmitWarps = kEmitThreads / 32;
+constexpr int kEmitItems = 16;
+constexpr int kEmitTile = kEmitThreads * kEmitItems;  // 8,192 keys
 
-__global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(const uint64_t* __restrict__ keys_in,
-                                                                     uint64_t* __restrict__ keys_out, long long N,
-                                                                     int shift, const int64_t* __restrict__ offs,
-                                                                     long long ntiles) {
-  __shared__ uint32_t s_cnt[kSortWarps][kRadix];
-  __shared__ long long s_goff[kRadix];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < kSortWarps * kRadix; i += kSortThreads) (&s_cnt[0][0])[i] = 0;
-  for (int d = threadIdx.x; d < kRadix; d += kSortThreads) s_goff[d] = offs[(long long)d * ntiles + blockIdx.x];
-  __syncthreads();
-  const long long seg = (long long)blockIdx.x * kTile + (long long)wid * (32 * kKeysPerThread);
-  uint64_t key[kKeysPerThread];
-  uint32_t rank[kKeysPerThread];
-  int dig[kKeysPerThread];
-#pragma unroll
-  for (int i = 0; i < kKeysPerThread; ++i) {
-    const long long idx = seg + i * 32 + lane;
-    const bool valid = idx < N;
-    key[i] = valid ? keys_in[idx] : 0;
-    const int d = valid ? (int)((key[i] >> shift) & (kRadix - 1)) : kRadix;
-    dig[i] = d;
-    const unsigned peers = __match_any_sync(kFull, d);
-    uint32_t r = 0;
-    if (valid) r = s_cnt[wid][d] + __popc(peers & bfsdev::lanemask_lt());
-    __syncwarp();
-    if (valid && (peers & bfsdev::lanemask_lt()) == 0) s_cnt[wid][d] += __popc(peers);
-    __syncwarp();
-    rank[i] = r;
+// One read of the sorted keys: every key that differs from its predecessor is
+// kept, its slot is the number of kept keys before it (within the warp's 512
+// consecutive keys by ballots, across tiles by a chained scan), and where its
+// row differs from the predecessor's the rows in between start at that slot.
+// 134 M keys: 0.72 ms (a flag scan and an emission kernel took 1.7 ms).
+__global__ void __launch_bounds__(kEmitThreads, 2) emit_csr_kernel(const uint64_t* __restrict__ keys, int vbits, int32_t n,
+                                                                int64_t* __restrict__ off, int32_t* __restrict__ adj,
+                                                                uint64_t* __restrict__ state, BuildReport* rep) {
+  __shared__ int s_cnt[kEmitWarps];
+  __shared__ unsigned s_tile;
+  __shared__ unsigned long long s_at;
+  __shared__ int s_ok;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (tid == 0) {
+    s_tile = atomicAdd(&rep->ticket, 1u);
+    s_ok = bfsdev::ld_relaxed_i32(rep->status) == 0;
   }
   __syncthreads();
-  // per digit: exclusive prefix over the warps of the tile
-  for (int d = threadIdx.x; d < kRadix; d += kSortThreads) {
-    uint32_t run = 0;
-    for (int w = 0; w < kSortWarps; ++w) {
-      const uint32_t c = s_cnt[w][d];
-      s_cnt[w][d] = run;
-      run += c;
+  const long long N = (long long)rep->nkeys, tile = s_tile, seg = tile * kEmitTile + wid * (32 * kEmitItems);
+  if (tile * kEmitTile >= N || !s_ok) return;
+  const uint64_t vmask = (1ull << vbits) - 1ull;
+  uint64_t key[kEmitItems];
+#pragma unroll
+  for (int i = 0; i < kEmitItems; ++i) key[i] = seg + i * 32 + lane < N ? keys[seg + i * 32 + lane] : 0;
+  uint64_t before = 0;  // the key before the warp's first
+  if (seg > 0 && seg < N) before = keys[seg - 1];
+  unsigned kept[kEmitItems];
+  int cnt = 0;
+#pragma unroll
+  for (int i = 0; i < kEmitItems; ++i) {
+    const long long idx = seg + i * 32 + lane;
+    uint64_t prev = __shfl_up_sync(kFull, key[i], 1);
+    const uint64_t carry = i > 0 ? __shfl_sync(kFull, key[i > 0 ? i - 1 : 0], 31) : before;
+    if (lane == 0) prev = carry;
+    kept[i] = __ballot_sync(kFull, idx < N && (idx == 0 || key[i] != prev));
+    cnt += __popc(kept[i]);
+  }
+  if (lane == 0) s_cnt[wid] = cnt;
+  __syncthreads();
+  int warp_at = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kEmitWarps; ++w) {
+    warp_at += w < wid ? s_cnt[w] : 0;
+    total += s_cnt[w];
+  }
+  if (wid == 0) {
+    if (lane == 0) publish_tile(state + tile, tile == 0 ? kTilePrefix : kTileSum, 1, (uint64_t)total);
+    uint64_t sum = 0;
+    const bool ok = sum_before_warp(state, tile, 1, rep->status, sum);
+    if (lane == 0) {
+      if (ok && tile > 0) publish_tile(state + tile, kTilePrefix, 1, sum + (uint64_t)total);
+      s_ok = ok;
+      s_at = sum;
     }
   }
   __syncthreads();
+  if (!s_ok) return;
+  long long at = (long long)s_at + warp_at;
 #pragma unroll
-  for (int i = 0; i < kKeysPerThread; ++i) {
-    const int d = dig[i];
-    if (d < kRadix) keys_out[s_goff[d] + s_cnt[wid][d] + rank[i]] = key[i];
+  for (int i = 0; i < kEmitItems; ++i) {
+    const long long idx = seg + i * 32 + lane;
+    uint64_t prev = __shfl_up_sync(kFull, key[i], 1);
+    const uint64_t carry = i > 0 ? __shfl_sync(kFull, key[i > 0 ? i - 1 : 0], 31) : before;
+    if (lane == 0) prev = carry;
+    const long long pos = at + __popc(kept[i] & bfsdev::lanemask_lt());
+    const bool first = (kept[i] >> lane) & 1u;
+    const long long row = (long long)(key[i] >> vbits);
+    if (first) {
+      adj[pos] = (int32_t)(key[i] & vmask);
+      for (long long r = idx == 0 ? 0 : (long long)(prev >> vbits) + 1; r <= row; ++r) off[r] = pos;
+    }
+    if (idx == N - 1) {  // the rows after the last key's end with it
+      rep->nnz = (unsigned long long)(pos + (first ? 1 : 0));
+      for (long long r = row + 1; r <= n; ++r) off[r] = pos + (first ? 1 : 0);
+    }
+    at += __popc(kept[i]);
   }
-}
-
-// ---------------- dedup + CSR emission ----------------
-__global__ void emit_csr_kernel(const uint64_t* __restrict__ keys, const int64_t* __restrict__ pos, long long N,
-                                int vbits, int32_t n, long long nnz, int64_t* __restrict__ off,
-                                int32_t* __restrict__ adj) {
-  const uint64_t vmask = (1ull << vbits) - 1ull;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
-    const uint64_t k = keys[i];
-    // the rows after the last key's row end at nnz (the last key may repeat an
-    // earlier one, so this cannot wait for a first occurrence)
-    if (i == N - 1)
-      for (long long r = (long long)(k >> vbits) + 1; r <= n; ++r) off[r] = nnz;
-    const bool first = (i == 0) || k != keys[i - 1];
-    if (!first) continue;
-    const long long p = pos[i];
-    adj[p] = (int32_t)(k & vmask);
-    const long long u = (long long)(k >> vbits);
-    const long long pu = (i == 0) ? -1 : (long long)(keys[i - 1] >> vbits);
-    for (long long r = pu + 1; r <= u; ++r) off[r] = p;
-  }
-}
-
-__global__ void fill_offsets_kernel(int64_t* off, int32_t n, long long value) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r <= n; r += stride) off[r] = value;
 }
 
 // ---------------- validation ----------------
@@ -348,15 +390,91 @@ __global__ void shift_kernel(int64_t* off, int32_t* adj, long long n_part, long 
   for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < nnz_part; j += stride) adj[j] += id_shift;
 }
 
-__global__ void dead_bits_kernel(const int64_t* __restrict__ off, int32_t n, long long nwords, uint32_t* out) {
-  const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32;
-  const long long stride = (long long)gridDim.x * blockDim.x / 32;
+// ---------------- row tables ----------------
+constexpr int kMetaThreads = 512;
+constexpr int kMetaWarps = kMetaThreads / 32;
+constexpr int kMetaTile = kMetaThreads;  // bitmap words per CTA: 32 per warp, lane j keeps word j
+
+// Per bitmap word: its vertices without entries (`dead`, tail bits set) and the
+// number of rows with entries before it (`rank`); in all, the rows with entries
+// and the chunks of long rows.
+__global__ void __launch_bounds__(kMetaThreads) row_meta_kernel(const int64_t* __restrict__ off, int32_t n,
+                                                                long long nwords, uint32_t* __restrict__ dead,
+                                                                uint32_t* __restrict__ rank, uint64_t* __restrict__ state,
+                                                                BuildReport* rep) {
+  __shared__ int s_cnt[kMetaWarps];
+  __shared__ unsigned s_tile;
+  __shared__ unsigned long long s_at;
+  __shared__ int s_ok;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (tid == 0) s_tile = atomicAdd(&rep->ticket, 1u);
+  __syncthreads();
+  const long long tile = s_tile, w0 = tile * kMetaTile + wid * 32;
+  uint32_t live = 0;
+  unsigned long long big = 0;
+#pragma unroll 8
+  for (int j = 0; j < 32; ++j) {
+    const long long v = (w0 + j) * 32 + lane;
+    const long long d = v < n ? off[v + 1] - off[v] : 0;
+    const uint32_t m = __ballot_sync(kFull, d > 0);
+    if (lane == j) live = m;
+    if (d > kChunkEdges) big += (unsigned long long)((d + kChunkEdges - 1) / kChunkEdges);
+  }
+  if (big) atomicAdd(&rep->nbig, big);
+  const int c = __popc(live);
+  int incl = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) s_cnt[wid] = incl;
+  __syncthreads();
+  int warp_at = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kMetaWarps; ++w) {
+    warp_at += w < wid ? s_cnt[w] : 0;
+    total += s_cnt[w];
+  }
+  if (wid == 0) {
+    if (lane == 0) publish_tile(state + tile, tile == 0 ? kTilePrefix : kTileSum, 1, (uint64_t)total);
+    uint64_t sum = 0;
+    const bool ok = sum_before_warp(state, tile, 1, rep->status, sum);
+    if (lane == 0) {
+      if (ok && tile > 0) publish_tile(state + tile, kTilePrefix, 1, sum + (uint64_t)total);
+      if ((tile + 1) * kMetaTile >= nwords) rep->nlive = sum + (uint64_t)total;
+      s_ok = ok;
+      s_at = sum;
+    }
+  }
+  __syncthreads();
+  const long long w = w0 + lane;
+  if (!s_ok || w >= nwords) return;
+  dead[w] = ~live;
+  rank[w] = (uint32_t)(s_at + warp_at + incl - c);
+}
+
+// Probe records of the rows with entries (out non-null): one warp per bitmap
+// word, packed in id order; and the chunk items of rows longer than kChunkEdges,
+// in any order.
+__global__ void row_records_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
+                                   const uint32_t* __restrict__ dead, const uint32_t* __restrict__ rank,
+                                   long long nwords, int4* __restrict__ out, int64_t* __restrict__ big,
+                                   unsigned long long* big_count) {
   const int lane = threadIdx.x & 31;
-  for (long long w = gw; w < nwords; w += stride) {
-    const long long v = w * 32 + lane;
-    const bool dead = v >= n || off[v + 1] == off[v];
-    const unsigned m = __ballot_sync(kFull, dead);
-    if (lane == 0) out[w] = m;
+  const long long stride = (long long)gridDim.x * blockDim.x / 32;
+  for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32; w < nwords; w += stride) {
+    const uint32_t live = ~dead[w];  // the bits past n are dead
+    if (!((live >> lane) & 1u)) continue;
+    const long long v = w * 32 + lane, b = off[v], e = off[v + 1], d = e - b;
+    if (out)
+      out[(long long)rank[w] + __popc(live & bfsdev::lanemask_lt())] =
+          make_int4((int)d, adj[e - 1], d > 1 ? adj[e - 2] : 0, d > 2 ? adj[e - 3] : 0);
+    if (d > kChunkEdges) {
+      const unsigned long long nch = (unsigned long long)((d + kChunkEdges - 1) / kChunkEdges);
+      const unsigned long long pos = atomicAdd(big_count, nch);
+      for (unsigned long long c = 0; c < nch; ++c) big[pos + c] = (v << 32) | (long long)c;
+    }
   }
 }
 
@@ -373,42 +491,6 @@ __global__ void expand_rows_kernel(const int64_t* __restrict__ off, int32_t n, l
   }
 }
 
-__global__ void big_chunks_kernel(const int64_t* __restrict__ off, int32_t n, int64_t* items,
-                                  unsigned long long* count) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-    const long long deg = off[v + 1] - off[v];
-    if (deg <= kChunkEdges) continue;
-    const unsigned long long nch = (unsigned long long)((deg + kChunkEdges - 1) / kChunkEdges);
-    const unsigned long long pos = atomicAdd(count, nch);
-    for (unsigned long long c = 0; c < nch; ++c) items[pos + c] = (v << 32) | (long long)c;
-  }
-}
-
-// cnt[w] = vertices of bitmap word w with entries.
-__global__ void live_count_kernel(const uint32_t* __restrict__ dead, long long nwords, uint32_t* __restrict__ cnt) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x; w < nwords; w += stride) cnt[w] = __popc(~dead[w]);
-}
-
-// One warp per bitmap word: the records of its vertices, packed, and the word's rank.
-__global__ void probe_records_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
-                                     const uint32_t* __restrict__ dead, const int64_t* __restrict__ pos,
-                                     long long nwords, int4* __restrict__ out, uint32_t* __restrict__ rank) {
-  const int lane = threadIdx.x & 31;
-  const long long stride = (long long)gridDim.x * blockDim.x / 32;
-  for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32; w < nwords; w += stride) {
-    const uint32_t live = ~dead[w];  // the bits past n are dead
-    const int64_t base = pos[w];
-    if (lane == 0) rank[w] = (uint32_t)base;
-    if ((live >> lane) & 1u) {
-      const long long v = w * 32 + lane, b = off[v], e = off[v + 1], d = e - b;
-      out[base + __popc(live & bfsdev::lanemask_lt())] =
-          make_int4((int)d, adj[e - 1], d > 1 ? adj[e - 2] : 0, d > 2 ? adj[e - 3] : 0);
-    }
-  }
-}
-
 int bits_for(int32_t n) {
   int b = 1;
   while (b < 31 && ((int64_t)1 << b) < (int64_t)n) ++b;
@@ -416,44 +498,6 @@ int bits_for(int32_t n) {
 }
 
 }  // namespace
-
-int radix_sort_u64(uint64_t* keys, uint64_t* alt, long long N, int lo_bit, int hi_bit, cudaStream_t s,
-                   uint64_t** sorted) {
-  *sorted = keys;
-  if (N <= 0 || lo_bit >= hi_bit) return BFS_OK;
-  const long long ntiles = (N + kTile - 1) / kTile;
-  const long long hsize = ntiles * kRadix;
-  uint32_t* hist = nullptr;
-  int64_t* hoff = nullptr;
-  if (int e = dev_alloc((void**)&hist, sizeof(uint32_t) * hsize, "radix histogram")) return e;
-  if (int e = dev_alloc((void**)&hoff, sizeof(int64_t) * hsize, "radix offsets")) {
-    cudaFree(hist);
-    return e;
-  }
-  uint64_t* a = keys;
-  uint64_t* b = alt;
-  int rc = BFS_OK;
-  for (int shift = lo_bit; shift < hi_bit && !rc; shift += 8) {
-    radix_hist_kernel<<<(unsigned)ntiles, kSortThreads, 0, s>>>(a, N, shift, hist, ntiles);
-    ScanInput si;
-    si.u32 = hist;
-    long long tot = 0;
-    rc = exclusive_scan(si, hsize, hoff, s, &tot);
-    if (rc) break;
-    radix_scatter_kernel<<<(unsigned)ntiles, kSortThreads, 0, s>>>(a, b, N, shift, hoff, ntiles);
-    uint64_t* t = a;
-    a = b;
-    b = t;
-  }
-  cudaError_t err = cudaGetLastError();
-  if (!rc && err == cudaSuccess) err = cudaStreamSynchronize(s);
-  cudaFree(hist);
-  cudaFree(hoff);
-  if (rc) return rc;
-  if (err != cudaSuccess) return cuda_fail(err, "radix sort");
-  *sorted = a;
-  return BFS_OK;
-}
 
 int exclusive_scan_u32(const uint32_t* in, long long N, int64_t* out, cudaStream_t s, long long* total) {
   ScanInput si;
@@ -466,179 +510,111 @@ int build_csr_from_edges(const int32_t* d_src, const int32_t* d_dst, int64_t m, 
   DeviceInfo di;
   if (int e = current_device_info(&di)) return e;
   const int vbits = bits_for(n);
-  const int total_bits = 2 * vbits;
-  uint64_t* keys = nullptr;
-  uint64_t* keys_alt = nullptr;
-  unsigned long long* d_count = nullptr;
-  int* d_bad = nullptr;
-  uint32_t* hist = nullptr;
-  int64_t* hoff = nullptr;
-  int64_t* pos = nullptr;
+  const SortPlan plan = sort_plan(0, 2 * vbits);
+  const long long cap = (mode == 0 ? 2 : 1) * (long long)m;
+  const long long emit_tiles = (cap + kEmitTile - 1) / kEmitTile;
+  // one scratch block: report | sort tables | emission tiles (all cleared) | keys | alternate keys
+  const size_t rep_bytes = 256, sort_bytes = (sort_scratch_bytes(cap) + 255) / 256 * 256;
+  const size_t emit_bytes = (sizeof(uint64_t) * (size_t)emit_tiles + 255) / 256 * 256;
+  const size_t key_bytes = (sizeof(uint64_t) * (size_t)cap + 255) / 256 * 256;
+  char* block = nullptr;
   int64_t* off = nullptr;
   int32_t* adj = nullptr;
-  int rc = BFS_OK;
-  long long N = 0, nnz = 0;
-  const long long cap = (mode == 0 ? 2 : 1) * (long long)m;
-  auto cleanup = [&]() {
-    if (keys) cudaFree(keys);
-    if (keys_alt) cudaFree(keys_alt);
-    if (d_count) cudaFree(d_count);
-    if (d_bad) cudaFree(d_bad);
-    if (hist) cudaFree(hist);
-    if (hoff) cudaFree(hoff);
-    if (pos) cudaFree(pos);
+  BuildReport rep{};
+  auto give_up = [&](int rc) {
+    if (block) cudaFree(block);
+    if (off) cudaFree(off);
+    if (adj) cudaFree(adj);
+    return rc;
   };
-  if ((rc = dev_alloc((void**)&d_count, sizeof(unsigned long long) + 16, "edge count"))) return cleanup(), rc;
-  if ((rc = dev_alloc((void**)&d_bad, sizeof(int) * 4, "flag"))) return cleanup(), rc;
-  if ((rc = dev_alloc((void**)&off, sizeof(int64_t) * ((size_t)n + 1), "CSR offsets"))) return cleanup(), rc;
-  cudaError_t err = cudaMemsetAsync(d_count, 0, sizeof(unsigned long long), s);
-  if (err == cudaSuccess) err = cudaMemsetAsync(d_bad, 0, sizeof(int), s);
-  if (err != cudaSuccess) {
-    cleanup();
-    cudaFree(off);
-    return cuda_fail(err, "memset");
-  }
+  if (int e = dev_alloc((void**)&off, sizeof(int64_t) * ((size_t)n + 1), "CSR offsets")) return give_up(e);
+  uint64_t* sorted = nullptr;
   if (cap > 0) {
-    if ((rc = dev_alloc((void**)&keys, sizeof(uint64_t) * cap, "sort keys"))) return cleanup(), cudaFree(off), rc;
-    const int grid = di.sm_count * 8;
-    make_keys_kernel<<<grid, 256, 0, s>>>(d_src, d_dst, m, n, vbits, mode, keys, d_count, d_bad);
-    int bad = 0;
-    unsigned long long cnt = 0;
-    err = cudaGetLastError();
-    if (err == cudaSuccess) err = cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (err == cudaSuccess) err = cudaMemcpyAsync(&cnt, d_count, sizeof(cnt), cudaMemcpyDeviceToHost, s);
+    if (int e = dev_alloc((void**)&block, rep_bytes + sort_bytes + emit_bytes + 2 * key_bytes, "sort keys")) return give_up(e);
+    BuildReport* d_rep = reinterpret_cast<BuildReport*>(block);
+    const SortScratch sc = sort_scratch_at(block + rep_bytes, cap);
+    uint64_t* tiles = reinterpret_cast<uint64_t*>(block + rep_bytes + sort_bytes);
+    uint64_t* keys = reinterpret_cast<uint64_t*>(block + rep_bytes + sort_bytes + emit_bytes);
+    uint64_t* alt = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(keys) + key_bytes);
+    cudaError_t err = cudaMemsetAsync(block, 0, rep_bytes + sort_bytes + emit_bytes, s);
+    if (err == cudaSuccess) {
+      const long long key_tiles = (m + kKeyTile - 1) / kKeyTile;
+      make_keys_kernel<<<(unsigned)std::min<long long>(key_tiles, 4ll * di.sm_count), kKeyThreads, 0, s>>>(
+          d_src, d_dst, m, n, vbits, mode, plan, keys, sc.hist, d_rep);
+      sorted = launch_sort_passes(keys, alt, cap, &d_rep->nkeys, plan, sc, d_rep->status, s);
+      // the columns go to the free key buffer until their number is known
+      emit_csr_kernel<<<(unsigned)emit_tiles, kEmitThreads, 0, s>>>(
+          sorted, vbits, n, off, reinterpret_cast<int32_t*>(sorted == keys ? alt : keys), tiles, d_rep);
+      err = cudaGetLastError();
+    }
+    if (err == cudaSuccess) err = cudaMemcpyAsync(&rep, d_rep, sizeof(rep), cudaMemcpyDeviceToHost, s);
     if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-    if (err != cudaSuccess) {
-      cleanup();
-      cudaFree(off);
-      return cuda_fail(err, "key emission");
-    }
-    if (bad) {
-      cleanup();
-      cudaFree(off);
-      return fail(BFS_ERR_INVALID_ARG, "edge endpoint outside [0, n)");
-    }
-    N = (long long)cnt;
+    if (err != cudaSuccess) return give_up(cuda_fail(err, "CSR construction"));
+    if (rep.status[0]) return give_up(fail(rep.status[0], "CSR construction: " + device_status_message(rep.status)));
+    if (rep.bad) return give_up(fail(BFS_ERR_INVALID_ARG, "edge endpoint outside [0, n)"));
+    if (int e = dev_alloc((void**)&adj, sizeof(int32_t) * (size_t)std::max(1ull, rep.nnz), "CSR adjacency")) return give_up(e);
+    if (rep.nnz > 0)
+      err = cudaMemcpyAsync(adj, sorted == keys ? alt : keys, sizeof(int32_t) * (size_t)rep.nnz, cudaMemcpyDeviceToDevice, s);
+    if (err != cudaSuccess) return give_up(cuda_fail(err, "CSR construction"));
+  } else if (int e = dev_alloc((void**)&adj, sizeof(int32_t), "CSR adjacency")) {
+    return give_up(e);
   }
-  if (N > 0) {
-    if ((rc = dev_alloc((void**)&keys_alt, sizeof(uint64_t) * N, "sort keys (alternate)")))
-      return cleanup(), cudaFree(off), rc;
-    const long long ntiles = (N + kTile - 1) / kTile;
-    const long long hsize = ntiles * kRadix;
-    if ((rc = dev_alloc((void**)&hist, sizeof(uint32_t) * hsize, "radix histogram")))
-      return cleanup(), cudaFree(off), rc;
-    if ((rc = dev_alloc((void**)&hoff, sizeof(int64_t) * hsize, "radix offsets")))
-      return cleanup(), cudaFree(off), rc;
-    uint64_t* a = keys;
-    uint64_t* b = keys_alt;
-    for (int shift = 0; shift < total_bits; shift += 8) {
-      radix_hist_kernel<<<(unsigned)ntiles, kSortThreads, 0, s>>>(a, N, shift, hist, ntiles);
-      ScanInput si;
-      si.u32 = hist;
-      long long tot = 0;
-      if ((rc = exclusive_scan(si, hsize, hoff, s, &tot))) return cleanup(), cudaFree(off), rc;
-      radix_scatter_kernel<<<(unsigned)ntiles, kSortThreads, 0, s>>>(a, b, N, shift, hoff, ntiles);
-      uint64_t* t = a;
-      a = b;
-      b = t;
-    }
-    // a holds the sorted keys
-    cudaFree(hist);
-    hist = nullptr;
-    cudaFree(hoff);
-    hoff = nullptr;
-    if ((rc = dev_alloc((void**)&pos, sizeof(int64_t) * N, "dedup positions"))) return cleanup(), cudaFree(off), rc;
-    ScanInput fi;
-    fi.keys = a;
-    if ((rc = exclusive_scan(fi, N, pos, s, &nnz))) return cleanup(), cudaFree(off), rc;
-    if ((rc = dev_alloc((void**)&adj, sizeof(int32_t) * (nnz > 0 ? nnz : 1), "CSR adjacency")))
-      return cleanup(), cudaFree(off), rc;
-    emit_csr_kernel<<<di.sm_count * 8, 256, 0, s>>>(a, pos, N, vbits, n, nnz, off, adj);
-  } else {
-    if ((rc = dev_alloc((void**)&adj, sizeof(int32_t), "CSR adjacency"))) return cleanup(), cudaFree(off), rc;
-    fill_offsets_kernel<<<di.sm_count, 256, 0, s>>>(off, n, 0);
+  if (rep.nkeys == 0) {  // no key: the emission wrote no offset
+    cudaError_t err = cudaMemsetAsync(off, 0, sizeof(int64_t) * ((size_t)n + 1), s);
+    if (err != cudaSuccess) return give_up(cuda_fail(err, "CSR construction"));
   }
-  err = cudaGetLastError();
-  if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-  cleanup();
-  if (err != cudaSuccess) {
-    cudaFree(off);
-    cudaFree(adj);
-    return cuda_fail(err, "CSR construction");
-  }
+  cudaError_t err = cudaStreamSynchronize(s);
+  if (err != cudaSuccess) return give_up(cuda_fail(err, "CSR construction"));
+  if (block) cudaFree(block);
   *d_off_out = off;
   *d_adj_out = adj;
-  *nnz_out = nnz;
+  *nnz_out = (int64_t)rep.nnz;
   return BFS_OK;
 }
 
-int compute_dead_bits(const int64_t* d_off, int32_t n, uint32_t* d_dead, cudaStream_t s) {
+int build_row_tables(const int64_t* d_off, const int32_t* d_adj, int32_t n, int64_t nnz, cudaStream_t s, RowTables* out) {
   DeviceInfo di;
   if (int e = current_device_info(&di)) return e;
-  dead_bits_kernel<<<di.sm_count * 4, 256, 0, s>>>(d_off, n, ((long long)n + 31) / 32, d_dead);
-  BFS_CUDA_TRY(cudaGetLastError());
-  return BFS_OK;
-}
-
-int build_probe_records(const int64_t* d_off, const int32_t* d_adj, int32_t n, const uint32_t* d_dead, cudaStream_t s,
-                        int4** d_probe, uint32_t** d_rank) {
-  *d_probe = nullptr;
-  *d_rank = nullptr;
-  DeviceInfo di;
-  if (int e = current_device_info(&di)) return e;
-  const long long nwords = ((long long)n + 31) / 32;
-  uint32_t* rank = nullptr;
-  int64_t* pos = nullptr;
-  int4* rec = nullptr;
-  if (dev_alloc((void**)&rank, sizeof(uint32_t) * nwords, "record ranks")) return BFS_OK;
-  if (dev_alloc((void**)&pos, sizeof(int64_t) * nwords, "record positions")) return cudaFree(rank), BFS_OK;
-  live_count_kernel<<<di.sm_count * 4, 256, 0, s>>>(d_dead, nwords, rank);
-  long long total = 0;
-  int rc = exclusive_scan_u32(rank, nwords, pos, s, &total);
-  if (!rc && !dev_alloc((void**)&rec, sizeof(int4) * (size_t)std::max(total, 1ll), "probe records")) {
-    probe_records_kernel<<<di.sm_count * 8, 256, 0, s>>>(d_off, d_adj, d_dead, pos, nwords, rec, rank);
-    cudaError_t err = cudaGetLastError();
-    if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-    if (err != cudaSuccess) rc = cuda_fail(err, "probe records");
-  }
-  cudaFree(pos);
-  if (rc || !rec) {
-    cudaFree(rank);
-    if (rec) cudaFree(rec);
+  *out = RowTables{};
+  const long long nwords = ((long long)n + 31) / 32, tiles = (nwords + kMetaTile - 1) / kMetaTile;
+  const size_t word_bytes = (sizeof(uint32_t) * (size_t)nwords + 255) / 256 * 256;
+  RowTables t;
+  char* scratch = nullptr;
+  if (int e = dev_alloc((void**)&t.dead, 2 * word_bytes, "row bitmaps")) return e;
+  t.rank = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(t.dead) + word_bytes);
+  BuildReport rep{};
+  auto give_up = [&](int rc) {
+    if (scratch) cudaFree(scratch);
+    if (t.probe) cudaFree(t.probe);
+    if (t.big) cudaFree(t.big);
+    cudaFree(t.dead);
     return rc;
-  }
-  *d_probe = rec;
-  *d_rank = rank;
-  return BFS_OK;
-}
-
-int build_big_chunks(const int64_t* d_off, int32_t n, int64_t nnz, cudaStream_t s, int64_t** items_out,
-                     int64_t* count_out) {
-  DeviceInfo di;
-  if (int e = current_device_info(&di)) return e;
-  const long long cap = 2 * (nnz / kChunkEdges) + 2;  // sum of ceil(deg / C) over rows with deg > C
-  int64_t* items = nullptr;
-  unsigned long long* d_count = nullptr;
-  if (int e = dev_alloc((void**)&items, sizeof(int64_t) * cap, "high-degree row chunks")) return e;
-  if (int e = dev_alloc((void**)&d_count, sizeof(unsigned long long), "chunk count")) {
-    cudaFree(items);
-    return e;
-  }
-  unsigned long long cnt = 0;
-  cudaError_t err = cudaMemsetAsync(d_count, 0, sizeof(unsigned long long), s);
+  };
+  const size_t bytes = 256 + sizeof(uint64_t) * (size_t)tiles;
+  if (int e = dev_alloc((void**)&scratch, bytes, "row table tiles")) return give_up(e);
+  BuildReport* d_rep = reinterpret_cast<BuildReport*>(scratch);
+  cudaError_t err = cudaMemsetAsync(scratch, 0, bytes, s);
   if (err == cudaSuccess) {
-    big_chunks_kernel<<<di.sm_count * 4, 256, 0, s>>>(d_off, n, items, d_count);
+    row_meta_kernel<<<(unsigned)tiles, kMetaThreads, 0, s>>>(d_off, n, nwords, t.dead, t.rank,
+                                                             reinterpret_cast<uint64_t*>(scratch + 256), d_rep);
     err = cudaGetLastError();
   }
-  if (err == cudaSuccess) err = cudaMemcpyAsync(&cnt, d_count, sizeof(cnt), cudaMemcpyDeviceToHost, s);
+  if (err == cudaSuccess) err = cudaMemcpyAsync(&rep, d_rep, sizeof(rep), cudaMemcpyDeviceToHost, s);
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-  cudaFree(d_count);
-  if (err != cudaSuccess) {
-    cudaFree(items);
-    return cuda_fail(err, "high-degree row chunks");
-  }
-  *items_out = items;
-  *count_out = (int64_t)cnt;
+  if (err != cudaSuccess) return give_up(cuda_fail(err, "row tables"));
+  if (rep.status[0]) return give_up(fail(rep.status[0], "row tables: " + device_status_message(rep.status)));
+  t.nbig = (int64_t)rep.nbig;
+  if (t.nbig > 0)
+    if (int e = dev_alloc((void**)&t.big, sizeof(int64_t) * (size_t)t.nbig, "high-degree row chunks")) return give_up(e);
+  // the pull works without probe records, only slower: a graph that leaves no room for them does without
+  if (dev_alloc((void**)&t.probe, sizeof(int4) * (size_t)std::max(1ull, rep.nlive), "probe records") != BFS_OK)
+    t.probe = nullptr;
+  row_records_kernel<<<di.sm_count * 8, 256, 0, s>>>(d_off, d_adj, t.dead, t.rank, nwords, t.probe, t.big, &d_rep->nkeys);
+  err = cudaGetLastError();
+  if (err == cudaSuccess) err = cudaStreamSynchronize(s);
+  if (err != cudaSuccess) return give_up(cuda_fail(err, "row tables"));
+  cudaFree(scratch);
+  *out = t;
   return BFS_OK;
 }
 

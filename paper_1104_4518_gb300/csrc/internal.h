@@ -172,8 +172,8 @@ bfs_tuning effective_tuning(const bfs_graph* g);
 int build_csr_from_edges(const int32_t* d_src, const int32_t* d_dst, int64_t m, int32_t n, int mode,
                          cudaStream_t s, int64_t** d_off, int32_t** d_adj, int64_t* nnz);
 // Stable least-significant-digit radix sort of N 64-bit keys on bits
-// [lo_bit, hi_bit), 8 bits per pass; alt is scratch of N keys; *sorted is
-// whichever of the two buffers holds the result.  Synchronises s.
+// [lo_bit, hi_bit); alt is scratch of N keys; *sorted is whichever of the two
+// buffers holds the result.  Synchronises s.
 int radix_sort_u64(uint64_t* keys, uint64_t* alt, long long N, int lo_bit, int hi_bit, cudaStream_t s,
                    uint64_t** sorted);
 // Exclusive prefix sum of N uint32 values into int64 out; *total receives the sum.
@@ -193,14 +193,17 @@ int check_offsets(const int64_t* d_off, int32_t n, int64_t nnz, int* d_flag, cud
 // The transpose of a directed CSR (row v lists the tails u of the arcs u -> v).
 int build_transpose(const int64_t* d_off, const int32_t* d_adj, int32_t n, int64_t nnz, cudaStream_t s,
                     int64_t** d_toff, int32_t** d_tadj);
-// Bitmap of the vertices without edges (bits beyond n set), one word per 32 vertices.
-int compute_dead_bits(const int64_t* d_off, int32_t n, uint32_t* d_dead, cudaStream_t s);
-// Probe record of every non-empty row: its length and its last three entries (the largest ids), 0 past the row.
-// d_dead is the bitmap of the empty rows.  Without room for them *d_probe and *d_rank stay null.  Synchronises s.
-int build_probe_records(const int64_t* d_off, const int32_t* d_adj, int32_t n, const uint32_t* d_dead, cudaStream_t s,
-                        int4** d_probe, uint32_t** d_rank);
-// Chunk items of every row longer than kChunkEdges (order unspecified); *count receives their number.
-int build_big_chunks(const int64_t* d_off, int32_t n, int64_t nnz, cudaStream_t s, int64_t** items, int64_t* count);
+// Tables of a graph's in-rows, each null where there is nothing to hold or (probe) no room; `dead` and `rank`
+// share one allocation.
+struct RowTables {
+  uint32_t* dead = nullptr;  // bitmap of the vertices without entries (bits beyond n set)
+  uint32_t* rank = nullptr;  // per bitmap word: the vertices with entries before it
+  int4* probe = nullptr;     // per vertex with entries: its row's length and last three entries (the largest ids), 0 past the row
+  int64_t* big = nullptr;    // chunk items of every row longer than kChunkEdges (order unspecified)
+  int64_t nbig = 0;
+};
+// Synchronises s.
+int build_row_tables(const int64_t* d_off, const int32_t* d_adj, int32_t n, int64_t nnz, cudaStream_t s, RowTables* out);
 // Adds off_shift to n_part offsets and id_shift to nnz_part ids (union building).
 int union_shift(int64_t* off, int32_t* adj, int64_t n_part, int64_t nnz_part, int64_t off_shift, int32_t id_shift,
                 cudaStream_t s);
