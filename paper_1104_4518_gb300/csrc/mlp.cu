@@ -18,7 +18,7 @@ using namespace bfsdev;
 
 constexpr int kFwdThreads = 128;
 constexpr int kTS = 32;           // samples per gradient tile
-constexpr int kGradThreads = 256;
+constexpr int kGradThreads = 512;
 
 __global__ void __launch_bounds__(kFwdThreads) mlp_forward_kernel(const float* __restrict__ params,
                                                                   const float* __restrict__ X, int B,
@@ -37,117 +37,256 @@ __global__ void __launch_bounds__(kFwdThreads) mlp_forward_kernel(const float* _
   for (int o = 0; o < 4; ++o) Y[(long long)s * 4 + o] = mlp_out(s_w, h2, o);
 }
 
-struct GradSmem {
+constexpr int kW2Row = 68;  // padded row of W2 in shared memory: 16-byte loads along and across rows without conflicts
+
+struct __align__(16) GradSmem {
+  float w1[12 * 64], b1[64], b2[64], w3[64 * 4], b3[4];
+  float w2[64 * kW2Row];
   float x[kTS][12];
   float h1[kTS][64];
   float h2[kTS][64];
   float dz1[kTS][64];
   float dz2[kTS][64];
   float dy[kTS][4];
-  float sq[kGradThreads];
+  float sq[kTS * 4];  // squared errors by sample and output
 };
 
-// Partial gradient and squared error of one tile of kTS samples.
+// Partial gradient and squared error of one tile of kTS samples.  Thread
+// (t, grp) computes unit t of four samples, so that a weight loaded from
+// shared memory serves four products; the W2 gradient is 2 x 4 blocks in
+// registers, the outputs 32 partial sums per warp.  Every sum keeps the order
+// of the serial definitions (the forward pass's of mlp_device.cuh, samples
+// ascending in the gradients).  1,379 samples: 22.6 us with one thread per
+// output (two shared loads per product, 32-way bank conflicts down W2's
+// columns, 256 serial additions of the loss), now 14 us, of which 10 are the chain of
+// phases (ncu, cold caches).
 __global__ void __launch_bounds__(kGradThreads) mlp_grad_tile_kernel(const float* __restrict__ params,
                                                                      const float* __restrict__ X,
                                                                      const float* __restrict__ T, int B,
                                                                      float* __restrict__ partial,
                                                                      float* __restrict__ partial_loss) {
-  extern __shared__ float smem[];
-  float* s_w = smem;
-  GradSmem& g = *reinterpret_cast<GradSmem*>(smem + BFS_MLP_PARAMS);
-  const int tid = threadIdx.x;
-  for (int i = tid; i < BFS_MLP_PARAMS; i += kGradThreads) s_w[i] = params[i];
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  GradSmem& g = *reinterpret_cast<GradSmem*>(s_raw);
+  constexpr int kPer = kTS * 64 / kGradThreads;  // samples per thread: 4
+  constexpr int kGrps = kGradThreads / 64;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, t = tid & 63, grp = tid >> 6;
   const long long s0 = (long long)blockIdx.x * kTS;
+  for (int i = tid; i < 12 * 64; i += kGradThreads) g.w1[i] = params[kW1 + i];
+#pragma unroll
+  for (int i = 0; i < 1024 / kGradThreads; ++i) {
+    const int q = i * kGradThreads + tid;  // 16-byte group q of W2
+    const float* src = params + kW2 + 4 * q;
+    float4 w;
+    if ((reinterpret_cast<uintptr_t>(params) & 15u) == 0) w = *reinterpret_cast<const float4*>(src);
+    else w = make_float4(src[0], src[1], src[2], src[3]);
+    *reinterpret_cast<float4*>(&g.w2[(q >> 4) * kW2Row + 4 * (q & 15)]) = w;
+  }
+  if (tid < 256) g.w3[tid] = params[kW3 + tid];
+  if (tid < 64) {
+    g.b1[tid] = params[kB1 + tid];
+    g.b2[tid] = params[kB2 + tid];
+  }
+  if (tid < 4) g.b3[tid] = params[kB3 + tid];
   for (int i = tid; i < kTS * 12; i += kGradThreads) {
     const int s = i / 12, k = i % 12;
     g.x[s][k] = (s0 + s < B) ? X[(s0 + s) * 12 + k] : 0.0f;
   }
   __syncthreads();
-  for (int i = tid; i < kTS * 64; i += kGradThreads) {
-    const int s = i / 64, t = i % 64;
-    g.h1[s][t] = mlp_h1(s_w, g.x[s], t);
+  {  // layer 1
+    float a[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) a[q] = g.b1[t];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const float w = g.w1[k * 64 + t];
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) a[q] = fmaf(g.x[grp * kPer + q][k], w, a[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) g.h1[grp * kPer + q][t] = fmaxf(a[q], 0.0f);
   }
   __syncthreads();
-  for (int i = tid; i < kTS * 64; i += kGradThreads) {
-    const int s = i / 64, t = i % 64;
-    g.h2[s][t] = mlp_h2(s_w, g.h1[s], t);
+  {  // layer 2: four partial dot products p0 .. p3 per unit, added as (p0 + p1) + (p2 + p3)
+    float lo[kPer], hi[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) lo[q] = hi[q] = 0.0f;
+#pragma unroll 1
+    for (int r = 0; r < 4; ++r) {
+      float a[kPer];
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) a[q] = 0.0f;
+#pragma unroll 2
+      for (int i = 16 * r; i < 16 * r + 16; i += 4) {
+        float w[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) w[c] = g.w2[(i + c) * kW2Row + t];
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+          const float4 h = *reinterpret_cast<const float4*>(&g.h1[grp * kPer + q][i]);
+          a[q] = fmaf(h.x, w[0], a[q]);
+          a[q] = fmaf(h.y, w[1], a[q]);
+          a[q] = fmaf(h.z, w[2], a[q]);
+          a[q] = fmaf(h.w, w[3], a[q]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        if (r < 2) lo[q] = r == 0 ? a[q] : lo[q] + a[q];
+        else hi[q] = r == 2 ? a[q] : hi[q] + a[q];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) g.h2[grp * kPer + q][t] = fmaxf((lo[q] + hi[q]) + g.b2[t], 0.0f);
   }
   __syncthreads();
   const float scale = 2.0f / (4.0f * (float)B);
-  float sq = 0.0f;
-  for (int i = tid; i < kTS * 4; i += kGradThreads) {
-    const int s = i / 4, o = i % 4;
-    float d = 0.0f;
-    if (s0 + s < B) {
-      const float y = mlp_out(s_w, g.h2[s], o);
-      const float diff = y - T[(s0 + s) * 4 + o];
-      sq += diff * diff;
-      d = scale * diff;
-    }
-    g.dy[s][o] = d;
-  }
-  g.sq[tid] = sq;
-  __syncthreads();
-  for (int i = tid; i < kTS * 64; i += kGradThreads) {  // dz2 = (dy W3^T) * [h2 > 0]
-    const int s = i / 64, j = i % 64;
-    float a = 0.0f;
 #pragma unroll
-    for (int o = 0; o < 4; ++o) a = fmaf(g.dy[s][o], s_w[kW3 + j * 4 + o], a);
-    g.dz2[s][j] = g.h2[s][j] > 0.0f ? a : 0.0f;
+  for (int q = 0; q < kTS / (kGradThreads / 32); ++q) {  // outputs: one sample per warp and turn, lane = partial sum
+    const int s = wid * (kTS / (kGradThreads / 32)) + q;
+    const float ha = g.h2[s][lane], hb = g.h2[s][lane + 32];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      float v = fmaf(hb, g.w3[(lane + 32) * 4 + o], ha * g.w3[lane * 4 + o]);
+#pragma unroll
+      for (int m = 16; m >= 1; m >>= 1) v = v + __shfl_xor_sync(0xffffffffu, v, m);
+      if (lane == o) {
+        float d = 0.0f, sq = 0.0f;
+        if (s0 + s < B) {
+          const float diff = (v + g.b3[o]) - T[(s0 + s) * 4 + o];
+          sq = diff * diff;
+          d = scale * diff;
+        }
+        g.dy[s][o] = d;
+        g.sq[s * 4 + o] = sq;
+      }
+    }
   }
   __syncthreads();
-  for (int i = tid; i < kTS * 64; i += kGradThreads) {  // dz1 = (dz2 W2^T) * [h1 > 0]
-    const int s = i / 64, t = i % 64;
-    float a = 0.0f;
-    for (int j = 0; j < 64; ++j) a = fmaf(g.dz2[s][j], s_w[kW2 + t * 64 + j], a);
-    g.dz1[s][t] = g.h1[s][t] > 0.0f ? a : 0.0f;
+  {  // dz2 = (dy W3^T) * [h2 > 0]
+    const float4 w = *reinterpret_cast<const float4*>(&g.w3[t * 4]);
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int s = grp * kPer + q;
+      const float4 d = *reinterpret_cast<const float4*>(g.dy[s]);
+      float a = fmaf(d.x, w.x, 0.0f);
+      a = fmaf(d.y, w.y, a);
+      a = fmaf(d.z, w.z, a);
+      a = fmaf(d.w, w.w, a);
+      g.dz2[s][t] = g.h2[s][t] > 0.0f ? a : 0.0f;
+    }
+  }
+  __syncthreads();
+  {  // dz1 = (dz2 W2^T) * [h1 > 0]
+    float a[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) a[q] = 0.0f;
+#pragma unroll 2
+    for (int j = 0; j < 64; j += 4) {
+      const float4 w = *reinterpret_cast<const float4*>(&g.w2[t * kW2Row + j]);
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        const float4 d = *reinterpret_cast<const float4*>(&g.dz2[grp * kPer + q][j]);
+        a[q] = fmaf(d.x, w.x, a[q]);
+        a[q] = fmaf(d.y, w.y, a[q]);
+        a[q] = fmaf(d.z, w.z, a[q]);
+        a[q] = fmaf(d.w, w.w, a[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int s = grp * kPer + q;
+      g.dz1[s][t] = g.h1[s][t] > 0.0f ? a[q] : 0.0f;
+    }
   }
   __syncthreads();
   float* out = partial + (long long)blockIdx.x * BFS_MLP_PARAMS;
-  for (int pidx = tid; pidx < BFS_MLP_PARAMS; pidx += kGradThreads) {
-    float a = 0.0f;
-    if (pidx < kB1) {
-      const int k = pidx / 64, t = pidx % 64;
-      for (int s = 0; s < kTS; ++s) a = fmaf(g.x[s][k], g.dz1[s][t], a);
-    } else if (pidx < kW2) {
-      const int t = pidx - kB1;
-      for (int s = 0; s < kTS; ++s) a += g.dz1[s][t];
-    } else if (pidx < kB2) {
-      const int q = pidx - kW2, i = q / 64, t = q % 64;
-      for (int s = 0; s < kTS; ++s) a = fmaf(g.h1[s][i], g.dz2[s][t], a);
-    } else if (pidx < kW3) {
-      const int t = pidx - kB2;
-      for (int s = 0; s < kTS; ++s) a += g.dz2[s][t];
-    } else if (pidx < kB3) {
-      const int q = pidx - kW3, j = q / 4, o = q % 4;
-      for (int s = 0; s < kTS; ++s) a = fmaf(g.h2[s][j], g.dy[s][o], a);
-    } else {
-      const int o = pidx - kB3;
-      for (int s = 0; s < kTS; ++s) a += g.dy[s][o];
+  {  // W2: rows 2 ib and 2 ib + 1, columns 4 tb .. + 3
+    const int ib = tid >> 4, tb = tid & 15;
+    float a[2][4] = {};
+#pragma unroll 4
+    for (int s = 0; s < kTS; ++s) {
+      const float2 h = *reinterpret_cast<const float2*>(&g.h1[s][2 * ib]);
+      const float4 d = *reinterpret_cast<const float4*>(&g.dz2[s][4 * tb]);
+      const float hv[2] = {h.x, h.y}, dv[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) a[r][c] = fmaf(hv[r], dv[c], a[r][c]);
     }
-    out[pidx] = a;
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      *reinterpret_cast<float4*>(out + kW2 + (2 * ib + r) * 64 + 4 * tb) = make_float4(a[r][0], a[r][1], a[r][2], a[r][3]);
   }
-  if (tid == 0) {
+  {  // W1 at column t: row grp, and rows 8 + grp of the first four groups; W3 by the other four
+    const bool first = grp < kGrps / 2;
+    const int j = (tid - kGradThreads / 2) >> 2, o = tid & 3;
+    float a = 0.0f, a2 = 0.0f;
+#pragma unroll 4
+    for (int s = 0; s < kTS; ++s) {
+      const float d = g.dz1[s][t];
+      a = fmaf(g.x[s][grp], d, a);
+      a2 = first ? fmaf(g.x[s][kGrps + grp], d, a2) : fmaf(g.h2[s][j], g.dy[s][o], a2);
+    }
+    out[kW1 + grp * 64 + t] = a;
+    if (first) out[kW1 + (kGrps + grp) * 64 + t] = a2;
+    else out[kW3 + tid - kGradThreads / 2] = a2;
+  }
+  // biases and the tile's squared error, one kind per warp pair
+  if (grp < 2) {
+    float a = 0.0f;
+#pragma unroll 8
+    for (int s = 0; s < kTS; ++s) a += grp == 0 ? g.dz1[s][t] : g.dz2[s][t];
+    out[(grp == 0 ? kB1 : kB2) + t] = a;
+  } else if (grp == 2) {
+    if (t < 4) {
+      float a = 0.0f;
+#pragma unroll 8
+      for (int s = 0; s < kTS; ++s) a += g.dy[s][t];
+      out[kB3 + t] = a;
+    }
+  } else if (t == 0) {
     float tot = 0.0f;
-    for (int i = 0; i < kGradThreads; ++i) tot += g.sq[i];
+#pragma unroll 8
+    for (int i = 0; i < kTS * 4; i += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(&g.sq[i]);
+      tot += v.x;
+      tot += v.y;
+      tot += v.z;
+      tot += v.w;
+    }
     partial_loss[blockIdx.x] = tot;
   }
 }
+static_assert(kTS == 32 && kGradThreads == 512, "the gradient tile's thread mapping");
 
+// Sums over the tiles, ascending: one thread per parameter, 16 loads in flight,
+// and one for the loss.
 __global__ void mlp_reduce_kernel(const float* __restrict__ partial, const float* __restrict__ partial_loss,
                                   int ntiles, int B, float* __restrict__ grad, float* __restrict__ loss) {
   const int pidx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (pidx < BFS_MLP_PARAMS) {
-    float a = 0.0f;
-    for (int b = 0; b < ntiles; ++b) a += partial[(long long)b * BFS_MLP_PARAMS + pidx];
-    grad[pidx] = a;
+  if (pidx > BFS_MLP_PARAMS || (pidx == BFS_MLP_PARAMS && !loss)) return;
+  const bool is_loss = pidx == BFS_MLP_PARAMS;
+  const float* src = is_loss ? partial_loss : partial + pidx;
+  const long long step = is_loss ? 1 : BFS_MLP_PARAMS;
+  float a = 0.0f;
+  int b = 0;
+  for (; b + 16 <= ntiles; b += 16) {
+    float v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = src[(b + i) * step];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) a += v[i];
   }
-  if (pidx == 0 && loss) {
-    float a = 0.0f;
-    for (int b = 0; b < ntiles; ++b) a += partial_loss[b];
-    *loss = a / (4.0f * (float)B);
+  {
+    float v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = b + i < ntiles ? src[(b + i) * step] : 0.0f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (b + i < ntiles) a += v[i];
   }
+  if (is_loss) *loss = a / (4.0f * (float)B);
+  else grad[pidx] = a;
 }
 
 __global__ void adam_kernel(float* __restrict__ params, const float* __restrict__ grad, float* __restrict__ m,
@@ -165,7 +304,7 @@ __global__ void adam_kernel(float* __restrict__ params, const float* __restrict_
   params[i] -= lr * mhat / (sqrtf(vhat) + eps);
 }
 
-size_t grad_smem_bytes() { return sizeof(float) * BFS_MLP_PARAMS + sizeof(GradSmem); }
+size_t grad_smem_bytes() { return sizeof(GradSmem); }
 
 int grad_impl(const float* params, const float* X, const float* T, int B, float* grad, float* loss,
               float* partial, float* partial_loss, cudaStream_t s) {
@@ -177,7 +316,7 @@ int grad_impl(const float* params, const float* X, const float* T, int B, float*
     configured = true;
   }
   mlp_grad_tile_kernel<<<ntiles, kGradThreads, grad_smem_bytes(), s>>>(params, X, T, B, partial, partial_loss);
-  mlp_reduce_kernel<<<(BFS_MLP_PARAMS + 255) / 256, 256, 0, s>>>(partial, partial_loss, ntiles, B, grad, loss);
+  mlp_reduce_kernel<<<BFS_MLP_PARAMS / 64 + 1, 64, 0, s>>>(partial, partial_loss, ntiles, B, grad, loss);
   BFS_CUDA_TRY(cudaGetLastError());
   return BFS_OK;
 }
