@@ -211,7 +211,7 @@ int exclusive_scan(const ScanInput& in, long long N, int64_t* out, cudaStream_t 
   if (tiles > 1) {
     if (int e = dev_alloc((void**)&sums, sizeof(int64_t) * tiles, "scan tile sums")) return e;
     if (int e = dev_alloc((void**)&sums_off, sizeof(int64_t) * tiles, "scan tile offsets")) {
-      cudaFree(sums);
+      dev_free(sums);
       return e;
     }
     scan_reduce_kernel<<<(unsigned)tiles, kScanThreads, 0, s>>>(in, N, sums);
@@ -219,8 +219,8 @@ int exclusive_scan(const ScanInput& in, long long N, int64_t* out, cudaStream_t 
     si.i64 = sums;
     long long t2 = 0;
     if (int e = exclusive_scan(si, tiles, sums_off, s, &t2)) {
-      cudaFree(sums);
-      cudaFree(sums_off);
+      dev_free(sums);
+      dev_free(sums_off);
       return e;
     }
   }
@@ -240,8 +240,8 @@ int exclusive_scan(const ScanInput& in, long long N, int64_t* out, cudaStream_t 
       if (err == cudaSuccess) err = cudaStreamSynchronize(s);
     }
   }
-  if (sums) cudaFree(sums);
-  if (sums_off) cudaFree(sums_off);
+  if (sums) dev_free(sums);
+  if (sums_off) dev_free(sums_off);
   if (err != cudaSuccess) return cuda_fail(err, "exclusive scan");
   *total = last_out + last_in;
   return BFS_OK;
@@ -522,9 +522,9 @@ int build_csr_from_edges(const int32_t* d_src, const int32_t* d_dst, int64_t m, 
   int32_t* adj = nullptr;
   BuildReport rep{};
   auto give_up = [&](int rc) {
-    if (block) cudaFree(block);
-    if (off) cudaFree(off);
-    if (adj) cudaFree(adj);
+    if (block) dev_free(block);
+    if (off) dev_free(off);
+    if (adj) dev_free(adj);
     return rc;
   };
   if (int e = dev_alloc((void**)&off, sizeof(int64_t) * ((size_t)n + 1), "CSR offsets")) return give_up(e);
@@ -565,7 +565,7 @@ int build_csr_from_edges(const int32_t* d_src, const int32_t* d_dst, int64_t m, 
   }
   cudaError_t err = cudaStreamSynchronize(s);
   if (err != cudaSuccess) return give_up(cuda_fail(err, "CSR construction"));
-  if (block) cudaFree(block);
+  if (block) dev_free(block);
   *d_off_out = off;
   *d_adj_out = adj;
   *nnz_out = (int64_t)rep.nnz;
@@ -584,10 +584,10 @@ int build_row_tables(const int64_t* d_off, const int32_t* d_adj, int32_t n, int6
   t.rank = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(t.dead) + word_bytes);
   BuildReport rep{};
   auto give_up = [&](int rc) {
-    if (scratch) cudaFree(scratch);
-    if (t.probe) cudaFree(t.probe);
-    if (t.big) cudaFree(t.big);
-    cudaFree(t.dead);
+    if (scratch) dev_free(scratch);
+    if (t.probe) dev_free(t.probe);
+    if (t.big) dev_free(t.big);
+    dev_free(t.dead);
     return rc;
   };
   const size_t bytes = 256 + sizeof(uint64_t) * (size_t)tiles;
@@ -613,7 +613,7 @@ int build_row_tables(const int64_t* d_off, const int32_t* d_adj, int32_t n, int6
   err = cudaGetLastError();
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);
   if (err != cudaSuccess) return give_up(cuda_fail(err, "row tables"));
-  cudaFree(scratch);
+  dev_free(scratch);
   *out = t;
   return BFS_OK;
 }
@@ -636,16 +636,16 @@ int build_transpose(const int64_t* d_off, const int32_t* d_adj, int32_t n, int64
   expand_rows_kernel<<<di.sm_count * 8, 256, 0, s>>>(d_off, n, nnz, src);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) {
-    cudaFree(src);
+    dev_free(src);
     return cuda_fail(err, "arc tails");
   }
   int64_t tnnz = 0;
   const int rc = build_csr_from_edges(src, d_adj, nnz, n, 2, s, d_toff, d_tadj, &tnnz);
-  cudaFree(src);
+  dev_free(src);
   if (rc) return rc;
   if (tnnz != nnz) {
-    cudaFree(*d_toff);
-    cudaFree(*d_tadj);
+    dev_free(*d_toff);
+    dev_free(*d_tadj);
     return fail(BFS_ERR_INVALID_GRAPH, "transpose: the CSR has repeated arcs or self-loops");
   }
   return BFS_OK;
@@ -681,7 +681,7 @@ int validate_csr(const int64_t* d_off, const int32_t* d_adj, int32_t n, int64_t 
   }
   if (err == cudaSuccess) err = cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-  cudaFree(d_bad);
+  dev_free(d_bad);
   if (err != cudaSuccess) return cuda_fail(err, "CSR validation");
   *ok = bad == 0;
   return BFS_OK;

@@ -187,7 +187,7 @@ int ensure_half(bfs_graph* g, cudaStream_t s, HalfSet* out) {
   int rc = dev_alloc((void**)&cnt, sizeof(uint32_t) * std::max(1, n), "half-row counts");
   if (!rc) rc = dev_alloc((void**)&hoff, sizeof(int64_t) * ((size_t)n + 1), "half offsets");
   if (rc) {
-    if (cnt) cudaFree(cnt);
+    if (cnt) dev_free(cnt);
     return rc;
   }
   half_count_kernel<<<blocks_for(n), kThreads, 0, s>>>(g->d_off, g->d_adj, n, cnt);
@@ -196,7 +196,7 @@ int ensure_half(bfs_graph* g, cudaStream_t s, HalfSet* out) {
   if (err == cudaSuccess) rc = exclusive_scan_u32(cnt, n, hoff, s, &total);
   if (err == cudaSuccess && !rc) err = cudaMemcpyAsync(hoff + n, &total, sizeof(int64_t), cudaMemcpyHostToDevice, s);
   if (err == cudaSuccess && !rc) err = cudaStreamSynchronize(s);
-  cudaFree(cnt);
+  dev_free(cnt);
   if (!rc && err == cudaSuccess) rc = dev_alloc((void**)&hadj, sizeof(int32_t) * std::max(1ll, total), "half adjacency");
   if (!rc && err == cudaSuccess) {
     half_copy_kernel<<<blocks_for((long long)n * 32), kThreads, 0, s>>>(g->d_off, g->d_adj, n, hoff, hadj);
@@ -204,8 +204,8 @@ int ensure_half(bfs_graph* g, cudaStream_t s, HalfSet* out) {
     if (err == cudaSuccess) err = cudaStreamSynchronize(s);
   }
   if (rc || err != cudaSuccess) {
-    cudaFree(hoff);
-    if (hadj) cudaFree(hadj);
+    dev_free(hoff);
+    if (hadj) dev_free(hadj);
     return rc ? rc : cuda_fail(err, "half storage");
   }
   HalfSet h;
@@ -224,8 +224,8 @@ void free_half(const bfs_graph* g) {
   std::lock_guard<std::mutex> lk(g_half_mu);
   auto it = g_half.find(g);
   if (it == g_half.end()) return;
-  cudaFree(it->second.off);
-  cudaFree(it->second.adj);
+  dev_free(it->second.off);
+  dev_free(it->second.adj);
   g_half.erase(it);
 }
 
@@ -266,8 +266,8 @@ int bfs_run_half(bfs_graph* g, int32_t source, int32_t* parent_out, int32_t* lev
   int rc = dev_alloc((void**)&bits, sizeof(uint32_t) * 4 * nwords, "half BFS bitmaps");
   if (!rc) rc = dev_alloc((void**)&count, sizeof(unsigned long long), "half BFS count");
   auto cleanup = [&]() {
-    if (bits) cudaFree(bits);
-    if (count) cudaFree(count);
+    if (bits) dev_free(bits);
+    if (count) dev_free(count);
   };
   if (rc) return cleanup(), rc;
   uint32_t *vis = bits, *cur = bits + nwords, *na = bits + 2 * nwords, *nb = bits + 3 * nwords;

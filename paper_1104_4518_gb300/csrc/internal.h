@@ -27,8 +27,12 @@ int cuda_fail(cudaError_t e, const char* what);
     if (_e != cudaSuccess) return bfsint::cuda_fail(_e, #expr); \
   } while (0)
 
-// Device allocation that reports OOM as BFS_ERR_OOM.
+// Device allocation that reports OOM as BFS_ERR_OOM; the contents are unspecified.
 int dev_alloc(void** p, size_t bytes, const char* what);
+// Waits for the device, then releases a block (null: nothing) to the library's cache or to the driver.
+void dev_free(void* p);
+// Gives the cached blocks that nothing has asked for lately back to the driver.
+void trim_device_cache();
 
 // ---------------- device properties ----------------
 struct DeviceInfo {

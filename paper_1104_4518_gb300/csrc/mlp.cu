@@ -338,7 +338,7 @@ const float* learned_params_device() {
     float* p = nullptr;
     if (cudaMalloc(&p, sizeof(float) * BFS_MLP_PARAMS) != cudaSuccess) return nullptr;
     if (cudaMemcpy(p, g_sel_host.data(), sizeof(float) * BFS_MLP_PARAMS, cudaMemcpyHostToDevice) != cudaSuccess) {
-      cudaFree(p);
+      dev_free(p);
       return nullptr;
     }
     g_sel_dev[dev] = p;
@@ -387,7 +387,7 @@ int bfs_mlp_loss_grad(const float* params, const float* X, const float* T, int32
     return e;
   int rc = grad_impl(params, X, T, B, grad, loss, partial, partial + (size_t)ntiles * BFS_MLP_PARAMS, s);
   cudaError_t err = cudaStreamSynchronize(s);
-  cudaFree(partial);
+  dev_free(partial);
   if (rc) return rc;
   if (err != cudaSuccess) return cuda_fail(err, "bfs_mlp_loss_grad");
   return BFS_OK;
@@ -426,7 +426,7 @@ int bfs_selector_train(float* params, const float* X, const float* T, int32_t B,
     if (rc == BFS_OK) rc = bfs_mlp_adam(params, grad, m, v, t, lr, 0.9f, 0.999f, 1e-8f, stream);
   }
   err = cudaStreamSynchronize(s);
-  cudaFree(buf);
+  dev_free(buf);
   if (rc) return rc;
   if (err != cudaSuccess) return cuda_fail(err, "bfs_selector_train");
   return BFS_OK;
@@ -435,7 +435,7 @@ int bfs_selector_train(float* params, const float* X, const float* T, int32_t B,
 int bfs_selector_set_params(const float* params) {
   std::lock_guard<std::mutex> lk(g_sel_mu);
   for (float* p : g_sel_dev)
-    if (p) cudaFree(p);
+    if (p) dev_free(p);
   g_sel_dev.clear();
   if (!params) {
     g_sel_host.clear();

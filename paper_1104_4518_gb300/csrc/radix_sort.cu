@@ -235,7 +235,7 @@ int radix_sort_u64(uint64_t* keys, uint64_t* alt, long long N, int lo_bit, int h
   }
   if (err == cudaSuccess && !rc) err = cudaMemcpyAsync(st, status, sizeof(st), cudaMemcpyDeviceToHost, s);
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-  cudaFree(block);
+  dev_free(block);
   if (rc) return rc;
   if (err != cudaSuccess) return cuda_fail(err, "radix sort");
   if (st[0]) return fail(st[0], "radix sort: " + device_status_message(st));

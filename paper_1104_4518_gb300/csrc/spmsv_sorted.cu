@@ -146,7 +146,7 @@ int spmsv_sorted(const bfs_graph* g, const int32_t* f, long long nf, const uint3
   int64_t* pos = nullptr;
   auto cleanup = [&]() {
     for (void* p : {(void*)d_ctr, (void*)d_bad, (void*)keys, (void*)alt, (void*)flag, (void*)pos})
-      if (p) cudaFree(p);
+      if (p) dev_free(p);
   };
   int rc = dev_alloc((void**)&d_ctr, 2 * sizeof(unsigned long long), "SpMSV counters");
   if (!rc) rc = dev_alloc((void**)&d_bad, 4 * sizeof(long long), "SpMSV flags");
@@ -234,7 +234,7 @@ int bfs_run_sorted(bfs_graph* g, int32_t source, int32_t* parent_out, int32_t* l
   int32_t* tv = nullptr;  // values of t
   auto cleanup = [&]() {
     for (void* p : {(void*)visited, (void*)fa, (void*)fb, (void*)tv})
-      if (p) cudaFree(p);
+      if (p) dev_free(p);
   };
   int rc = dev_alloc((void**)&visited, sizeof(uint32_t) * nwords, "visited bitmap");
   if (!rc) rc = dev_alloc((void**)&fa, sizeof(int32_t) * n, "frontier");

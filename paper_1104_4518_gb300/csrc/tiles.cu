@@ -116,11 +116,11 @@ int ceil_log2(long long x) {
 
 void free_tiles(TileSet* t) {
   if (!t) return;
-  cudaFree(t->jc);
-  cudaFree(t->cp);
-  cudaFree(t->ir);
-  cudaFree(t->tdir_jc);
-  cudaFree(t->tdir_ir);
+  dev_free(t->jc);
+  dev_free(t->cp);
+  dev_free(t->ir);
+  dev_free(t->tdir_jc);
+  dev_free(t->tdir_ir);
   delete t;
 }
 
@@ -144,10 +144,10 @@ int build_tiles(const bfs_graph* g, int sm_count, int rb_bits, int cb_bits, cuda
   uint32_t* flags = nullptr;
   int64_t* colpos = nullptr;
   auto fail_clean = [&](int rc) {
-    cudaFree(keys);
-    cudaFree(alt);
-    cudaFree(flags);
-    cudaFree(colpos);
+    dev_free(keys);
+    dev_free(alt);
+    dev_free(flags);
+    dev_free(colpos);
     free_tiles(ts);
     return rc;
   };
@@ -175,7 +175,7 @@ int build_tiles(const bfs_graph* g, int sm_count, int rb_bits, int cb_bits, cuda
     }
     if (e0 == cudaSuccess) e0 = cudaMemcpyAsync(h_bad, d_bad, sizeof(h_bad), cudaMemcpyDeviceToHost, s);
     if (e0 == cudaSuccess) e0 = cudaStreamSynchronize(s);
-    cudaFree(d_bad);
+    dev_free(d_bad);
     if (e0 != cudaSuccess) return fail_clean(cuda_fail(e0, "tile keys"));
     if (h_bad[0])
       return fail_clean(fail(bfsdev::kBoundsCheck ? BFS_ERR_BOUNDS : BFS_ERR_INVALID_GRAPH,
@@ -184,9 +184,9 @@ int build_tiles(const bfs_graph* g, int sm_count, int rb_bits, int cb_bits, cuda
     uint64_t* sorted = nullptr;
     if ((rc = radix_sort_u64(keys, alt, N, 16, 32 + std::max(1, ceil_log2(T)), s, &sorted))) return fail_clean(rc);
     if (sorted == keys) {
-      cudaFree(alt);
+      dev_free(alt);
     } else {
-      cudaFree(keys);
+      dev_free(keys);
       keys = alt;
     }
     alt = nullptr;
@@ -203,9 +203,9 @@ int build_tiles(const bfs_graph* g, int sm_count, int rb_bits, int cb_bits, cuda
   }
   cudaError_t err = cudaGetLastError();
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-  cudaFree(keys);
-  cudaFree(flags);
-  cudaFree(colpos);
+  dev_free(keys);
+  dev_free(flags);
+  dev_free(colpos);
   keys = nullptr;
   flags = nullptr;
   colpos = nullptr;
