@@ -209,4 +209,20 @@ __device__ __forceinline__ void flush_claims_if_full(const P& p, int knext, Clai
   }
 }
 
+// Brings a level's counters to shared memory (thread 0, at the barrier before
+// the level).  Loaded by every warp of every CTA, the one line cost a level
+// 1.3 us of queueing at its L2 slice.
+struct FetchCtr {
+  const LevelCtr* src;
+  LevelCtr* dst;
+  __device__ void operator()() const {
+    constexpr int kParts = sizeof(LevelCtr) / 16;
+    int4 v[kParts];
+#pragma unroll
+    for (int i = 0; i < kParts; ++i) v[i] = __ldcg(reinterpret_cast<const int4*>(src) + i);
+#pragma unroll
+    for (int i = 0; i < kParts; ++i) reinterpret_cast<int4*>(dst)[i] = v[i];
+  }
+};
+
 }  // namespace bfsint

@@ -213,6 +213,7 @@ __device__ __forceinline__ void end_phase(const LoopParams& p, int knext, Acc& a
 }
 
 struct Smem {
+  LevelCtr ctr;  // counters of the level to expand, fetched by thread 0 at the barrier before it
   int owner;
   int cu;
   long long cb, ce;
@@ -227,11 +228,73 @@ struct Smem {
 // ---------------- top-down phase ----------------
 // Dynamic shared memory of the top-down and tiled phases: frontier rows of a
 // CTA with the prefix sums of their lengths.
+constexpr int kFlatRows = 4 * kBlock;  // frontier vertices of a level whose edges are dealt to the whole grid
 struct FlatSmem {
-  long long tb[kBlock];
-  int tu[kBlock];
-  int tpref[kBlock + 1];
+  long long tb[kFlatRows];
+  int tu[kFlatRows];
+  int tpref[kFlatRows + 1];
 };
+
+// The last of `rows` rows whose prefix sum is at most idx (a non-empty one when idx is below the total).
+__device__ __forceinline__ int flat_owner(const FlatSmem& fl, int rows, int idx) {
+  int lo = 0, hi = rows;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (fl.tpref[mid] <= idx) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// Top-down level of a small frontier (at most kFlatRows vertices, few enough
+// edges for the CTAs' claim buffers): every CTA takes in the whole frontier and
+// the prefix sums of its degrees, and edge i goes to thread i of the grid, so
+// that a level is one round of loads wherever its edges are.  By rows, the
+// first levels of an R-MAT traversal (2 to 100 vertices with hundreds to
+// thousands of edges each) ran on as many CTAs as they had rows or 1,024-edge
+// chunks, two visits deep: 22 us at scale 16 for 7 rows, 30 us at scale 22 for
+// 98.
+__device__ void flat_phase(const LoopParams& p, int k, unsigned count, Smem& sm, FlatSmem& fl, Acc& acc, unsigned G) {
+  const uint32_t* cur = p.bits[k % 3];
+  uint32_t* nxt = p.bits[(k + 1) % 3];
+  const int32_t* Q = p.queue[k % 3];
+  const int tid = threadIdx.x, per = ((int)count + kBlock - 1) / kBlock, rows = per * kBlock;
+  int u[4], deg[4], sum = 0;
+  long long b[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) u[r] = r < per && tid * per + r < (int)count ? Q[tid * per + r] : -1;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    b[r] = u[r] >= 0 ? __ldg(&p.off[u[r]]) : 0;
+    deg[r] = u[r] >= 0 ? (int)(__ldg(&p.off[u[r] + 1]) - b[r]) : 0;
+    sum += deg[r];
+  }
+  int at = 0;
+  const int total = block_exclusive_scan(sum, sm.warp_tmp, at);
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    if (r < per) {
+      fl.tu[tid * per + r] = u[r];
+      fl.tb[tid * per + r] = b[r];
+      fl.tpref[tid * per + r] = at;
+      at += deg[r];
+      if (u[r] >= 0 && (unsigned)(tid * per + r) % G == blockIdx.x) atomicOr(&p.vis[u[r] >> 5], 1u << (u[r] & 31));
+    }
+  }
+  __syncthreads();
+  int room = kQBuf / kBlock;  // steps that the CTA's claim buffer is sure to hold
+  for (int base = (int)blockIdx.x * kBlock; base < total; base += (int)G * kBlock) {
+    if (room-- == 0) {
+      flush_claims_if_full(p, k + 1, sm.cl, kBlock, kBigBuf / 2);
+      room = 0;
+    }
+    const int idx = base + tid;
+    if (idx < total) {
+      const int o = flat_owner(fl, rows, idx);
+      td_visit(p, cur, nxt, k, fl.tu[o], __ldg(&p.adj[fl.tb[o] + (idx - fl.tpref[o])]), acc, sm.cl);
+    }
+  }
+}
 
 __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned count, unsigned nchunks, Smem& sm,
                               FlatSmem& fl, Acc& acc, unsigned G) {
@@ -329,12 +392,7 @@ __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned 
       for (int base = 0; base < total; base += kBlock) {
         const int idx = base + tid;
         if (idx < total) {
-          int lo = 0, hi = kBlock;  // largest slot with tpref <= idx (and a non-empty row)
-          while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (fl.tpref[mid] <= idx) lo = mid;
-            else hi = mid;
-          }
+          const int lo = flat_owner(fl, kBlock, idx);
           const int ou = fl.tu[lo];
           td_visit(p, cur, nxt, k, ou, __ldg(&p.adj[fl.tb[lo] + (idx - fl.tpref[lo])]), acc, sm.cl);
         }
@@ -816,12 +874,7 @@ __device__ void tiled_phase(const LoopParams& p, int k, Smem& sm, FlatSmem& fl, 
         for (int base = 0; base < total; base += kBlock) {
           const int idx = base + tid;
           if (idx < total) {
-            int lo = 0, hi = kBlock;  // largest slot with tpref <= idx (a frontier column with rows)
-            while (hi - lo > 1) {
-              const int mid = (lo + hi) >> 1;
-              if (fl.tpref[mid] <= idx) lo = mid;
-              else hi = mid;
-            }
+            const int lo = flat_owner(fl, kBlock, idx);  // a frontier column with rows
             const int r = p.t_ir[fl.tb[lo] + (idx - fl.tpref[lo])];
             if (!((done[r >> 5] >> (r & 31)) & 1u)) {
               atomicMax(&p.parent[(rb << p.t_rb_bits) + r], (cb << p.t_cb_bits) + fl.tu[lo]);
@@ -902,8 +955,9 @@ __device__ __forceinline__ int heuristic_variant(const LoopParams& p, int prev_v
 }
 
 constexpr size_t kFlatBytes = (sizeof(FlatSmem) + 15) / 16 * 16;
-constexpr size_t kPhaseBytes = sizeof(PullSmem);  // the largest phase's area
-static_assert(kPhaseBytes >= kFlatBytes + sizeof(uint32_t) * 3 * kTileWordsMax, "the tiled phase fits the pull's area");
+// the largest phase's area, without and with the tiled phase
+constexpr size_t kPhaseBytes = std::max(sizeof(PullSmem), kFlatBytes);
+constexpr size_t kTiledBytes = std::max(kPhaseBytes, kFlatBytes + sizeof(uint32_t) * 3 * kTileWordsMax);
 
 // kTiles: the kernel can run the tiled phase.  Runs that cannot pick the tiled
 // variant launch the instance without it: on R-MAT scale 26 the tiled phase's
@@ -1004,7 +1058,7 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
       if (deg > p.chunk_deg) push_chunks(p, 0, s0, deg);
     }
   }
-  if (!bfsdev::grid_barrier(p.bar, nblocks, bar_target, p.spin_limit, p.status)) return;
+  if (!bfsdev::grid_barrier(p.bar, nblocks, bar_target, p.spin_limit, p.status, FetchCtr{&p.ctr[0], &sm.ctr})) return;
 
   if (!single) {  // seed level 0 with the sources (block 0)
     if (blockIdx.x == 0) {
@@ -1022,29 +1076,28 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
       if (tid == 0) p.ctr[0].count = (unsigned)p.nsources;
       end_phase(p, 0, acc, sm);
     }
-    if (!bfsdev::grid_barrier(p.bar, nblocks, bar_target, p.spin_limit, p.status)) return;
+    if (!bfsdev::grid_barrier(p.bar, nblocks, bar_target, p.spin_limit, p.status, FetchCtr{&p.ctr[0], &sm.ctr})) return;
   }
 
   // ---- level loop
   long long cum_count = 0, cum_edges = 0;
   int prev_variant = -1;
   unsigned prev_count = 0;
+  int clr_first = -1;
   uint64_t t_prev = 0;
   if (blockIdx.x == 0 && tid == 0) t_prev = bfsdev::global_timer_ns();
   int k = 0;
   Acc acc;
   for (;; ++k) {
     PHASE_TS(k, 0);
-    // one round of loads: the counters of f_k and the first entry of f_{k-1} to recycle
-    const LevelCtr* c = &p.ctr[k % kCtrRing];
-    const unsigned count = __ldcg(&c->count);
-    const unsigned nchunks = __ldcg(&c->chunks);
-    const long long edges = (long long)__ldcg(&c->edges);
-    const long long binv = (learned && tid < 3) ? (long long)__ldcg(&c->bins[tid]) : 0;
-    const unsigned long long big_rows = __ldcg(&c->bins[1]) | __ldcg(&c->bins[2]);
+    const LevelCtr& c = sm.ctr;  // (the next fetch comes after this level's work and a CTA barrier)
+    const unsigned count = c.count;
+    const unsigned nchunks = c.chunks;
+    const long long edges = (long long)c.edges;
+    const long long binv = (learned && tid < 3) ? (long long)c.bins[tid] : 0;
+    const bool big_rows = (c.bins[1] | c.bins[2]) != 0;
     const bool sparse_clr = k >= 1 && (long long)prev_count * 4 < p.nwords;
     const int32_t* PQ = p.queue[(k + 2) % 3];
-    const int clr0 = (sparse_clr && gtid < prev_count) ? PQ[gtid] : -1;
     if (count == 0) break;
     cum_count += count;
     cum_edges += edges;
@@ -1067,7 +1120,7 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
     if (k >= 1 && part) {
       uint32_t* clr = p.bits[(k + 2) % 3];
       if (sparse_clr) {
-        if (clr0 >= 0) clr[clr0 >> 5] = 0u;
+        if (clr_first >= 0) clr[clr_first >> 5] = 0u;
         for (long long i = gtid + pthreads; i < prev_count; i += pthreads) clr[PQ[i] >> 5] = 0u;
       } else {
         for (long long w = gtid; w < p.nwords; w += pthreads) clr[w] = 0u;
@@ -1089,7 +1142,7 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
       __syncthreads();
       variant = sm.choice;
     } else {
-      variant = heuristic_variant(p, prev_variant, count, prev_count, edges, unvisited_edges, big_rows == 0);
+      variant = heuristic_variant(p, prev_variant, count, prev_count, edges, unvisited_edges, !big_rows);
     }
     if (variant < 0 || variant >= BFS_NUM_VARIANTS) variant = BFS_VARIANT_TD_BINNED;
     if (variant == BFS_VARIANT_TILED && (!kTiles || p.t_jc == nullptr)) variant = BFS_VARIANT_PULL;  // the SpMV untiled
@@ -1097,13 +1150,21 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
     if (part) {
       if (variant == BFS_VARIANT_PULL) pull_phase(p, k, count, sm, s_pull, acc, G);
       else if (kTiles && variant == BFS_VARIANT_TILED) tiled_phase(p, k, sm, s_flat, s_tile, acc, G);
+      // the degree-binned variant deals a small frontier's edges out flat
+      else if (variant == BFS_VARIANT_TD_BINNED && count <= (unsigned)kFlatRows && edges <= 16ll * pthreads)
+        flat_phase(p, k, count, sm, s_flat, acc, G);
       else topdown_phase(p, k, variant, count, nchunks, sm, s_flat, acc, G);
       PHASE_TS(k, 3);
       end_phase(p, k + 1, acc, sm);
     }
     PHASE_TS(k, 4);
     PHASE_ARRIVAL(k);
-    if (!bfsdev::grid_barrier_partial(p.bar, G, bar_target, p.spin_limit, p.status)) return;
+    // the first entry of f_k that this thread clears in the next level: in flight across the barrier
+    clr_first = gtid < count ? p.queue[k % 3][gtid] : -1;
+    const int4 level_bins = p.want_stats && blockIdx.x == 0 && tid == 0
+                                ? make_int4((int)c.bins[0], (int)c.bins[1], (int)c.bins[2], 0)
+                                : make_int4(0, 0, 0, 0);
+    if (!bfsdev::grid_barrier_partial(p.bar, G, bar_target, p.spin_limit, p.status, FetchCtr{&p.ctr[(k + 1) % kCtrRing], &sm.ctr})) return;
     PHASE_TS(k, 6);
 
     if (p.want_stats && blockIdx.x == 0 && tid == 0 && k < kMaxStatLevels) {
@@ -1111,9 +1172,9 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
       bfs_level_stat st;
       st.frontier_count = count;
       st.frontier_edges = edges;
-      st.bin_count[0] = (int64_t)__ldcg(&c->bins[0]);  // level k's slot is recycled only in phase k + 4
-      st.bin_count[1] = (int64_t)__ldcg(&c->bins[1]);
-      st.bin_count[2] = (int64_t)__ldcg(&c->bins[2]);
+      st.bin_count[0] = level_bins.x;
+      st.bin_count[1] = level_bins.y;
+      st.bin_count[2] = level_bins.z;
       st.unvisited_count = unvisited;
       st.unvisited_edges = unvisited_edges;
       st.time_ns = (int64_t)(t - t_prev);
@@ -1236,7 +1297,9 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
   // top-down's atomics on the parent array get dearer once 4 bytes per vertex
   // no longer fit in L2, so the switch to pull comes earlier on large graphs
   p.alpha = (float)(t.alpha * (1.0 + 4.0 * (double)g->n / (double)(di.l2_bytes > 0 ? di.l2_bytes : (1ll << 27))));
-  p.beta = t.beta;
+  // a pull level costs about one microsecond per 45,000 bitmap words plus its live rows, a top-down one 1 us per
+  // 16,000 edges: they meet near n / 90 vertices (R-MAT scale 26, 1.6 M vertices: pull 48 us, top-down 112 us)
+  p.beta = 4.0f * t.beta;
   p.parts = g->parts;
   p.part_base = g->d_part_base;
   p.part_out = r.part_out;
@@ -1256,7 +1319,7 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
   // the pull / tiled phase's area follows the network's parameters in dynamic shared memory
   const size_t mlp_bytes = p.mlp ? (sizeof(float) * BFS_MLP_PARAMS + 15) / 16 * 16 : 0;
   p.phase_smem_off = (int32_t)mlp_bytes;
-  const size_t dyn_smem = mlp_bytes + kPhaseBytes;
+  const size_t dyn_smem = mlp_bytes + (p.t_jc ? kTiledBytes : kPhaseBytes);
   const void* kernel = p.t_jc ? (const void*)level_loop_kernel<true> : (const void*)level_loop_kernel<false>;
   {  // the attribute belongs to the current device: set it once per device
     static std::mutex mu;
@@ -1264,7 +1327,7 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
     std::lock_guard<std::mutex> lk(mu);
     if (di.device < 0 || di.device >= 64) return fail(BFS_ERR_UNSUPPORTED, "device ordinal out of range");
     if (!configured[di.device]) {
-      const int max_dyn = (int)((sizeof(float) * BFS_MLP_PARAMS + 15) / 16 * 16 + kPhaseBytes);
+      const int max_dyn = (int)((sizeof(float) * BFS_MLP_PARAMS + 15) / 16 * 16 + kTiledBytes);
       BFS_CUDA_TRY(cudaFuncSetAttribute((const void*)level_loop_kernel<false>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn));
       BFS_CUDA_TRY(cudaFuncSetAttribute((const void*)level_loop_kernel<true>,
