@@ -223,7 +223,7 @@ __device__ __forceinline__ Bits resolve_row(const BatchParams& p, const Word* F,
 // has deg entries ending at e and `need` roots to find.  Adds the roots found
 // to `found` and takes them from `need`.  list: 32 ints of the warp.
 template <typename Word, int kSlots, int kLoads>
-__device__ __forceinline__ void resolve_packed(const BatchParams& p, const Word* F, int v0, int skip, int deg,
+__device__ __forceinline__ void resolve_packed(const BatchParams& p, const Word* F, int v, int skip, int deg,
                                                long long e, Bits& need, Bits& found, int lane, int* list) {
   constexpr int kRows = 32 / kSlots;  // rows per load
   const bool open = need != 0 && deg > skip;
@@ -262,7 +262,8 @@ __device__ __forceinline__ void resolve_packed(const BatchParams& p, const Word*
         const unsigned seg = (kSlots == 32 ? kFull : (1u << kSlots) - 1u) << (j * kSlots);
         if (!(any & seg)) continue;
         const int o = __shfl_sync(kFull, own[q], j * kSlots);
-        const Bits fr = store_parents<Word, false>(p, v0 + o, m0 & seg, m1 & seg, u[q], lane);
+        const Bits fr =
+            store_parents<Word, false>(p, __shfl_sync(kFull, v, o), m0 & seg, m1 & seg, u[q], lane);
         if (lane == o) got = fr;
       }
     }
@@ -272,22 +273,22 @@ __device__ __forceinline__ void resolve_packed(const BatchParams& p, const Word*
   __syncwarp();  // the list is free again
 }
 
-// Resolves 32 vertices v0 .. v0 + 31 against frontier F: lane l's row has deg
+// Resolves 32 vertices against frontier F: lane l's vertex v has a row of deg
 // entries ending at e and `need` roots to find.  First the top kTop entries of
 // every row, 32 / kTop rows per load: a dense level ends most rows there, and
 // short rows fill the lanes that a row each would leave idle; then the next
-// kNext entries, four rows in flight; then row by row.  Returns the lane's bits found.
+// kNext entries, a row per load; then row by row.  Returns the lane's bits found.
 template <typename Word>
-__device__ __forceinline__ Bits resolve_group(const BatchParams& p, const Word* F, int v0, int deg, long long e,
+__device__ __forceinline__ Bits resolve_group(const BatchParams& p, const Word* F, int v, int deg, long long e,
                                               Bits need, int lane, int* list) {
   Bits found = 0;
-  resolve_packed<Word, kTop, kTopLoads>(p, F, v0, 0, deg, e, need, found, lane, list);
-  resolve_packed<Word, kNext, kNextLoads>(p, F, v0, kTop, deg, e, need, found, lane, list);
+  resolve_packed<Word, kTop, kTopLoads>(p, F, v, 0, deg, e, need, found, lane, list);
+  resolve_packed<Word, kNext, kNextLoads>(p, F, v, kTop, deg, e, need, found, lane, list);
   for (unsigned lm = __ballot_sync(kFull, need != 0 && deg > kTop + kNext); lm; lm &= lm - 1u) {
     const int l = __ffs(lm) - 1;
     const long long el = __shfl_sync(kFull, e, l);
-    const Bits fr = resolve_row<Word, false>(p, F, v0 + l, el - __shfl_sync(kFull, deg, l), el - kTop - kNext,
-                                             __shfl_sync(kFull, need, l), lane);
+    const Bits fr = resolve_row<Word, false>(p, F, __shfl_sync(kFull, v, l), el - __shfl_sync(kFull, deg, l),
+                                             el - kTop - kNext, __shfl_sync(kFull, need, l), lane);
     if (lane == l) found |= fr;
   }
   return found;
@@ -342,12 +343,34 @@ __device__ __forceinline__ void pull_chunk(const BatchParams& p, const Word* Fc,
   warp_enqueue(p, knext, wq, nbuf, claimed, v, lane, false);
 }
 
+// The rows of a frontier of at most one CTA's threads, with the prefix sums of
+// their lengths.  (Their starts and words are read again at each visit, from L1:
+// 8 KB more shared memory per CTA takes enough L1 to slow the pull levels by 3 %.)
+struct FlatRows {
+  int u[kBBlock];
+  int pref[kBBlock];
+};
+
+// Vertices of a warp that have roots to find, waiting to be 32.
+template <typename Word>
+struct Pending {
+  int v[64];
+  Word need[64];
+};
+
 template <typename Word>
 __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
   Word* F[3] = {static_cast<Word*>(p.F[0]), static_cast<Word*>(p.F[1]), static_cast<Word*>(p.F[2])};
   Word* V = static_cast<Word*>(p.V);
   __shared__ Claims cl;
-  __shared__ int row_list[kBWarps][32];  // pull: the lanes of a word with roots to find
+  __shared__ LevelCtr s_ctr;             // counters of the level to expand, fetched by thread 0 at the barrier before it
+  __shared__ int row_list[kBWarps][32];  // pull: the lanes whose rows a packed step examines
+  __shared__ union {
+    FlatRows flat;                 // top-down: the rows of a small frontier
+    Pending<Word> pend[kBWarps];   // pull
+  } s_rows;
+  FlatRows& flat = s_rows.flat;
+  __shared__ int scan_warp[kBWarps + 1];
   const int tid = threadIdx.x, lane = tid & 31;
   unsigned long long bar_target = 0;
   if (tid == 0) {
@@ -395,15 +418,16 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
       if (deg > kChunkEdges) push_chunks(p, 0, s, deg);
     }
   }
-  if (!bfsdev::grid_barrier(p.bar, nblocks, bar_target, p.spin_limit, p.status)) return;
+  if (!bfsdev::grid_barrier(p.bar, nblocks, bar_target, p.spin_limit, p.status, FetchCtr{&p.ctr[0], &s_ctr})) return;
 
   int k = 0;
+  unsigned prev_count = 0;
   uint64_t t_prev = 0;
   if (p.stats && blockIdx.x == 0 && tid == 0) t_prev = bfsdev::global_timer_ns();
   for (;; ++k) {
-    const unsigned count = __ldcg(&p.ctr[k % kCtrRing].count);
+    const unsigned count = s_ctr.count;  // (the next fetch comes after this level's work and a CTA barrier)
     if (count == 0) break;
-    const unsigned nchunks = __ldcg(&p.ctr[k % kCtrRing].chunks);
+    const unsigned nchunks = s_ctr.chunks;
     const Word* Fc = F[k % 3];
     Word* Fn = F[(k + 1) % 3];
     const int32_t* Q = p.queue[k % 3];
@@ -412,7 +436,7 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
       reinterpret_cast<unsigned long long*>(&p.ctr[(k + 4) % kCtrRing])[tid] = 0ull;
     if (k >= 1) {  // clear F_{k-1} for reuse as F_{k+2}
       Word* clr = F[(k + 2) % 3];
-      const unsigned pc = __ldcg(&p.ctr[(k + kCtrRing - 1) % kCtrRing].count);
+      const unsigned pc = prev_count;
       if ((long long)pc * 8 < p.n) {
         const int32_t* PQ = p.queue[(k + 2) % 3];
         for (long long i = gtid; i < pc; i += gthreads) clr[PQ[i]] = 0;
@@ -429,7 +453,51 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
 
     const bool topdown = (long long)count <= p.td_limit;
     const int wid = tid >> 5;
-    if (topdown) {
+    // A small frontier with few edges (the roots' own level, a traversal's tail):
+    // every CTA takes in all its rows and edge i goes to thread i of the grid.  A
+    // warp per row walked rows of up to kChunkEdges entries 32 at a time (17 roots
+    // at scale 19: 18 us for the roots' level, 64 at scale 24: 105 us).
+    int flat_total = INT_MAX;
+    if (topdown && count <= (unsigned)kBBlock) {
+      int u = -1, deg = 0, at = 0;
+      if (tid < (int)count) {
+        u = Q[tid];
+        deg = (int)min((long long)__ldg(&p.off[u + 1]) - __ldg(&p.off[u]), 1ll << 21);  // the sum stays below 2^31
+      }
+      const int total = block_exclusive_scan(deg, scan_warp, at);
+      if (total <= min(8 * gthreads, (1ll << 21) - 1)) {  // (no length was cut)
+        flat_total = total;
+        flat.u[tid] = u;
+        flat.pref[tid] = at;
+        if (u >= 0 && (unsigned)tid % nblocks == blockIdx.x) {
+          const Bits f = (Bits)Fc[u];
+          V[u] = (Word)((Bits)V[u] | f);
+          add_level<Word>(p, u, f, k);
+        }
+        __syncthreads();
+      }
+    }
+    if (flat_total != INT_MAX) {
+      int room = kQBuf / kBBlock;  // steps that the CTA's claim buffer is sure to hold
+      for (long long base = (long long)blockIdx.x * kBBlock; base < flat_total; base += gthreads) {
+        if (room-- == 0) {
+          flush_claims_if_full(p, knext, cl, kBBlock, kBigBuf / 2);
+          room = 0;
+        }
+        const int idx = (int)base + tid;
+        if (idx < flat_total) {
+          int lo = 0, hi = kBBlock;  // the last row whose prefix sum is at most idx
+          while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (flat.pref[mid] <= idx) lo = mid;
+            else hi = mid;
+          }
+          const int u = flat.u[lo];
+          const int w = __ldg(&p.adj[__ldg(&p.off[u]) + (idx - flat.pref[lo])]);
+          td_visit(p, Fc, Fn, V, knext, (Bits)Fc[u], u, w, cl);
+        }
+      }
+    } else if (topdown) {
       // frontier rows above kChunkEdges: one CTA per chunk item, with room in the
       // CTA's buffers for the item's claims
       const int64_t* items = p.chunks[k & 1];
@@ -496,25 +564,60 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
         const int w1 = ww < S ? ww + gw : ww + 1;
         return w1 < (ww < S ? S : wend) ? w1 : take_group();
       };
-      for (int ww = (int)gwarp < S ? (int)gwarp : take_group(); ww < nw; ww = next_word(ww)) {
-        const int v = ww * 32 + lane;
-        const bool in = v < p.n;  // (n rounded up to 32 fits: n < 2^31 - 1)
-        Bits need = 0, vv = 0, fv = 0;
-        int deg = 0;
-        long long e = 0;
-        if (in) {
-          vv = (Bits)V[v];
-          fv = (Bits)Fc[v];
-          e = __ldg(&p.toff[v + 1]);
-          const long long d = e - __ldg(&p.toff[v]);
-          need = d == 0 || d > kChunkEdges ? 0ull : ~(vv | fv) & p.mask;
-          deg = (int)d;
+      // A warp goes through its words, folds F_k into V and collects the vertices
+      // that have roots to find; 32 of them at a time are resolved, one per lane, so
+      // that a step's lanes and loads are filled however few of a word's vertices
+      // are left (word by word a late level cost a chain of dependent loads for one
+      // vertex: 64 roots at scale 24, level 5: 450 us).
+      Pending<Word>& pend = s_rows.pend[wid];
+      int npend = 0;
+      for (int ww = (int)gwarp < S ? (int)gwarp : take_group();;) {
+        const bool more = ww < nw;
+        if (more) {
+          const int v = ww * 32 + lane;  // (n rounded up to 32 fits: n < 2^31 - 1)
+          const uint32_t dead = __ldg(&p.dead[ww]);  // the bits past n are set
+          Bits need = 0;
+          if (!((dead >> lane) & 1u)) {
+            const Bits vv = (Bits)V[v], fv = (Bits)Fc[v];
+            need = ~(vv | fv) & p.mask;
+            if (fv) {
+              V[v] = (Word)(vv | fv);
+              add_level<Word>(p, v, fv, k);
+            }
+          } else if (v < p.n) {  // only a root can be here: no arc enters v
+            const Bits fv = (Bits)Fc[v];
+            if (fv) {
+              V[v] = (Word)((Bits)V[v] | fv);
+              add_level<Word>(p, v, fv, k);
+            }
+          }
+          const unsigned m = __ballot_sync(kFull, need != 0);
+          if (need) {
+            const int at = npend + __popc(m & bfsdev::lanemask_lt());
+            pend.v[at] = v;
+            pend.need[at] = (Word)need;
+          }
+          npend += __popc(m);
+          __syncwarp();
+          ww = next_word(ww);
         }
-        const Bits found = resolve_group(p, Fc, v - lane, deg, e, need, lane, list);
-        if (in) {
-          const Bits nv = vv | fv | found;
-          if (nv != vv) V[v] = (Word)nv;
-          if (fv) add_level<Word>(p, v, fv, k);
+        if (npend >= 32 || (!more && npend > 0)) {
+          const int take = min(32, npend);
+          npend -= take;
+          int v = 0, deg = 0;
+          long long e = 0;
+          Bits need = 0;
+          if (lane < take) {
+            v = pend.v[npend + lane];
+            e = __ldg(&p.toff[v + 1]);
+            const long long d = e - __ldg(&p.toff[v]);
+            if (d <= kChunkEdges) {  // (longer rows went by chunks above)
+              deg = (int)d;
+              need = (Bits)pend.need[npend + lane];
+            }
+          }
+          __syncwarp();  // the entries are taken before the next word adds its own
+          const Bits found = resolve_group(p, Fc, v, deg, e, need, lane, list);
           if (found) {
             Fn[v] = (Word)found;
             if (p.directed) {  // the next level's top-down expansion needs the chunks of a long out-row
@@ -522,13 +625,18 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
               if (dout > kChunkEdges) push_chunks_cta(p, knext, cl, v, dout);
             }
           }
+          warp_enqueue(p, knext, wq, nbuf, found != 0, v, lane, false);
+        } else if (!more) {
+          break;
         }
-        warp_enqueue(p, knext, wq, nbuf, found != 0, v, lane, false);
       }
       warp_enqueue(p, knext, wq, nbuf, false, 0, lane, true);
     }
     flush_claims(p, knext, cl);
-    if (!bfsdev::grid_barrier(p.bar, nblocks, bar_target, p.spin_limit, p.status)) return;
+    if (!bfsdev::grid_barrier(p.bar, nblocks, bar_target, p.spin_limit, p.status,
+                              FetchCtr{&p.ctr[(k + 1) % kCtrRing], &s_ctr}))
+      return;
+    prev_count = count;
     if (p.stats && blockIdx.x == 0 && tid == 0 && k < kMaxStatLevels) {
       const uint64_t t = bfsdev::global_timer_ns();
       bfs_level_stat st{};
