@@ -119,7 +119,7 @@ typedef struct bfs_tuning {
                             edges (>= 1024, default 1024) */
   float alpha;           /* heuristic: go PULL when frontier edges * alpha' > unvisited edges and the
                             frontier grows, alpha' = alpha * (1 + 4 n / L2 bytes) (default 20) */
-  float beta;            /* heuristic: leave PULL when frontier count < n / beta', beta' = 4 beta (default 24) */
+  float beta;            /* heuristic: leave PULL when frontier count < n / beta (default 24) */
   int32_t batch_topdown_limit; /* batched: levels with at most this many active vertices expand top-down (default n/64) */
   int32_t small_frontier; /* heuristic: a top-down level whose frontier has at most this many vertices, none of
                              degree above 32, runs TD_WARP instead of TD_BINNED (0 = default: the warps resident

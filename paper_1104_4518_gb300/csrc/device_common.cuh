@@ -115,19 +115,24 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
 // every CTA's writes.
 // `after` runs on thread 0 once the barrier is passed and before the CTA's
 // other threads go on (it fetches what every CTA needs next, with one request
-// per CTA instead of one per warp).
-struct NothingAfter {
+// per CTA instead of one per warp); `meanwhile` starts copies on every thread
+// once the CTA has arrived, which the wait hides, and sees them land at its end.
+struct Nothing {
   __device__ void operator()() const {}
+  __device__ void start() const {}
+  __device__ void finish() const {}
 };
-template <typename After = NothingAfter>
+template <typename After = Nothing, typename Meanwhile = Nothing>
 __device__ __forceinline__ bool grid_barrier(GridBarrier* bar, unsigned nblocks, unsigned long long& target,
-                                             unsigned spin_limit, int* status, After after = After{}) {
+                                             unsigned spin_limit, int* status, After after = After{},
+                                             Meanwhile meanwhile = Meanwhile{}) {
   __shared__ int s_ok;
   __syncthreads();
+  if (threadIdx.x == 0) red_release_add_u64(&bar->count, 1ull);
+  meanwhile.start();
   if (threadIdx.x == 0) {
     int ok = 1;
     target += nblocks;
-    red_release_add_u64(&bar->count, 1ull);
     unsigned polls = 0;
     while (ld_acquire_u64(&bar->count) < target) {
       if (++polls > spin_limit || ld_relaxed_i32(status) != 0) {
@@ -140,6 +145,7 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier* bar, unsigned nblocks,
     else after();
     s_ok = ok;
   }
+  meanwhile.finish();
   __syncthreads();
   return s_ok != 0;
 }
@@ -150,18 +156,18 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier* bar, unsigned nblocks,
 // often, since nothing waits on them).  Every CTA must pass the same
 // `arrivals`.  A launch that used such barriers must pad the counter to a
 // multiple of its grid size before it ends (barrier_pad).
-template <typename After = NothingAfter>
+template <typename After = Nothing, typename Meanwhile = Nothing>
 __device__ __forceinline__ bool grid_barrier_partial(GridBarrier* bar, unsigned arrivals, unsigned long long& target,
-                                                     unsigned spin_limit, int* status, After after = After{}) {
+                                                     unsigned spin_limit, int* status, After after = After{},
+                                                     Meanwhile meanwhile = Meanwhile{}) {
   __shared__ int s_ok;
   __syncthreads();
+  const bool arrive = blockIdx.x < arrivals;
+  if (threadIdx.x == 0 && arrive) red_release_add_u64(&bar->count, 1ull);
+  meanwhile.start();
   if (threadIdx.x == 0) {
     int ok = 1;
-    const bool arrive = blockIdx.x < arrivals;
     target += arrivals;
-    if (arrive) {
-      red_release_add_u64(&bar->count, 1ull);
-    }
     unsigned polls = 0;
     while (ld_acquire_u64(&bar->count) < target) {
       if (++polls > spin_limit || ld_relaxed_i32(status) != 0) {
@@ -174,6 +180,7 @@ __device__ __forceinline__ bool grid_barrier_partial(GridBarrier* bar, unsigned 
     else after();
     s_ok = ok;
   }
+  meanwhile.finish();
   __syncthreads();
   return s_ok != 0;
 }

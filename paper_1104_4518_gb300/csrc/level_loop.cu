@@ -126,9 +126,9 @@ struct LoopParams {
   const int64_t* __restrict__ t_dir_jc;
   const int64_t* __restrict__ t_dir_ir;
   int32_t t_rb_bits, t_cb_bits, t_nrb, t_ncb;
-  int32_t phase_smem_off;  // byte offset of the pull / tiled phase's area in dynamic shared memory
   const int4* __restrict__ probe;  // per vertex an arc enters: in-degree and its row's largest three ids, or null
   const uint32_t* __restrict__ rank;  // per bitmap word: the records before it
+  long long flat_visits;           // top-down: visits per thread up to which a small frontier's edges are dealt flat
   int32_t pull_words;              // bitmap words per pull chunk
   int32_t claim_by_parent;         // top-down: the first offer to a parent claims the vertex (else the next bitmap does)
   int32_t fr_shift;                // pull: log2 of the vertices per shared-memory frontier bit
@@ -251,6 +251,7 @@ __device__ __forceinline__ void end_phase(const LoopParams& p, int knext, Acc& a
 }
 
 struct Smem {
+  float4 mlp_y;  // outputs of the selector network
   LevelCtr ctr;  // counters of the level to expand, fetched by thread 0 at the barrier before it
   int owner;
   int cu;
@@ -258,8 +259,6 @@ struct Smem {
   int warp_tmp[kWarps + 1];
   unsigned long long acc[4];
   Claims cl;
-  __align__(16) float h1[64];  // selector network: hidden layer 1, choice
-  int choice;
   unsigned long long next_item;  // top-down: the next chunk item of this CTA
 };
 
@@ -320,7 +319,7 @@ __device__ void flat_phase(const LoopParams& p, int k, unsigned count, Smem& sm,
     }
   }
   __syncthreads();
-  int room = kQBuf / (kBlock);  // steps that the CTA's claim buffer is sure to hold
+  int room = kQBuf / kBlock;  // steps that the CTA's claim buffer is sure to hold
   for (int base = (int)blockIdx.x * kBlock; base < total; base += (int)G * kBlock) {
     if (room-- == 0) {
       flush_claims_if_full(p, k + 1, sm.cl, kBlock, kBigBuf / 2);
@@ -334,8 +333,14 @@ __device__ void flat_phase(const LoopParams& p, int k, unsigned count, Smem& sm,
   }
 }
 
-__device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned count, unsigned nchunks, Smem& sm,
-                              FlatSmem& fl, Acc& acc, unsigned G) {
+// A frontier row fetched ahead of the phase (u < 0: none).
+struct FirstRow {
+  int u = -1;
+  long long b = 0, e = 0;
+};
+
+__device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned count, unsigned nchunks,
+                              const FirstRow& first, Smem& sm, FlatSmem& fl, Acc& acc, unsigned G) {
   const uint32_t* cur = p.bits[k % 3];
   uint32_t* nxt = p.bits[(k + 1) % 3];
   const int32_t* Q = p.queue[k % 3];
@@ -370,12 +375,17 @@ __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned 
     }
   } else if (variant == BFS_VARIANT_TD_WARP) {
     const long long gwarps = gthreads / 32;
+    FirstRow row = first;  // the row of entry blockIdx.x + warp * G, where it was fetched
     for (long long i = blockIdx.x + (long long)(tid >> 5) * G; i < count; i += gwarps) {
-      const int u = Q[i];
-      if (lane == 0) atomicOr(&p.vis[u >> 5], 1u << (u & 31));
-      const long long b = __ldg(&p.off[u]), e = __ldg(&p.off[u + 1]);
-      if (e - b > p.chunk_deg) continue;
-      for (long long j = b + lane; j < e; j += 32) td_visit(p, cur, nxt, k, u, __ldg(&p.adj[j]), acc, sm.cl);
+      if (row.u < 0) {
+        row.u = Q[i];
+        row.b = __ldg(&p.off[row.u]);
+        row.e = __ldg(&p.off[row.u + 1]);
+      }
+      if (lane == 0) atomicOr(&p.vis[row.u >> 5], 1u << (row.u & 31));
+      if (row.e - row.b <= p.chunk_deg)
+        for (long long j = row.b + lane; j < row.e; j += 32) td_visit(p, cur, nxt, k, row.u, __ldg(&p.adj[j]), acc, sm.cl);
+      row.u = -1;
     }
   } else {  // BFS_VARIANT_TD_BINNED
     for (long long tile = 0; tile < count; tile += gthreads) {
@@ -965,18 +975,15 @@ __device__ void tiled_phase(const LoopParams& p, int k, Smem& sm, FlatSmem& fl, 
   warp_enqueue(p, knext, wq, nbuf, false, 0, lane, true);
 }
 
-// The selector network on one warp: every lane computes the 12 level features
-// in registers (lane j < 3 brings bin count j), then the warp evaluates the
-// network on the parameters in the warp layout; returns the chosen variant on
-// every lane.  Kept out of line so that its registers do not crowd the phases.
-__device__ __noinline__ int learned_choice(const LoopParams& p, const float* w, float* h1, int lane, int k,
-                                           long long count, long long edges, long long unvisited,
-                                           long long unvisited_edges, long long binv) {
+// The selector network on four warps of the CTA (tid counts from their first),
+// on the parameters in the warp layout; its outputs go to y.
+__device__ __forceinline__ void learned_outputs(const LoopParams& p, const float* w, bfsdev::MlpScratch& sc, float* y,
+                                             int tid, int k, const LevelCtr& c, long long unvisited,
+                                             long long unvisited_edges) {
   float x[12];
-  bfsdev::level_features(p.feat_log_n, p.feat_log_nnz, p.feat_inv_n, p.feat_inv_nnz, k, count, edges, unvisited,
-                         unvisited_edges, __shfl_sync(kFull, binv, 0), __shfl_sync(kFull, binv, 1),
-                         __shfl_sync(kFull, binv, 2), x);
-  return bfsdev::warp_mlp_argmin(w, x, h1, lane);
+  bfsdev::warp_level_features(p.feat_log_n, p.feat_log_nnz, p.feat_inv_n, p.feat_inv_nnz, k, c.count,
+                              (long long)c.edges, unvisited, unvisited_edges, c.bins, tid & 31, x);
+  bfsdev::warps_mlp_outputs(w, x, sc, y, tid >> 5, tid & 31);
 }
 
 // Direction choice in the manner of direction-optimising BFS: go pull when the
@@ -997,22 +1004,44 @@ __device__ __forceinline__ int heuristic_variant(const LoopParams& p, int prev_v
 constexpr size_t kFlatBytes = (sizeof(FlatSmem) + 15) / 16 * 16;
 // the largest phase's area, without and with the tiled phase
 constexpr size_t kPhaseBytes = std::max(sizeof(PullSmem), kFlatBytes);
+constexpr size_t kMlpBytes = (sizeof(float) * BFS_MLP_PARAMS + 15) / 16 * 16;
+static_assert(kPhaseBytes >= kMlpBytes + sizeof(bfsdev::MlpScratch), "the network fits the phases' area");
 constexpr size_t kTiledBytes = std::max(kPhaseBytes, kFlatBytes + sizeof(uint32_t) * 3 * kTileWordsMax);
+
+// Brings the selector network's parameters to shared memory during a barrier.
+template <bool kLearned>
+struct FetchMlp {
+  float* dst;
+  const float* src;
+  __device__ void start() const {
+    if constexpr (kLearned) {
+      static_assert(BFS_MLP_PARAMS % 4 == 0, "whole 16-byte groups");
+      for (int i = threadIdx.x; i < BFS_MLP_PARAMS / 4; i += kBlock)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst + 4 * i)), "l"(src + 4 * i) : "memory");
+    }
+  }
+  __device__ void finish() const {
+    if constexpr (kLearned) asm volatile("cp.async.wait_all;" ::: "memory");
+  }
+};
 
 // kTiles: the kernel can run the tiled phase.  Runs that cannot pick the tiled
 // variant launch the instance without it: on R-MAT scale 26 the tiled phase's
 // code alone made the other phases 5 % slower.
-template <bool kTiles>
+// kLearned: the selector network may choose the variants.  Learned runs never
+// pick the tiled variant, and the other runs do without the network's code.
+template <bool kTiles, bool kLearned>
 __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
   __shared__ Smem sm;
-  // dynamic shared memory: the selector network's parameters (BFS_MLP_PARAMS
-  // floats) when the learned selector is on, then one area that the phases use
-  // in turn: PullSmem, or FlatSmem and the tiled phase's 3 * kTileWordsMax words
+  // dynamic shared memory: one area that the phases use in turn (PullSmem, or
+  // FlatSmem and the tiled phase's 3 * kTileWordsMax words), and between phases
+  // the selector network's parameters
   extern __shared__ __align__(16) unsigned char s_dyn[];
-  float* s_mlp = reinterpret_cast<float*>(s_dyn);
-  FlatSmem& s_flat = *reinterpret_cast<FlatSmem*>(s_dyn + p.phase_smem_off);
-  uint32_t* s_tile = reinterpret_cast<uint32_t*>(s_dyn + p.phase_smem_off + kFlatBytes);
-  PullSmem& s_pull = *reinterpret_cast<PullSmem*>(s_dyn + p.phase_smem_off);
+  FlatSmem& s_flat = *reinterpret_cast<FlatSmem*>(s_dyn);
+  uint32_t* s_tile = reinterpret_cast<uint32_t*>(s_dyn + kFlatBytes);
+  PullSmem& s_pull = *reinterpret_cast<PullSmem*>(s_dyn);
+  [[maybe_unused]] float* const s_mlp = reinterpret_cast<float*>(s_dyn);
+  [[maybe_unused]] bfsdev::MlpScratch& s_mlp_scratch = *reinterpret_cast<bfsdev::MlpScratch*>(s_dyn + kMlpBytes);
   const int tid = threadIdx.x;
   unsigned long long bar_target = 0;
   if (tid == 0) {
@@ -1021,9 +1050,11 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
     claims_reset(sm.cl);
     sm.acc[0] = sm.acc[1] = sm.acc[2] = sm.acc[3] = 0;
   }
-  const bool learned = p.selector == BFS_SELECT_LEARNED && p.mlp != nullptr;
-  if (learned)
-    for (int i = tid; i < BFS_MLP_PARAMS; i += kBlock) s_mlp[bfsdev::warp_layout_index(i)] = p.mlp[i];
+  // The network's parameters come to the phases' area during every barrier, when
+  // it is free.  Kept in 21 KB of their own they left the expansion half the L1
+  // (learned runs, in their own 21 KB against brought at each barrier: 4 roots at scale 26 5,880 us and 5,635, scale
+  // 21 442 and 413, Erdos-Renyi 1 M 232 and 222; grid 128^3, all narrow levels, 2,702 and 2,763).
+  const FetchMlp<kLearned> fetch_mlp{s_mlp, p.mlp};
 
   const long long gtid = (long long)blockIdx.x * kBlock + tid;
   const long long gthreads = (long long)gridDim.x * kBlock;
@@ -1098,7 +1129,8 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
       if (deg > p.chunk_deg) push_chunks(p, 0, s0, deg);
     }
   }
-  if (!bfsdev::grid_barrier(p.bar, nblocks, bar_target, p.spin_limit, p.status, FetchCtr{&p.ctr[0], &sm.ctr})) return;
+  if (!bfsdev::grid_barrier(p.bar, nblocks, bar_target, p.spin_limit, p.status, FetchCtr{&p.ctr[0], &sm.ctr}, fetch_mlp))
+    return;
 
   if (!single) {  // seed level 0 with the sources (block 0)
     if (blockIdx.x == 0) {
@@ -1116,7 +1148,8 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
       if (tid == 0) p.ctr[0].count = (unsigned)p.nsources;
       end_phase(p, 0, acc, sm);
     }
-    if (!bfsdev::grid_barrier(p.bar, nblocks, bar_target, p.spin_limit, p.status, FetchCtr{&p.ctr[0], &sm.ctr})) return;
+    if (!bfsdev::grid_barrier(p.bar, nblocks, bar_target, p.spin_limit, p.status, FetchCtr{&p.ctr[0], &sm.ctr}, fetch_mlp))
+      return;
   }
 
   // ---- level loop
@@ -1134,7 +1167,6 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
     const unsigned count = c.count;
     const unsigned nchunks = c.chunks;
     const long long edges = (long long)c.edges;
-    const long long binv = (learned && tid < 3) ? (long long)c.bins[tid] : 0;
     const bool big_rows = (c.bins[1] | c.bins[2]) != 0;
     const bool sparse_clr = k >= 1 && (long long)prev_count * 4 < p.nwords;
     const int32_t* PQ = p.queue[(k + 2) % 3];
@@ -1169,18 +1201,25 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
     PHASE_TS(k, 1);
 
     int variant;
-    if (p.selector == BFS_SELECT_FORCED) {
+    FirstRow first;
+    if constexpr (kLearned) {
+      // every CTA evaluates the network (all compute the same bits)
+      // The last four warps compute the outputs, about 0.9 us of latencies; meanwhile each other warp fetches the
+      // row it starts with if the level goes a warp per vertex (a narrow level's vertices all sit in those warps).
+      if (tid >= kBlock - bfsdev::kMlpThreads) {
+        learned_outputs(p, s_mlp, s_mlp_scratch, &sm.mlp_y.x, tid - (kBlock - bfsdev::kMlpThreads), k, c, unvisited,
+                        unvisited_edges);
+      } else if (part && blockIdx.x + (unsigned)(tid >> 5) * G < count) {
+        first.u = p.queue[k % 3][blockIdx.x + (unsigned)(tid >> 5) * G];
+        first.b = __ldg(&p.off[first.u]);
+        first.e = __ldg(&p.off[first.u + 1]);
+      }
+      __syncthreads();  // the outputs are there, and the network's area is free for the phase
+      variant = bfsdev::mlp_argmin(sm.mlp_y);
+    } else if (p.selector == BFS_SELECT_FORCED) {
       variant = p.forced;
     } else if (p.selector == BFS_SELECT_SCHEDULE && k < p.schedule_len) {
       variant = p.schedule[k];
-    } else if (learned) {
-      // warp 0 of every CTA evaluates the network (all CTAs compute the same bits)
-      if (tid < 32) {
-        const int best = learned_choice(p, s_mlp, sm.h1, tid, k, count, edges, unvisited, unvisited_edges, binv);
-        if (tid == 0) sm.choice = best;
-      }
-      __syncthreads();
-      variant = sm.choice;
     } else {
       variant = heuristic_variant(p, prev_variant, count, prev_count, edges, unvisited_edges, !big_rows);
     }
@@ -1191,9 +1230,9 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
       if (variant == BFS_VARIANT_PULL) pull_phase(p, k, count, sm, s_pull, acc, G);
       else if (kTiles && variant == BFS_VARIANT_TILED) tiled_phase(p, k, sm, s_flat, s_tile, acc, G);
       // the degree-binned variant deals a small frontier's edges out flat
-      else if (variant == BFS_VARIANT_TD_BINNED && count <= (unsigned)kFlatRows && edges <= 16ll * pthreads)
+      else if (variant == BFS_VARIANT_TD_BINNED && count <= (unsigned)kFlatRows && edges <= p.flat_visits * pthreads)
         flat_phase(p, k, count, sm, s_flat, acc, G);
-      else topdown_phase(p, k, variant, count, nchunks, sm, s_flat, acc, G);
+      else topdown_phase(p, k, variant, count, nchunks, first, sm, s_flat, acc, G);
       PHASE_TS(k, 3);
       end_phase(p, k + 1, acc, sm);
     }
@@ -1204,7 +1243,9 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
     const int4 level_bins = p.want_stats && blockIdx.x == 0 && tid == 0
                                 ? make_int4((int)c.bins[0], (int)c.bins[1], (int)c.bins[2], 0)
                                 : make_int4(0, 0, 0, 0);
-    if (!bfsdev::grid_barrier_partial(p.bar, G, bar_target, p.spin_limit, p.status, FetchCtr{&p.ctr[(k + 1) % kCtrRing], &sm.ctr})) return;
+    if (!bfsdev::grid_barrier_partial(p.bar, G, bar_target, p.spin_limit, p.status,
+                                      FetchCtr{&p.ctr[(k + 1) % kCtrRing], &sm.ctr}, fetch_mlp))
+      return;
     PHASE_TS(k, 6);
 
     if (p.want_stats && blockIdx.x == 0 && tid == 0 && k < kMaxStatLevels) {
@@ -1337,9 +1378,7 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
   // top-down's atomics on the parent array get dearer once 4 bytes per vertex
   // no longer fit in L2, so the switch to pull comes earlier on large graphs
   p.alpha = (float)(t.alpha * (1.0 + 4.0 * (double)g->n / (double)(di.l2_bytes > 0 ? di.l2_bytes : (1ll << 27))));
-  // a pull level costs about one microsecond per 45,000 bitmap words plus its live rows, a top-down one 1 us per
-  // 16,000 edges: they meet near n / 90 vertices (R-MAT scale 26, 1.6 M vertices: pull 48 us, top-down 112 us)
-  p.beta = 4.0f * t.beta;
+  p.beta = t.beta;
   p.parts = g->parts;
   p.part_base = g->d_part_base;
   p.part_out = r.part_out;
@@ -1356,22 +1395,18 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
     p.t_ncb = ts->ncb;
   }
 
-  // the pull / tiled phase's area follows the network's parameters in dynamic shared memory
-  const size_t mlp_bytes = p.mlp ? (sizeof(float) * BFS_MLP_PARAMS + 15) / 16 * 16 : 0;
-  p.phase_smem_off = (int32_t)mlp_bytes;
-  const size_t dyn_smem = mlp_bytes + (p.t_jc ? kTiledBytes : kPhaseBytes);
-  const void* kernel = p.t_jc ? (const void*)level_loop_kernel<true> : (const void*)level_loop_kernel<false>;
+  const size_t dyn_smem = p.t_jc ? kTiledBytes : kPhaseBytes;
+  const void* const kernels[] = {(const void*)level_loop_kernel<false, false>, (const void*)level_loop_kernel<true, false>,
+                                 (const void*)level_loop_kernel<false, true>};
+  const void* kernel = kernels[p.mlp ? 2 : p.t_jc ? 1 : 0];
   {  // the attribute belongs to the current device: set it once per device
     static std::mutex mu;
     static bool configured[64] = {};
     std::lock_guard<std::mutex> lk(mu);
     if (di.device < 0 || di.device >= 64) return fail(BFS_ERR_UNSUPPORTED, "device ordinal out of range");
     if (!configured[di.device]) {
-      const int max_dyn = (int)((sizeof(float) * BFS_MLP_PARAMS + 15) / 16 * 16 + kTiledBytes);
-      BFS_CUDA_TRY(cudaFuncSetAttribute((const void*)level_loop_kernel<false>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn));
-      BFS_CUDA_TRY(cudaFuncSetAttribute((const void*)level_loop_kernel<true>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn));
+      for (const void* f : kernels)
+        BFS_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTiledBytes));
       configured[di.device] = true;
     }
   }
@@ -1387,6 +1422,9 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
   // that conflict less (Erdos-Renyi, n = 1 M, 77 K-vertex level: 32 -> 27 us; grid 128^3: 2.56 -> 2.50 ms); once
   // the parents no longer sit in L2 its result comes from DRAM (scale 26, 7 M edges: 425 -> 496 us).
   p.claim_by_parent = 4ll * g->n <= (di.l2_bytes > 0 ? di.l2_bytes : (1ll << 27)) / 2;
+  // 32 parts of a ragged batch, 0.9 M edges: flat 28 us, by rows and chunks 55 us; at scale 26, 2.1 M edges, the
+  // chunks' two visits in flight win (171 us against 223)
+  p.flat_visits = p.claim_by_parent ? 16 : 4;
   // one chunk per resident warp while a lane per word allows it (see pull_phase)
   const long long grid_warps = (long long)grid * kWarps;
   p.pull_words = (int)std::min<long long>(32, std::max<long long>(1, (w->nwords + grid_warps - 1) / grid_warps));

@@ -335,10 +335,12 @@ const float* learned_params_device() {
   if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
   if ((int)g_sel_dev.size() <= dev) g_sel_dev.resize(dev + 1, nullptr);
   if (!g_sel_dev[dev]) {
+    std::vector<float> warp(BFS_MLP_PARAMS);
+    for (int i = 0; i < BFS_MLP_PARAMS; ++i) warp[bfsdev::warp_layout_index(i)] = g_sel_host[i];
     float* p = nullptr;
     if (cudaMalloc(&p, sizeof(float) * BFS_MLP_PARAMS) != cudaSuccess) return nullptr;
-    if (cudaMemcpy(p, g_sel_host.data(), sizeof(float) * BFS_MLP_PARAMS, cudaMemcpyHostToDevice) != cudaSuccess) {
-      dev_free(p);
+    if (cudaMemcpy(p, warp.data(), sizeof(float) * BFS_MLP_PARAMS, cudaMemcpyHostToDevice) != cudaSuccess) {
+      cudaFree(p);
       return nullptr;
     }
     g_sel_dev[dev] = p;

@@ -46,12 +46,12 @@ def training_graphs():
     for i, (sc, ef, a) in enumerate(rm):
         b = rmat_bc(a)
         specs.append((f"rmat-s{sc}-ef{ef}-a{a}", (lambda sc=sc, ef=ef, a=a, b=b, i=i:
-                                                   inputs.rmat(sc, ef, a, b, b, seed=600 + i)), 700 + i, 6))
+                                                   inputs.rmat(sc, ef, a, b, b, seed=600 + i)), 700 + i, 12))
     for N in (64, 96, 128, 160, 192):
         specs.append((f"grid{N}", (lambda N=N: inputs.grid3d(N)), None, 1))
     for i, (lg, d) in enumerate([(20, 4), (20, 16), (21, 8), (21, 16), (22, 4), (22, 32)]):
         specs.append((f"er-{lg}-d{d}", (lambda lg=lg, d=d, i=i: inputs.erdos_renyi(1 << lg, d, seed=650 + i)),
-                      750 + i, 3))
+                      750 + i, 6))
     return specs
 
 
@@ -197,7 +197,7 @@ def main(argv=None):
     ap.add_argument("--out", default=DEFAULT_WEIGHTS)
     ap.add_argument("--weights", default=DEFAULT_WEIGHTS)
     ap.add_argument("--report", default=None)
-    ap.add_argument("--steps", type=int, default=4000)
+    ap.add_argument("--steps", type=int, default=12000)
     ap.add_argument("--lr", type=float, default=3e-3)
     ap.add_argument("--reps", type=int, default=3)
     args = ap.parse_args(argv)
