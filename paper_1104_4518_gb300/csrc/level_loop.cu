@@ -1273,16 +1273,35 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
     p.misc[0] = k;
     *p.edges_out = p.directed ? cum_edges : cum_edges / 2;  // arcs, or undirected edges
   }
-  // ragged: copy the union-space outputs into each part's arrays, local ids
+  // ragged: copy the union-space outputs into each part's arrays, local ids.  One pass over the union with four
+  // vertices of a thread in flight: bound by loads that hit L2 and by the stores.  A pass per part kept the grid
+  // waiting for each part's loads in turn (32 parts of 2^12 to 2^20 vertices, whole call: 417 -> 383 us).
   if (p.part_out != nullptr) {
-    for (int q = 0; q < p.parts; ++q) {
-      const long long base = p.part_base[q], size = p.part_base[q + 1] - base;
-      int32_t* lo = p.part_out[q];
-      int32_t* po = p.part_out[p.parts + q];
-      for (long long v = gtid; v < size; v += gthreads) {
-        lo[v] = p.level[base + v];
-        const int par = p.parent[base + v];
-        po[v] = par >= 0 ? (int)(par - base) : -1;
+    constexpr int kFlight = 4;
+    for (long long v0 = gtid; v0 < p.n; v0 += kFlight * gthreads) {
+      int lev[kFlight], par[kFlight];
+#pragma unroll
+      for (int j = 0; j < kFlight; ++j) {
+        const long long v = v0 + j * gthreads;
+        if (v < p.n) {
+          lev[j] = p.level[v];
+          par[j] = p.parent[v];
+        }
+      }
+      int q = 0;
+#pragma unroll
+      for (int j = 0; j < kFlight; ++j) {
+        const long long v = v0 + j * gthreads;
+        if (v >= p.n) break;
+        int last = p.parts - 1;  // v's part: the last one that starts at or before v (v grows with j, so q only rises)
+        while (q < last) {
+          const int mid = (q + last + 1) / 2;
+          if (p.part_base[mid] <= v) q = mid;
+          else last = mid - 1;
+        }
+        const long long base = p.part_base[q];
+        p.part_out[q][v - base] = lev[j];
+        p.part_out[p.parts + q][v - base] = par[j] >= 0 ? (int)(par[j] - base) : -1;
       }
     }
   }
