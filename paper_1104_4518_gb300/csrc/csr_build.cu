@@ -51,7 +51,8 @@ constexpr int kKeyTile = kKeyThreads * kKeyItems;  // 2,048 edges
 // v -> u, mode 1 u -> v only, mode 2 v -> u only (the transpose).  A tile's
 // keys take their places with one atomic (one per warp and step on the same
 // word made this kernel 1.48 ms for 67 M edges), in any order: the sort orders
-// them, and equal keys are alike.
+// them, and equal keys are alike.  0.36 ms for 67 M edges, 0.24 of them the DRAM
+// traffic's due; 0.62 while the plan was indexed at run time, from a local copy.
 __global__ void __launch_bounds__(kKeyThreads) make_keys_kernel(const int32_t* __restrict__ src,
                                                                 const int32_t* __restrict__ dst, int64_t m, int32_t n,
                                                                 int vbits, int mode, SortPlan plan,
@@ -66,8 +67,9 @@ __global__ void __launch_bounds__(kKeyThreads) make_keys_kernel(const int32_t* _
   for (int i = tid; i < plan.passes * kSortBins; i += kKeyThreads) s_h[i] = 0;
   __syncthreads();
   auto count = [&](uint64_t k) {
-    for (int q = 0; q < plan.passes; ++q)
-      atomicAdd(&s_h[q * kSortBins + (int)(k >> plan.shift[q] & ((1u << plan.bits[q]) - 1u))], 1u);
+#pragma unroll
+    for (int q = 0; q < kSortMaxPasses; ++q)
+      if (q < plan.passes) atomicAdd(&s_h[q * kSortBins + (int)(k >> plan.shift[q] & ((1u << plan.bits[q]) - 1u))], 1u);
   };
   for (long long base = (long long)blockIdx.x * kKeyTile; base < m; base += (long long)gridDim.x * kKeyTile) {
     int u[kKeyItems], v[kKeyItems];
@@ -257,7 +259,9 @@ constexpr int kEmitTile = kEmitThreads * kEmitItems;  // 8,192 keys
 // kept, its slot is the number of kept keys before it (within the warp's 512
 // consecutive keys by ballots, across tiles by a chained scan), and where its
 // row differs from the predecessor's the rows in between start at that slot.
-// 134 M keys: 0.72 ms (a flag scan and an emission kernel took 1.7 ms).
+// 134 M keys: 0.60 ms, 0.24 of them the
+// DRAM traffic's due (a flag scan and an emission kernel took 1.7 ms; with 64-bit
+// end tests and four shuffles per key and step 0.72).
 __global__ void __launch_bounds__(kEmitThreads, 2) emit_csr_kernel(const uint64_t* __restrict__ keys, int vbits, int32_t n,
                                                                 int64_t* __restrict__ off, int32_t* __restrict__ adj,
                                                                 uint64_t* __restrict__ state, BuildReport* rep) {
@@ -274,20 +278,21 @@ __global__ void __launch_bounds__(kEmitThreads, 2) emit_csr_kernel(const uint64_
   const long long N = (long long)rep->nkeys, tile = s_tile, seg = tile * kEmitTile + wid * (32 * kEmitItems);
   if (tile * kEmitTile >= N || !s_ok) return;
   const uint64_t vmask = (1ull << vbits) - 1ull;
+  const int left = (int)max(0ll, min(32ll * kEmitItems, N - seg));  // the warp's keys
   uint64_t key[kEmitItems];
 #pragma unroll
-  for (int i = 0; i < kEmitItems; ++i) key[i] = seg + i * 32 + lane < N ? keys[seg + i * 32 + lane] : 0;
-  uint64_t before = 0;  // the key before the warp's first
+  for (int i = 0; i < kEmitItems; ++i) key[i] = i * 32 + lane < left ? keys[seg + i * 32 + lane] : 0;
+  uint64_t before = ~0ull;  // the key before the warp's first
   if (seg > 0 && seg < N) before = keys[seg - 1];
   unsigned kept[kEmitItems];
   int cnt = 0;
+  uint64_t carry = before;  // lane 0's predecessor
 #pragma unroll
   for (int i = 0; i < kEmitItems; ++i) {
-    const long long idx = seg + i * 32 + lane;
-    uint64_t prev = __shfl_up_sync(kFull, key[i], 1);
-    const uint64_t carry = i > 0 ? __shfl_sync(kFull, key[i > 0 ? i - 1 : 0], 31) : before;
-    if (lane == 0) prev = carry;
-    kept[i] = __ballot_sync(kFull, idx < N && (idx == 0 || key[i] != prev));
+    const uint64_t turned = __shfl_sync(kFull, key[i], (lane + 31) & 31);
+    const uint64_t prev = lane == 0 ? carry : turned;
+    carry = turned;
+    kept[i] = __ballot_sync(kFull, i * 32 + lane < left && key[i] != prev);
     cnt += __popc(kept[i]);
   }
   if (lane == 0) s_cnt[wid] = cnt;
@@ -311,20 +316,19 @@ __global__ void __launch_bounds__(kEmitThreads, 2) emit_csr_kernel(const uint64_
   __syncthreads();
   if (!s_ok) return;
   long long at = (long long)s_at + warp_at;
+  int carry_row = seg > 0 ? (int)(before >> vbits) : -1;
 #pragma unroll
   for (int i = 0; i < kEmitItems; ++i) {
-    const long long idx = seg + i * 32 + lane;
-    uint64_t prev = __shfl_up_sync(kFull, key[i], 1);
-    const uint64_t carry = i > 0 ? __shfl_sync(kFull, key[i > 0 ? i - 1 : 0], 31) : before;
-    if (lane == 0) prev = carry;
+    const int row = (int)(key[i] >> vbits), turned = __shfl_sync(kFull, row, (lane + 31) & 31);
+    const int prev = lane == 0 ? carry_row : turned;
+    carry_row = turned;
     const long long pos = at + __popc(kept[i] & bfsdev::lanemask_lt());
     const bool first = (kept[i] >> lane) & 1u;
-    const long long row = (long long)(key[i] >> vbits);
     if (first) {
       adj[pos] = (int32_t)(key[i] & vmask);
-      for (long long r = idx == 0 ? 0 : (long long)(prev >> vbits) + 1; r <= row; ++r) off[r] = pos;
+      for (int r = prev + 1; r <= row; ++r) off[r] = pos;
     }
-    if (idx == N - 1) {  // the rows after the last key's end with it
+    if (seg + i * 32 + lane == N - 1) {  // the rows after the last key's end with it
       rep->nnz = (unsigned long long)(pos + (first ? 1 : 0));
       for (long long r = row + 1; r <= n; ++r) off[r] = pos + (first ? 1 : 0);
     }
