@@ -51,6 +51,29 @@ struct __align__(16) GradSmem {
   float sq[kTS * 4];  // squared errors by sample and output
 };
 
+// The reduction and the Adam step are launched to start while the kernel before
+// them runs out (programmatic dependent launch): their CTAs take their places
+// early and wait there for that kernel's end before they touch memory, which hides
+// a launch's latency of about 2 us (1,379 samples: a gradient call 27.8 -> 25.7 us,
+// a training step 22.5 -> 18.5).  What they read is not const __restrict__, as
+// it may still be written when they start.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... K, typename... A>
+cudaError_t launch_early(void (*kernel)(K...), unsigned grid, unsigned block, cudaStream_t s, A... args) {
+  cudaLaunchAttribute early[1];
+  early[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = s;
+  cfg.attrs = early;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
+
 // Partial gradient and squared error of one tile of kTS samples.  Thread
 // (t, grp) computes unit t of four samples, so that a weight loaded from
 // shared memory serves four products; the W2 gradient is 2 x 4 blocks in
@@ -65,6 +88,7 @@ __global__ void __launch_bounds__(kGradThreads) mlp_grad_tile_kernel(const float
                                                                      const float* __restrict__ T, int B,
                                                                      float* __restrict__ partial,
                                                                      float* __restrict__ partial_loss) {
+  launch_dependents();
   extern __shared__ __align__(16) unsigned char s_raw[];
   GradSmem& g = *reinterpret_cast<GradSmem*>(s_raw);
   constexpr int kPer = kTS * 64 / kGradThreads;  // samples per thread: 4
@@ -261,8 +285,10 @@ static_assert(kTS == 32 && kGradThreads == 512, "the gradient tile's thread mapp
 
 // Sums over the tiles, ascending: one thread per parameter, 16 loads in flight,
 // and one for the loss.
-__global__ void mlp_reduce_kernel(const float* __restrict__ partial, const float* __restrict__ partial_loss,
+__global__ void mlp_reduce_kernel(const float* partial, const float* partial_loss,
                                   int ntiles, int B, float* __restrict__ grad, float* __restrict__ loss) {
+  launch_dependents();
+  wait_for_previous_kernel();
   const int pidx = blockIdx.x * blockDim.x + threadIdx.x;
   if (pidx > BFS_MLP_PARAMS || (pidx == BFS_MLP_PARAMS && !loss)) return;
   const bool is_loss = pidx == BFS_MLP_PARAMS;
@@ -289,9 +315,10 @@ __global__ void mlp_reduce_kernel(const float* __restrict__ partial, const float
   else grad[pidx] = a;
 }
 
-__global__ void adam_kernel(float* __restrict__ params, const float* __restrict__ grad, float* __restrict__ m,
+__global__ void adam_kernel(float* __restrict__ params, const float* grad, float* __restrict__ m,
                             float* __restrict__ v, float lr, float beta1, float beta2, float eps, float bc1,
                             float bc2) {
+  wait_for_previous_kernel();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= BFS_MLP_PARAMS) return;
   const float gi = grad[i];
@@ -316,8 +343,8 @@ int grad_impl(const float* params, const float* X, const float* T, int B, float*
     configured = true;
   }
   mlp_grad_tile_kernel<<<ntiles, kGradThreads, grad_smem_bytes(), s>>>(params, X, T, B, partial, partial_loss);
-  mlp_reduce_kernel<<<BFS_MLP_PARAMS / 64 + 1, 64, 0, s>>>(partial, partial_loss, ntiles, B, grad, loss);
   BFS_CUDA_TRY(cudaGetLastError());
+  BFS_CUDA_TRY(launch_early(mlp_reduce_kernel, BFS_MLP_PARAMS / 64 + 1, 64, s, partial, partial_loss, ntiles, B, grad, loss));
   return BFS_OK;
 }
 
@@ -400,9 +427,8 @@ int bfs_mlp_adam(float* params, const float* grad, float* m, float* v, int32_t t
   if (!params || !grad || !m || !v || t < 1) return fail(BFS_ERR_INVALID_ARG, "bfs_mlp_adam: bad argument");
   const float bc1 = (float)(1.0 - std::pow((double)beta1, (double)t));
   const float bc2 = (float)(1.0 - std::pow((double)beta2, (double)t));
-  adam_kernel<<<(BFS_MLP_PARAMS + 255) / 256, 256, 0, (cudaStream_t)stream>>>(params, grad, m, v, lr, beta1, beta2,
-                                                                              eps, bc1, bc2);
-  BFS_CUDA_TRY(cudaGetLastError());
+  BFS_CUDA_TRY(launch_early(adam_kernel, (BFS_MLP_PARAMS + 255) / 256, 256, (cudaStream_t)stream, params, grad, m, v, lr,
+                            beta1, beta2, eps, bc1, bc2));
   return BFS_OK;
 }
 
