@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(kBBlock, 2) batch_kernel(BatchParams p) {
     for (int c = 0; c < ngroups; ++c) {
       const unsigned on = (unsigned)(vv >> (4 * c)) & 15u;
       int4 pv = make_int4(-1, -1, -1, -1);
-      if (on) pv = __ldg(row + c);
+      if (on) pv = __ldcg(row + c);  // this launch wrote the rows, so not __ldg; used once, so from L2
       unsigned lb[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) lb[q] = 0;
