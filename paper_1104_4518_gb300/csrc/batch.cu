@@ -337,7 +337,8 @@ __device__ __forceinline__ void pull_chunk(const BatchParams& p, const Word* Fc,
     const Bits old = atomic_or_word(&Fn[v], found);
     if (old == 0) {
       claimed = true;
-      push_chunks_cta(p, knext, cl, v, __ldg(&p.off[v + 1]) - __ldg(&p.off[v]));
+      const long long dout = __ldg(&p.off[v + 1]) - __ldg(&p.off[v]);  // (a directed graph's out-row may be short)
+      if (dout > kChunkEdges) push_chunks_cta(p, knext, cl, v, dout);
     }
   }
   warp_enqueue(p, knext, wq, nbuf, claimed, v, lane, false);
