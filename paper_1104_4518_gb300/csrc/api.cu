@@ -246,9 +246,10 @@ int get_workspace(bfs_graph* g, cudaStream_t s, Workspace** out) {
     if (e != cudaSuccess) rc = cuda_fail(e, "pinned staging");
   }
   if (!rc) {
-    cudaError_t e = cudaMemset(w->barrier, 0, 2 * sizeof(bfsdev::GridBarrier));
-    if (e == cudaSuccess) e = cudaMemset(w->status, 0, sizeof(int) * 4);
-    if (e == cudaSuccess) e = cudaMemset(w->ctr, 0, sizeof(LevelCtr) * kCtrRing);
+    // on s: a non-blocking stream would not wait for fills on the default stream
+    cudaError_t e = cudaMemsetAsync(w->barrier, 0, 2 * sizeof(bfsdev::GridBarrier), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w->status, 0, sizeof(int) * 4, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w->ctr, 0, sizeof(LevelCtr) * kCtrRing, s);
     if (e != cudaSuccess) rc = cuda_fail(e, "workspace initialisation");
   }
   if (rc) {
@@ -340,8 +341,8 @@ static int read_status(Workspace* w, cudaStream_t s) {
   e = cudaMemcpy(st, w->status, sizeof(st), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "status read");
   if (st[0] != 0) {
-    cudaMemset(w->status, 0, sizeof(st));
-    cudaMemset(w->barrier, 0, 2 * sizeof(bfsdev::GridBarrier));
+    cudaMemsetAsync(w->status, 0, sizeof(st), s);  // before the next traversal on s
+    cudaMemsetAsync(w->barrier, 0, 2 * sizeof(bfsdev::GridBarrier), s);
     w->bar_grid[0] = w->bar_grid[1] = 0;
     return fail(st[0], device_status_message(st));
   }
@@ -588,7 +589,8 @@ int bfs_graph_union(bfs_graph* const* graphs, int32_t count, void* stream, bfs_g
     bfs_graph_destroy(u);
     return e;
   }
-  cudaError_t err = cudaMemcpy(u->d_part_base, base.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice);
+  cudaError_t err = cudaMemcpyAsync(u->d_part_base, base.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice, s);
+  if (err == cudaSuccess) err = cudaStreamSynchronize(s);
   if (err != cudaSuccess) {
     bfs_graph_destroy(u);
     return cuda_fail(err, "part table copy");
@@ -856,9 +858,9 @@ int bfs_run_ragged(bfs_graph* u, const int32_t* sources, int32_t* const* parent_
   if (!w->part_out) {
     if (int e = dev_alloc((void**)&w->part_out, sizeof(int32_t*) * 2 * parts, "part output table")) return e;
   }
-  // the pointer table changes rarely; it is copied synchronously
+  // the pointer table changes rarely; the call waits for its copy, which is on s as the traversal after it is
+  BFS_CUDA_TRY(cudaMemcpyAsync(w->part_out, table.data(), sizeof(int32_t*) * 2 * parts, cudaMemcpyHostToDevice, s));
   BFS_CUDA_TRY(cudaStreamSynchronize(s));
-  BFS_CUDA_TRY(cudaMemcpy(w->part_out, table.data(), sizeof(int32_t*) * 2 * parts, cudaMemcpyHostToDevice));
   RunRequest r;
   r.g = u;
   r.w = w;

@@ -1386,7 +1386,7 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
   p.forced = r.forced;
   p.schedule = w->schedule;
   p.schedule_len = sched_len;
-  p.mlp = r.selector == BFS_SELECT_LEARNED ? learned_params_device() : nullptr;
+  p.mlp = r.selector == BFS_SELECT_LEARNED ? learned_params_device(s) : nullptr;
   graph_feature_constants(g->n, g->nnz, &p.feat_log_n, &p.feat_log_nnz, &p.feat_inv_n, &p.feat_inv_nnz);
   p.want_stats = r.want_stats ? 1 : 0;
   p.spin_limit = r.spin_limit ? r.spin_limit : (1u << 25);

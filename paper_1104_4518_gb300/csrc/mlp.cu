@@ -355,7 +355,7 @@ std::vector<float*> g_sel_dev;  // per device ordinal
 
 }  // namespace
 
-const float* learned_params_device() {
+const float* learned_params_device(cudaStream_t s) {
   std::lock_guard<std::mutex> lk(g_sel_mu);
   if (g_sel_host.empty()) return nullptr;
   int dev = 0;
@@ -366,7 +366,9 @@ const float* learned_params_device() {
     for (int i = 0; i < BFS_MLP_PARAMS; ++i) warp[bfsdev::warp_layout_index(i)] = g_sel_host[i];
     float* p = nullptr;
     if (cudaMalloc(&p, sizeof(float) * BFS_MLP_PARAMS) != cudaSuccess) return nullptr;
-    if (cudaMemcpy(p, warp.data(), sizeof(float) * BFS_MLP_PARAMS, cudaMemcpyHostToDevice) != cudaSuccess) {
+    // there before any stream reads them: a pageable copy may still be on its way when the call returns
+    if (cudaMemcpyAsync(p, warp.data(), sizeof(float) * BFS_MLP_PARAMS, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess) {
       cudaFree(p);
       return nullptr;
     }

@@ -47,7 +47,7 @@ unsigned char* g_addr[64] = {nullptr};  // device address of g_static_scratch, p
 
 // Set-up on the first call on a device (that device current): look up the
 // array's device address and clear the barrier and status words.
-int scratch_address(unsigned char** out) {
+int scratch_address(unsigned char** out, cudaStream_t s) {
   int dev = 0;
   BFS_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return fail(BFS_ERR_UNSUPPORTED, "bfs_run_static: device ordinal out of range");
@@ -56,7 +56,8 @@ int scratch_address(unsigned char** out) {
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_static_scratch);
     if (e != cudaSuccess) return cuda_fail(e, "bfs_run_static: cudaGetSymbolAddress of the static scratch");
-    e = cudaMemset(static_cast<unsigned char*>(p) + kOffBarrier, 0, kBarrierBytes + kSmallBytes);
+    e = cudaMemsetAsync(static_cast<unsigned char*>(p) + kOffBarrier, 0, kBarrierBytes + kSmallBytes, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "bfs_run_static: clearing the static scratch");
     g_addr[dev] = static_cast<unsigned char*>(p);
   }
@@ -80,8 +81,8 @@ extern "C" int bfs_run_static(const int64_t* offsets, const int32_t* adj, int32_
     return fail(BFS_ERR_INVALID_ARG, "bfs_run_static: NULL pointer");
   if (source < 0 || source >= n) return fail(BFS_ERR_INVALID_ARG, "bfs_run_static: source outside [0, n)");
   unsigned char* base = nullptr;
-  if (int e = scratch_address(&base)) return e;
   cudaStream_t s = (cudaStream_t)stream;
+  if (int e = scratch_address(&base, s)) return e;
   if (bfsdev::kBoundsCheck) {  // the caller's rows must lie inside [0, nnz) before the kernel trusts them
     int ok = 0;
     if (int e = check_offsets(offsets, n, nnz, reinterpret_cast<int*>(base + kOffSmall + 192), s, &ok)) return e;
