@@ -269,37 +269,39 @@ static int stage0_ready(Workspace* w, cudaStream_t s) {
   return BFS_OK;
 }
 
+// Device memory for *p unless it is there already: a buffer set whose allocation
+// failed half way is completed by the next call.
+template <typename T>
+static int alloc_once(T** p, size_t bytes, const char* what) {
+  return *p ? BFS_OK : dev_alloc((void**)p, bytes, what);
+}
+
 int ensure_tmp_outputs(bfs_graph* g, Workspace* w) {
-  if (w->tmp_level) return BFS_OK;
   const size_t nq = sizeof(int32_t) * (size_t)g->n;
-  if (int e = dev_alloc((void**)&w->tmp_level, nq, "union-space levels")) return e;
-  if (int e = dev_alloc((void**)&w->tmp_parent, nq, "union-space parents")) return e;
-  return BFS_OK;
+  if (int e = alloc_once(&w->tmp_level, nq, "union-space levels")) return e;
+  return alloc_once(&w->tmp_parent, nq, "union-space parents");
 }
 
 int ensure_async_outputs(bfs_graph* g, Workspace* w) {
   if (int e = ensure_tmp_outputs(g, w)) return e;
-  if (w->copy_stream) return BFS_OK;
+  if (w->copy_stream) return BFS_OK;  // (made last)
   const size_t nq = sizeof(int32_t) * (size_t)g->n;
-  if (int e = dev_alloc((void**)&w->tmp2_level, nq, "second staging levels")) return e;
-  if (int e = dev_alloc((void**)&w->tmp2_parent, nq, "second staging parents")) return e;
+  if (int e = alloc_once(&w->tmp2_level, nq, "second staging levels")) return e;
+  if (int e = alloc_once(&w->tmp2_parent, nq, "second staging parents")) return e;
   for (int i = 0; i < 2; ++i) {
-    BFS_CUDA_TRY(cudaEventCreateWithFlags(&w->staged_ev[i], cudaEventDisableTiming));
-    BFS_CUDA_TRY(cudaEventCreateWithFlags(&w->copied_ev[i], cudaEventDisableTiming));
+    if (!w->staged_ev[i]) BFS_CUDA_TRY(cudaEventCreateWithFlags(&w->staged_ev[i], cudaEventDisableTiming));
+    if (!w->copied_ev[i]) BFS_CUDA_TRY(cudaEventCreateWithFlags(&w->copied_ev[i], cudaEventDisableTiming));
   }
   BFS_CUDA_TRY(cudaStreamCreateWithFlags(&w->copy_stream, cudaStreamNonBlocking));
   return BFS_OK;
 }
 
 int ensure_batch_state(bfs_graph* g, Workspace* w) {
-  if (w->bset[0]) return BFS_OK;
   const size_t n8 = sizeof(uint64_t) * (size_t)g->n;
   for (int i = 0; i < 3; ++i)
-    if (int e = dev_alloc((void**)&w->bset[i], n8, "batch frontier bitsets")) return e;
-  if (int e = dev_alloc((void**)&w->bvis, n8, "batch visited bitsets")) return e;
-  if (int e = dev_alloc((void**)&w->bscr, sizeof(int32_t) * 2 * 64 * (size_t)g->n, "batch scratch results"))
-    return e;
-  return BFS_OK;
+    if (int e = alloc_once(&w->bset[i], n8, "batch frontier bitsets")) return e;
+  if (int e = alloc_once(&w->bvis, n8, "batch visited bitsets")) return e;
+  return alloc_once(&w->bscr, sizeof(int32_t) * 2 * 64 * (size_t)g->n, "batch scratch results");
 }
 
 int prepare_barrier(Workspace* w, int kind, int grid, cudaStream_t s, bfsdev::GridBarrier** out) {

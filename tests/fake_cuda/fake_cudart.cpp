@@ -25,8 +25,9 @@ struct Entry {
 std::recursive_mutex mu;
 std::vector<Entry> entries;
 std::map<void*, size_t> live;
-size_t live_bytes = 0, total_bytes = (size_t)64 << 30;
-long long fail_malloc_in = -1;  // 0: the next allocation fails
+size_t live_bytes = 0, total_bytes = (size_t)64 << 30;  // in use; the device's memory
+size_t reported_total = (size_t)64 << 30;                       // what cudaMemGetInfo says of it
+long long mallocs_left = -1;  // allocations that still succeed (negative: all)
 cudaError_t sync_error = cudaSuccess;
 int device = 0;
 unsigned long long context = 1;
@@ -46,11 +47,11 @@ FAKE const char* fake_log_entry(int i, const void** p, size_t* bytes, void** str
   return entries[i].what;
 }
 FAKE void fake_log_clear() { entries.clear(); }
-FAKE void fake_fail_malloc_in(long long n) { fail_malloc_in = n; }
+FAKE void fake_set_mallocs_left(long long n) { mallocs_left = n; }
 FAKE void fake_sync_error(int e) { sync_error = (cudaError_t)e; }
 FAKE void fake_set_device(int d) { device = d; }
 FAKE void fake_set_context(unsigned long long id) { context = id; }
-FAKE void fake_set_total(size_t b) { total_bytes = b; }
+FAKE void fake_set_reported_total(size_t b) { reported_total = b; }
 FAKE size_t fake_live_bytes() { return live_bytes; }
 FAKE int fake_is_live(void* p) { return live.count(p) != 0; }
 
@@ -59,12 +60,11 @@ FAKE int fake_is_live(void* p) { return live.count(p) != 0; }
 CUDA cudaMalloc(void** p, size_t bytes) {
   std::lock_guard<std::recursive_mutex> lk(mu);
   *p = nullptr;
-  if (fail_malloc_in == 0 || live_bytes + bytes > total_bytes) {
-    if (fail_malloc_in == 0) fail_malloc_in = -1;
+  if (mallocs_left == 0 || live_bytes + bytes > total_bytes) {
     note("malloc failed", nullptr, bytes);
     return cudaErrorMemoryAllocation;
   }
-  if (fail_malloc_in > 0) --fail_malloc_in;
+  if (mallocs_left > 0) --mallocs_left;
   void* m = mmap(nullptr, bytes, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
   if (m == MAP_FAILED) return cudaErrorMemoryAllocation;
   memset(m, 0xa5, bytes < 4096 ? bytes : 4096);
@@ -87,13 +87,21 @@ CUDA cudaFree(void* p) {
 }
 CUDA cudaMallocHost(void** p, size_t bytes) { return (*p = malloc(bytes)) ? cudaSuccess : cudaErrorMemoryAllocation; }
 CUDA cudaFreeHost(void* p) { return free(p), cudaSuccess; }
-CUDA cudaMemGetInfo(size_t* f, size_t* t) { return *f = total_bytes - live_bytes, *t = total_bytes, cudaSuccess; }
-CUDA cudaMemset(void* p, int v, size_t n) { return memset(p, v, n), note("memset", p, n), cudaSuccess; }
-CUDA cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t s) { return memset(p, v, n), note("memset", p, n, s), cudaSuccess; }
-CUDA cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { return memcpy(d, s, n), note("memcpy", d, n), cudaSuccess; }
-CUDA cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t st) {
-  return memcpy(d, s, n), note("memcpy", d, n, st), cudaSuccess;
+CUDA cudaMemGetInfo(size_t* f, size_t* t) { return *f = total_bytes - live_bytes, *t = reported_total, cudaSuccess; }
+namespace {
+cudaError_t fill(void* p, int v, size_t n, void* s) {
+  if (n && !p) return note("memset failed", p, n, s), cudaErrorInvalidValue;
+  return memset(p, v, n), note("memset", p, n, s), cudaSuccess;
 }
+cudaError_t copy(void* d, const void* from, size_t n, void* s) {
+  if (n && (!d || !from)) return note("memcpy failed", d, n, s), cudaErrorInvalidValue;
+  return memcpy(d, from, n), note("memcpy", d, n, s), cudaSuccess;
+}
+}  // namespace
+CUDA cudaMemset(void* p, int v, size_t n) { return fill(p, v, n, nullptr); }
+CUDA cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t s) { return fill(p, v, n, s); }
+CUDA cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { return copy(d, s, n, nullptr); }
+CUDA cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t st) { return copy(d, s, n, st); }
 CUDA cudaDeviceSynchronize() { return note("device sync"), sync_error; }
 CUDA cudaStreamSynchronize(cudaStream_t s) { return note("stream sync", nullptr, 0, s), cudaSuccess; }
 CUDA cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return *s = (cudaStream_t)malloc(1), cudaSuccess; }
