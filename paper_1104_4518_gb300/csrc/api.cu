@@ -40,7 +40,8 @@ int cuda_fail(cudaError_t e, const char* what) {
 // cost more than its kernels (2.2 GB of sort keys: 0.6 ms to allocate, 1.0 ms to
 // free; at scale 16 some 0.4 ms of calls around 0.13 ms of kernels).
 //   - dev_free waits for the device, as cudaFree does, so a cached block is idle
-//     and any stream and thread may have it next;
+//     and any stream and thread may have it next (a block whose wait failed, or
+//     whose device is not the current one, goes to cudaFree);
 //   - the cache of a device holds at most 1/64 of its memory, and a block only
 //     serves requests that use four fifths of it (or all but 1 MB);
 //   - a block that has waited for more than a second goes back to the driver at
@@ -134,7 +135,7 @@ int dev_alloc(void** p, size_t bytes, const char* what) {
 void dev_free(void* p) {
   if (!p) return;
   bool keep = false;
-  cudaDeviceSynchronize();
+  const bool idle = cudaDeviceSynchronize() == cudaSuccess;  // (it fails during another thread's stream capture)
   {
     std::lock_guard<std::mutex> lk(g_mem_mu);
     auto it = g_mem_size.find(p);
@@ -144,7 +145,7 @@ void dev_free(void* p) {
       size_t held = bytes;
       for (const CachedBlock& c : g_mem_idle) held += c.device == dev ? c.bytes : 0;
       int cur = -1;
-      keep = cudaGetDevice(&cur) == cudaSuccess && cur == dev && held <= cache_limit(dev);
+      keep = idle && cudaGetDevice(&cur) == cudaSuccess && cur == dev && held <= cache_limit(dev);
       if (keep) g_mem_idle.push_back({p, bytes, dev, std::chrono::steady_clock::now()});
     }
   }
