@@ -45,8 +45,8 @@ int cuda_fail(cudaError_t e, const char* what) {
 //   - the cache of a device holds at most 1/64 of its memory, and a block only
 //     serves requests that use four fifths of it (or all but 1 MB);
 //   - a block that has waited for more than a second goes back to the driver at
-//     the library's next allocation, release or bfs_sync, and all of them do when
-//     an allocation fails.
+//     the library's next allocation or release, and all of them do when an
+//     allocation fails.
 namespace {
 struct CachedBlock {
   void* p;
@@ -881,7 +881,6 @@ int bfs_run_ragged(bfs_graph* u, const int32_t* sources, int32_t* const* parent_
 
 int bfs_sync(bfs_graph* g, void* stream) {
   NvtxRange nvtx_range("bfs_sync");
-  trim_device_cache();
   if (int e = check_graph(g)) return e;
   cudaStream_t s = (cudaStream_t)stream;
   Workspace* w = nullptr;
