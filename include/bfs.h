@@ -214,8 +214,17 @@ BFS_API int bfs_graph_csr(const bfs_graph* g, const int64_t** offsets, const int
  * adj_out int32[nnz] (device memory, or host with BFS_HOST_PTRS).  Synchronous. */
 BFS_API int bfs_graph_copy_csr(const bfs_graph* g, int64_t* offsets_out, int32_t* adj_out, uint32_t flags);
 
-/* Frees the graph and every workspace created for it.  Synchronises the device. */
+/* Releases the graph and every workspace created for it.  Synchronises the device.
+ * Released device memory stays in a cache of the library for its next calls: at
+ * most 1/64 of the device's memory.  A block that has been there for more than a
+ * second goes back to the driver at the library's next allocation or release;
+ * while no such call follows it stays, until bfs_memory_trim. */
 BFS_API void bfs_graph_destroy(bfs_graph* g);
+
+/* Gives all device memory that the library holds unused, on every device, back
+ * to the driver (cudaFree, which waits for the device).  For a process that is
+ * done with its graphs, or that wants the memory elsewhere. */
+BFS_API int bfs_memory_trim(void);
 
 /*
  * One BFS from `source` (Algorithm 3 on one GPU): writes level_out and

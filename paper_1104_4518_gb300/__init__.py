@@ -140,6 +140,7 @@ def _declare(lib):
         "bfs_selector_save": [ctypes.c_char_p],
         "bfs_level_features": [i32, i64, i32, i64, i64, i64, i64, ctypes.POINTER(i64), ctypes.POINTER(f32)],
         "bfs_bounds_checked": [],
+        "bfs_memory_trim": [],
     }
     for name, args in sig.items():
         fn = getattr(lib, name)
@@ -489,6 +490,11 @@ def bfs_run_static(offsets, adj, source: int, parent_out, level_out, stream=None
 def bfs_sync(g: Graph, stream=None):
     """Waits for the stream; raises the device status of the last run on it."""
     _check(lib().bfs_sync(g.handle, _stream_handle(stream)))
+
+
+def bfs_memory_trim():
+    """Gives the device memory that the library holds unused back to the driver."""
+    _check(lib().bfs_memory_trim())
 
 
 def bfs_set_tuning(g: Graph, **knobs):

@@ -46,7 +46,7 @@ int cuda_fail(cudaError_t e, const char* what) {
 //     serves requests that use four fifths of it (or all but 1 MB);
 //   - a block that has waited for more than a second goes back to the driver at
 //     the library's next allocation or release, and all of them do when an
-//     allocation fails.
+//     allocation fails or the caller asks for it (bfs_memory_trim).
 namespace {
 struct CachedBlock {
   void* p;
@@ -86,11 +86,12 @@ std::vector<void*> take_idle(int device, std::chrono::steady_clock::duration age
   }
   return out;
 }
-}  // namespace
 
+// Gives the cached blocks that nothing has asked for lately back to the driver.
 void trim_device_cache() {
   for (void* p : take_idle(-1, std::chrono::seconds(1))) cudaFree(p);
 }
+}  // namespace
 
 int dev_alloc(void** p, size_t bytes, const char* what) {
   *p = nullptr;
@@ -644,6 +645,16 @@ void bfs_graph_destroy(bfs_graph* g) {
   free_tiles(g->tiles);
   free_half(g);
   delete g;
+}
+
+int bfs_memory_trim(void) {
+  NvtxRange nvtx_range("bfs_memory_trim");
+  cudaError_t err = cudaSuccess;
+  for (void* p : take_idle(-1, std::chrono::steady_clock::duration::zero())) {
+    const cudaError_t e = cudaFree(p);
+    if (e != cudaSuccess) err = e;
+  }
+  return err == cudaSuccess ? BFS_OK : cuda_fail(err, "bfs_memory_trim");
 }
 
 int bfs_graph_tiles(bfs_graph* g, int32_t rb_bits, int32_t cb_bits, bfs_tile_info* info, void* stream) {

@@ -31,8 +31,6 @@ int cuda_fail(cudaError_t e, const char* what);
 int dev_alloc(void** p, size_t bytes, const char* what);
 // Waits for the device, then releases a block (null: nothing) to the library's cache or to the driver.
 void dev_free(void* p);
-// Gives the cached blocks that nothing has asked for lately back to the driver.
-void trim_device_cache();
 
 // ---------------- device properties ----------------
 struct DeviceInfo {

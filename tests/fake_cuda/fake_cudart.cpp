@@ -31,7 +31,7 @@ long long mallocs_left = -1;  // allocations that still succeed (negative: all)
 cudaError_t sync_error = cudaSuccess;
 int device = 0;
 unsigned long long context = 1;
-struct { dim3 grid, block; size_t smem; void* stream; } config;
+thread_local struct { dim3 grid, block; size_t smem; void* stream; } config;
 
 void note(const char* what, const void* p = nullptr, size_t bytes = 0, void* stream = nullptr) {
   std::lock_guard<std::recursive_mutex> lk(mu);
@@ -51,9 +51,12 @@ FAKE void fake_set_mallocs_left(long long n) { mallocs_left = n; }
 FAKE void fake_sync_error(int e) { sync_error = (cudaError_t)e; }
 FAKE void fake_set_device(int d) { device = d; }
 FAKE void fake_set_context(unsigned long long id) { context = id; }
+FAKE void fake_set_total(size_t b) { total_bytes = b; }
 FAKE void fake_set_reported_total(size_t b) { reported_total = b; }
-FAKE size_t fake_live_bytes() { return live_bytes; }
-FAKE int fake_is_live(void* p) { return live.count(p) != 0; }
+FAKE size_t fake_live_bytes() {
+  std::lock_guard<std::recursive_mutex> lk(mu);
+  return live_bytes;
+}
 
 #define CUDA extern "C" __attribute__((visibility("default"))) cudaError_t
 

@@ -46,3 +46,101 @@ def test_waiting_for_a_stream_frees_nothing(lib):
     log = lib.taken(lambda: lib.c.bfs_sync(g, ctypes.c_void_p(0x5150)))
     assert "stream sync" in whats(log)
     assert not {"free", "device sync"} & set(whats(log))
+
+
+def test_bound(lib):
+    """At most 1/64 of the device's memory is kept."""
+    lib.c.fake_set_reported_total(ctypes.c_size_t(64 * 10000))
+    log = lib.taken(lambda: cycle(lib))
+    assert "free" in whats(log)
+    assert 0 < lib.c.fake_live_bytes() <= 10000
+
+
+def test_blocks_go_back_after_a_second_and_on_request(lib):
+    cycle(lib)
+    assert lib.c.fake_live_bytes() > 0
+    time.sleep(1.1)
+    lib.c.bfs_graph_destroy(lib.graph(3))
+    assert lib.c.fake_live_bytes() <= 16 * 512  # what the small graph left
+    cycle(lib)
+    assert lib.c.bfs_memory_trim() == 0
+    assert lib.c.fake_live_bytes() == 0
+    lib.c.fake_set_device(1)  # blocks of any device
+    cycle(lib)
+    lib.c.fake_set_device(0)
+    cycle(lib)
+    assert lib.c.bfs_memory_trim() == 0
+    assert lib.c.fake_live_bytes() == 0
+
+
+def test_request_leaves_blocks_in_use_alone(lib):
+    g = lib.graph(N)
+    cycle(lib)
+    used = lib.c.fake_live_bytes()
+    assert lib.c.bfs_memory_trim() == 0
+    assert 0 < lib.c.fake_live_bytes() < used
+    assert lib.run(g, N) == 0 and lib.c.bfs_sync(g, None) == 0
+
+
+def test_a_failed_allocation_takes_the_idle_blocks_first(lib):
+    cycle(lib, 20 * N)
+    assert lib.c.fake_live_bytes() > 300000
+    lib.c.fake_set_total(ctypes.c_size_t(700000))  # not for both graphs
+    g = None
+
+    def create():
+        nonlocal g
+        g = lib.graph(40 * N)
+    log = whats(lib.taken(create))
+    at = log.index("malloc failed")
+    assert log[at + 1] == "free" and "malloc" in log[at:]
+
+
+def test_release_with_another_device_current(lib):
+    """A block of another device is not idle after a wait for the current one; and a device gets its own blocks only."""
+    g = lib.graph(N)
+    lib.c.fake_set_device(1)
+    before = lib.c.fake_live_bytes()
+    lib.c.bfs_graph_destroy(g)
+    assert lib.c.fake_live_bytes() < before
+    lib.c.fake_set_device(0)
+    cycle(lib)
+    lib.c.fake_set_device(1)
+    kept = lib.c.fake_live_bytes()
+    g = lib.graph(N)
+    assert lib.c.fake_live_bytes() > kept
+    lib.c.bfs_graph_destroy(g)
+
+
+def test_two_threads(lib):
+    """Graphs made, run and destroyed by two threads at once: no block has two owners."""
+    owned, mu, bad = set(), threading.Lock(), []
+
+    def work(seed):
+        n = 50 + seed
+        for i in range(200):
+            g = lib.graph(n)
+            off, adj = ctypes.c_void_p(), ctypes.c_void_p()
+            lib.c.bfs_graph_csr(g, ctypes.byref(off), ctypes.byref(adj))
+            with mu:
+                if off.value in owned or adj.value in owned:
+                    bad.append((seed, i))
+                owned.update((off.value, adj.value))
+            ok = lib.run(g, n, 0x1000 + seed) == 0 and lib.c.bfs_sync(g, ctypes.c_void_p(0x1000 + seed)) == 0
+            rows = (ctypes.c_int64 * (n + 1)).from_address(off.value)
+            if not ok or rows[n] != 2 * (n - 1) or rows[1] != 1:
+                bad.append((seed, i))
+            with mu:
+                owned.difference_update((off.value, adj.value))
+            lib.c.bfs_graph_destroy(g)
+            if i % 50 == 49:
+                lib.c.bfs_memory_trim()
+
+    threads = [threading.Thread(target=work, args=(s,)) for s in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
+    assert lib.c.bfs_memory_trim() == 0
+    assert lib.c.fake_live_bytes() == 0
