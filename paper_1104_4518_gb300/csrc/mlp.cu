@@ -365,11 +365,11 @@ const float* learned_params_device(cudaStream_t s) {
     std::vector<float> warp(BFS_MLP_PARAMS);
     for (int i = 0; i < BFS_MLP_PARAMS; ++i) warp[bfsdev::warp_layout_index(i)] = g_sel_host[i];
     float* p = nullptr;
-    if (cudaMalloc(&p, sizeof(float) * BFS_MLP_PARAMS) != cudaSuccess) return nullptr;
+    if (dev_alloc((void**)&p, sizeof(float) * BFS_MLP_PARAMS, "selector parameters") != BFS_OK) return nullptr;
     // there before any stream reads them: a pageable copy may still be on its way when the call returns
     if (cudaMemcpyAsync(p, warp.data(), sizeof(float) * BFS_MLP_PARAMS, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
-      cudaFree(p);
+      dev_free(p);
       return nullptr;
     }
     g_sel_dev[dev] = p;

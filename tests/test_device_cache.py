@@ -144,3 +144,16 @@ def test_two_threads(lib):
     assert not bad
     assert lib.c.bfs_memory_trim() == 0
     assert lib.c.fake_live_bytes() == 0
+
+
+def test_the_selectors_parameters_may_take_an_idle_block(lib):
+    """With no memory left but what the library holds unused, a learned run still runs the network."""
+    import paper_1104_4518_gb300 as bfs
+    g = lib.graph(N)
+    assert lib.run(g, N) == 0
+    cycle(lib, 20 * N)
+    lib.c.fake_set_total(ctypes.c_size_t(lib.c.fake_live_bytes()))
+    assert lib.c.bfs_selector_set_params((ctypes.c_float * bfs.BFS_MLP_PARAMS)()) == 0
+    o = bfs.bfs_opts(selector=bfs.BFS_SELECT_LEARNED)
+    log = lib.taken(lambda: lib.run(g, N, 0, ctypes.byref(o)))
+    assert [e for e in log if e.what == "memcpy" and e.bytes == 4 * bfs.BFS_MLP_PARAMS]
