@@ -42,21 +42,40 @@ int cuda_fail(cudaError_t e, const char* what) {
 //   - dev_free waits for the device, as cudaFree does, so a cached block is idle
 //     and any stream and thread may have it next (a block whose wait failed, or
 //     whose device is not the current one, goes to cudaFree);
+//   - a block belongs to the context it was allocated in: cudaDeviceReset frees
+//     them all, and those of a context that is no longer the device's are forgotten;
 //   - the cache of a device holds at most 1/64 of its memory, and a block only
 //     serves requests that use four fifths of it (or all but 1 MB);
 //   - a block that has waited for more than a second goes back to the driver at
 //     the library's next allocation or release, and all of them do when an
 //     allocation fails or the caller asks for it (bfs_memory_trim).
 namespace {
-struct CachedBlock {
-  void* p;
+struct Block {
   size_t bytes;
   int device;
+  unsigned long long context;
+};
+struct CachedBlock : Block {
+  void* p;
   std::chrono::steady_clock::time_point since;
 };
 std::mutex g_mem_mu;
-std::unordered_map<void*, std::pair<size_t, int>> g_mem_size;  // blocks in use: size, device
+std::unordered_map<void*, Block> g_mem_used;
 std::vector<CachedBlock> g_mem_idle;
+
+// Identity of the calling thread's current context, never used twice in a process; 0: none, or not known.
+unsigned long long current_context() {
+  using GetId = int (*)(void*, unsigned long long*);  // cuCtxGetId
+  static const GetId get_id = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &found);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? (GetId)f : nullptr;
+  }();
+  unsigned long long id = 0;
+  return get_id && get_id(nullptr, &id) == 0 ? id : 0;
+}
 
 size_t cache_limit(int device) {
   static size_t limit[64] = {};  // under g_mem_mu
@@ -69,15 +88,19 @@ size_t cache_limit(int device) {
   return limit[device];
 }
 
-// Takes the cached blocks of `device` (all devices: -1) that have been idle for longer than `age` out of the cache.
-std::vector<void*> take_idle(int device, std::chrono::steady_clock::duration age) {
+// Takes the current device's cached blocks that have been idle for longer than `age` out of the cache.
+std::vector<void*> take_idle(std::chrono::steady_clock::duration age) {
   std::vector<void*> out;
   const auto now = std::chrono::steady_clock::now();
+  const unsigned long long context = current_context();
+  int device = -1;
+  if (context == 0 || cudaGetDevice(&device) != cudaSuccess) return out;
   std::lock_guard<std::mutex> lk(g_mem_mu);
   for (size_t i = 0; i < g_mem_idle.size();) {
     CachedBlock& c = g_mem_idle[i];
-    if ((device < 0 || c.device == device) && now - c.since >= age) {
-      out.push_back(c.p);
+    const bool stale = c.context != context;  // freed by cudaDeviceReset
+    if (c.device == device && (stale || now - c.since >= age)) {
+      if (!stale) out.push_back(c.p);
       c = g_mem_idle.back();
       g_mem_idle.pop_back();
     } else {
@@ -89,7 +112,7 @@ std::vector<void*> take_idle(int device, std::chrono::steady_clock::duration age
 
 // Gives the cached blocks that nothing has asked for lately back to the driver.
 void trim_device_cache() {
-  for (void* p : take_idle(-1, std::chrono::seconds(1))) cudaFree(p);
+  for (void* p : take_idle(std::chrono::seconds(1))) cudaFree(p);
 }
 }  // namespace
 
@@ -99,17 +122,18 @@ int dev_alloc(void** p, size_t bytes, const char* what) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
   trim_device_cache();
+  const unsigned long long context = current_context();
   {
     std::lock_guard<std::mutex> lk(g_mem_mu);
     size_t best = g_mem_idle.size();
     for (size_t i = 0; i < g_mem_idle.size(); ++i) {
       const CachedBlock& c = g_mem_idle[i];
-      if (c.device != dev || c.bytes < need || c.bytes > need + std::max(need / 4, (size_t)1 << 20)) continue;
+      if (c.device != dev || c.context != context || c.bytes < need || c.bytes > need + std::max(need / 4, (size_t)1 << 20)) continue;
       if (best == g_mem_idle.size() || c.bytes < g_mem_idle[best].bytes) best = i;
     }
     if (best < g_mem_idle.size()) {
       *p = g_mem_idle[best].p;
-      g_mem_size[*p] = {g_mem_idle[best].bytes, dev};
+      g_mem_used[*p] = g_mem_idle[best];
       g_mem_idle[best] = g_mem_idle.back();
       g_mem_idle.pop_back();
       return BFS_OK;
@@ -118,7 +142,7 @@ int dev_alloc(void** p, size_t bytes, const char* what) {
   cudaError_t e = cudaMalloc(p, need);
   if (e == cudaErrorMemoryAllocation) {  // give back what the cache holds and try once more
     cudaGetLastError();
-    for (void* q : take_idle(dev, std::chrono::steady_clock::duration::zero())) cudaFree(q);
+    for (void* q : take_idle(std::chrono::steady_clock::duration::zero())) cudaFree(q);
     e = cudaMalloc(p, need);
   }
   if (e != cudaSuccess) {
@@ -128,8 +152,9 @@ int dev_alloc(void** p, size_t bytes, const char* what) {
                 std::string("device allocation of ") + std::to_string(bytes) + " bytes for " + what + " failed: " +
                     cudaGetErrorString(e));
   }
+  const Block b{need, dev, current_context()};  // (the process's first allocation made the context)
   std::lock_guard<std::mutex> lk(g_mem_mu);
-  g_mem_size[*p] = {need, dev};
+  g_mem_used[*p] = b;
   return BFS_OK;
 }
 
@@ -137,17 +162,19 @@ void dev_free(void* p) {
   if (!p) return;
   bool keep = false;
   const bool idle = cudaDeviceSynchronize() == cudaSuccess;  // (it fails during another thread's stream capture)
+  const unsigned long long context = current_context();
   {
     std::lock_guard<std::mutex> lk(g_mem_mu);
-    auto it = g_mem_size.find(p);
-    if (it != g_mem_size.end()) {
-      const auto [bytes, dev] = it->second;
-      g_mem_size.erase(it);
-      size_t held = bytes;
-      for (const CachedBlock& c : g_mem_idle) held += c.device == dev ? c.bytes : 0;
+    auto it = g_mem_used.find(p);
+    if (it != g_mem_used.end()) {
+      const Block b = it->second;
+      g_mem_used.erase(it);
+      size_t held = b.bytes;
+      for (const CachedBlock& c : g_mem_idle) held += c.device == b.device ? c.bytes : 0;
       int cur = -1;
-      keep = idle && cudaGetDevice(&cur) == cudaSuccess && cur == dev && held <= cache_limit(dev);
-      if (keep) g_mem_idle.push_back({p, bytes, dev, std::chrono::steady_clock::now()});
+      keep = idle && cudaGetDevice(&cur) == cudaSuccess && cur == b.device && context != 0 && context == b.context &&
+             held <= cache_limit(b.device);
+      if (keep) g_mem_idle.push_back({b, p, std::chrono::steady_clock::now()});
     }
   }
   if (!keep) cudaFree(p);
@@ -649,11 +676,23 @@ void bfs_graph_destroy(bfs_graph* g) {
 
 int bfs_memory_trim(void) {
   NvtxRange nvtx_range("bfs_memory_trim");
+  std::vector<int> devices;
+  {
+    std::lock_guard<std::mutex> lk(g_mem_mu);
+    for (const CachedBlock& c : g_mem_idle)
+      if (std::find(devices.begin(), devices.end(), c.device) == devices.end()) devices.push_back(c.device);
+  }
+  int current = 0;
+  BFS_CUDA_TRY(cudaGetDevice(&current));
   cudaError_t err = cudaSuccess;
-  for (void* p : take_idle(-1, std::chrono::steady_clock::duration::zero())) {
-    const cudaError_t e = cudaFree(p);
+  for (int d : devices) {
+    cudaError_t e = cudaSetDevice(d);
+    if (e == cudaSuccess)
+      for (void* p : take_idle(std::chrono::steady_clock::duration::zero()))
+        if (cudaError_t f = cudaFree(p); f != cudaSuccess) e = f;
     if (e != cudaSuccess) err = e;
   }
+  if (!devices.empty() && cudaSetDevice(current) != cudaSuccess && err == cudaSuccess) err = cudaErrorInvalidDevice;
   return err == cudaSuccess ? BFS_OK : cuda_fail(err, "bfs_memory_trim");
 }
 

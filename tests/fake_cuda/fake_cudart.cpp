@@ -117,6 +117,7 @@ CUDA cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 CUDA cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 CUDA cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { return *ms = 1.0f, cudaSuccess; }
 CUDA cudaGetDevice(int* d) { return *d = device, cudaSuccess; }
+CUDA cudaSetDevice(int d) { return device = d, cudaSuccess; }
 CUDA cudaGetLastError() { return cudaSuccess; }
 extern "C" __attribute__((visibility("default"))) const char* cudaGetErrorString(cudaError_t) { return "fake error"; }
 extern "C" __attribute__((visibility("default"))) const char* cudaGetErrorName(cudaError_t) { return "fakeError"; }

@@ -157,3 +157,22 @@ def test_the_selectors_parameters_may_take_an_idle_block(lib):
     o = bfs.bfs_opts(selector=bfs.BFS_SELECT_LEARNED)
     log = lib.taken(lambda: lib.run(g, N, 0, ctypes.byref(o)))
     assert [e for e in log if e.what == "memcpy" and e.bytes == 4 * bfs.BFS_MLP_PARAMS]
+
+
+def test_blocks_of_a_context_that_was_reset_are_forgotten(lib):
+    """cudaDeviceReset frees everything: what the cache held then is neither handed out nor freed again (its address
+    may belong to someone else by then)."""
+    cycle(lib)
+    old = {e.ptr for e in lib.taken(lambda: cycle(lib, 20 * N)) if e.what == "malloc"}
+    g = lib.graph(N)
+    lib.c.fake_set_context(2)
+    log = lib.taken(lambda: cycle(lib))
+    assert "malloc" in whats(log) and "free" not in whats(log)
+    assert not old & {e.ptr for e in log if e.what in ("memset", "memcpy")}
+    time.sleep(1.1)
+    log = lib.taken(lambda: (cycle(lib), lib.c.bfs_memory_trim()))
+    assert not old & {e.ptr for e in log if e.what == "free"}
+    kept = lib.c.fake_live_bytes()
+    lib.c.bfs_graph_destroy(g)  # a graph of the old context: its blocks are not kept either
+    lib.c.bfs_memory_trim()
+    assert lib.c.fake_live_bytes() <= kept
