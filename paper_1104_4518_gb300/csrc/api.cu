@@ -651,6 +651,7 @@ int bfs_graph_copy_csr(const bfs_graph* g, int64_t* offsets_out, int32_t* adj_ou
   const cudaMemcpyKind kind = (flags & BFS_HOST_PTRS) ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
   BFS_CUDA_TRY(cudaMemcpy(offsets_out, g->d_off, sizeof(int64_t) * ((size_t)g->n + 1), kind));
   if (g->nnz > 0) BFS_CUDA_TRY(cudaMemcpy(adj_out, g->d_adj, sizeof(int32_t) * (size_t)g->nnz, kind));
+  if (kind == cudaMemcpyDeviceToDevice) BFS_CUDA_TRY(cudaStreamSynchronize(nullptr));  // such a copy does not wait
   return BFS_OK;
 }
 

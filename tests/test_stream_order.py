@@ -96,3 +96,14 @@ def test_clearing_a_reported_error(lib):
     fills = [e for e in log if e.what == "memset"]
     assert status in [e.ptr for e in fills] and ctypes.c_int.from_address(status).value == 0
     assert all(e.stream == S for e in fills)
+
+
+def test_copying_the_rows_out_waits_for_the_copies(lib):
+    """bfs_graph_copy_csr is synchronous, to device memory too (cudaMemcpy between device arrays does not wait)."""
+    n = 100
+    g = lib.graph(n)
+    off, adj = (ctypes.c_int64 * (n + 1))(), (ctypes.c_int32 * (2 * n))()
+    log = lib.taken(lambda: lib.c.bfs_graph_copy_csr(g, off, adj, 0))
+    copies = [i for i, e in enumerate(log) if e.what == "memcpy"]
+    assert len(copies) == 2
+    assert any(e.what == "stream sync" and e.stream == log[copies[-1]].stream for e in log[copies[-1]:])
