@@ -88,18 +88,26 @@ size_t cache_limit(int device) {
   return limit[device];
 }
 
-// Takes the current device's cached blocks that have been idle for longer than `age` out of the cache.
-std::vector<void*> take_idle(std::chrono::steady_clock::duration age) {
-  std::vector<void*> out;
-  const auto now = std::chrono::steady_clock::now();
-  const unsigned long long context = current_context();
+// The device and context that the calling thread's next allocation is for.
+struct Here {
   int device = -1;
-  if (context == 0 || cudaGetDevice(&device) != cudaSuccess) return out;
+  unsigned long long context = current_context();
+  Here() {
+    if (cudaGetDevice(&device) != cudaSuccess) device = -1;
+  }
+};
+
+// Takes the device's cached blocks that have been idle for longer than `age` out of the cache.
+std::vector<void*> take_idle(const Here& here, std::chrono::steady_clock::duration age) {
+  std::vector<void*> out;
+  if (here.context == 0) return out;
   std::lock_guard<std::mutex> lk(g_mem_mu);
+  if (g_mem_idle.empty()) return out;
+  const auto now = std::chrono::steady_clock::now();
   for (size_t i = 0; i < g_mem_idle.size();) {
     CachedBlock& c = g_mem_idle[i];
-    const bool stale = c.context != context;  // freed by cudaDeviceReset
-    if (c.device == device && (stale || now - c.since >= age)) {
+    const bool stale = c.context != here.context;  // freed by cudaDeviceReset
+    if (c.device == here.device && (stale || now - c.since >= age)) {
       if (!stale) out.push_back(c.p);
       c = g_mem_idle.back();
       g_mem_idle.pop_back();
@@ -111,24 +119,22 @@ std::vector<void*> take_idle(std::chrono::steady_clock::duration age) {
 }
 
 // Gives the cached blocks that nothing has asked for lately back to the driver.
-void trim_device_cache() {
-  for (void* p : take_idle(std::chrono::seconds(1))) cudaFree(p);
+void trim_device_cache(const Here& here) {
+  for (void* p : take_idle(here, std::chrono::seconds(1))) cudaFree(p);
 }
 }  // namespace
 
 int dev_alloc(void** p, size_t bytes, const char* what) {
   *p = nullptr;
   const size_t need = (bytes + 511) / 512 * 512 + (bytes == 0 ? 512 : 0);
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
-  trim_device_cache();
-  const unsigned long long context = current_context();
+  Here here;
+  trim_device_cache(here);
   {
     std::lock_guard<std::mutex> lk(g_mem_mu);
     size_t best = g_mem_idle.size();
     for (size_t i = 0; i < g_mem_idle.size(); ++i) {
       const CachedBlock& c = g_mem_idle[i];
-      if (c.device != dev || c.context != context || c.bytes < need || c.bytes > need + std::max(need / 4, (size_t)1 << 20)) continue;
+      if (c.device != here.device || c.context != here.context || c.bytes < need || c.bytes > need + std::max(need / 4, (size_t)1 << 20)) continue;
       if (best == g_mem_idle.size() || c.bytes < g_mem_idle[best].bytes) best = i;
     }
     if (best < g_mem_idle.size()) {
@@ -142,7 +148,7 @@ int dev_alloc(void** p, size_t bytes, const char* what) {
   cudaError_t e = cudaMalloc(p, need);
   if (e == cudaErrorMemoryAllocation) {  // give back what the cache holds and try once more
     cudaGetLastError();
-    for (void* q : take_idle(std::chrono::steady_clock::duration::zero())) cudaFree(q);
+    for (void* q : take_idle(here, std::chrono::steady_clock::duration::zero())) cudaFree(q);
     e = cudaMalloc(p, need);
   }
   if (e != cudaSuccess) {
@@ -152,9 +158,9 @@ int dev_alloc(void** p, size_t bytes, const char* what) {
                 std::string("device allocation of ") + std::to_string(bytes) + " bytes for " + what + " failed: " +
                     cudaGetErrorString(e));
   }
-  const Block b{need, dev, current_context()};  // (the process's first allocation made the context)
+  if (here.context == 0) here.context = current_context();  // the thread's first call made it current
   std::lock_guard<std::mutex> lk(g_mem_mu);
-  g_mem_used[*p] = b;
+  g_mem_used[*p] = {need, here.device, here.context};
   return BFS_OK;
 }
 
@@ -162,7 +168,7 @@ void dev_free(void* p) {
   if (!p) return;
   bool keep = false;
   const bool idle = cudaDeviceSynchronize() == cudaSuccess;  // (it fails during another thread's stream capture)
-  const unsigned long long context = current_context();
+  const Here here;
   {
     std::lock_guard<std::mutex> lk(g_mem_mu);
     auto it = g_mem_used.find(p);
@@ -171,14 +177,13 @@ void dev_free(void* p) {
       g_mem_used.erase(it);
       size_t held = b.bytes;
       for (const CachedBlock& c : g_mem_idle) held += c.device == b.device ? c.bytes : 0;
-      int cur = -1;
-      keep = idle && cudaGetDevice(&cur) == cudaSuccess && cur == b.device && context != 0 && context == b.context &&
+      keep = idle && here.device == b.device && here.context != 0 && here.context == b.context &&
              held <= cache_limit(b.device);
       if (keep) g_mem_idle.push_back({b, p, std::chrono::steady_clock::now()});
     }
   }
   if (!keep) cudaFree(p);
-  trim_device_cache();
+  trim_device_cache(here);
 }
 
 int current_device_info(DeviceInfo* out) {
@@ -689,7 +694,7 @@ int bfs_memory_trim(void) {
   for (int d : devices) {
     cudaError_t e = cudaSetDevice(d);
     if (e == cudaSuccess)
-      for (void* p : take_idle(std::chrono::steady_clock::duration::zero()))
+      for (void* p : take_idle(Here{}, std::chrono::steady_clock::duration::zero()))
         if (cudaError_t f = cudaFree(p); f != cudaSuccess) e = f;
     if (e != cudaSuccess) err = e;
   }
