@@ -17,6 +17,8 @@
 #include <cooperative_groups.h>
 #include <cooperative_groups/scan.h>
 
+#include <cstddef>
+
 #include "device_common.cuh"
 #include "internal.h"
 
@@ -31,7 +33,7 @@ constexpr int kBigBuf = kClaimBlock;      // per-CTA buffer of claimed vertices 
 static_assert(kQBuf >= 2 * 64 * 33, "the batched transpose tiles live in the CTA buffer");
 
 struct Claims {
-  int qn;    // entries in cq (may exceed kQBuf: the excess went straight to the queue)
+  int qn;    // entries in the buffer (may exceed its room: the excess went straight to the queue)
   int nbig;  // entries in bigv (may exceed kBigBuf: the excess went straight to the chunk list)
   unsigned qbase, bbase;
   int scan_tmp[kClaimWarps + 1];
@@ -41,6 +43,10 @@ struct Claims {
     int cq[kQBuf];
     int wq[kClaimWarps][kWQBuf];
   };
+  // cq's first entry, for a phase whose buffer goes on into the shared memory behind this struct
+  __device__ __forceinline__ int* queue() {
+    return reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(this) + offsetof(Claims, cq));
+  }
 };
 
 __device__ __forceinline__ void claims_reset(Claims& cl) {
@@ -114,12 +120,14 @@ __device__ __forceinline__ void push_chunks_cta(const P& p, int knext, Claims& c
 
 // Appends w to the CTA's next-frontier buffer; when the buffer is full the
 // vertex goes to the queue directly (one atomic per group of converged threads).
+// room: the buffer's entries, kQBuf or more, the same for all claims of a phase
+// and for its flush.
 template <typename P>
-__device__ __forceinline__ void cta_enqueue(const P& p, int knext, Claims& cl, int w) {
+__device__ __forceinline__ void cta_enqueue(const P& p, int knext, Claims& cl, int w, int room = kQBuf) {
   namespace cg = cooperative_groups;
   const int pos = atomicAdd(&cl.qn, 1);
-  if (pos < kQBuf) {
-    cl.cq[pos] = w;
+  if (pos < room) {
+    cl.queue()[pos] = w;
   } else {
     cg::coalesced_group g = cg::coalesced_threads();
     unsigned base = 0;
@@ -154,10 +162,10 @@ __device__ __forceinline__ void warp_enqueue(const P& p, int knext, int* wq, int
 // global memory.  Called by every thread of the CTA (it synchronises); the
 // buffers are empty on return.
 template <typename P>
-__device__ __forceinline__ void flush_claims(const P& p, int knext, Claims& cl) {
+__device__ __forceinline__ void flush_claims(const P& p, int knext, Claims& cl, int room = kQBuf) {
   __syncthreads();
   const int nbig = min(cl.nbig, kBigBuf);
-  const int nq = min(cl.qn, kQBuf);
+  const int nq = min(cl.qn, room);
   if (nbig == 0 && nq == 0) return;  // nothing buffered (the counters are zero already)
   int nch_total = 0;
   if (nbig > 0) {  // inclusive prefix sums of the chunk counts, two entries per thread
@@ -176,7 +184,7 @@ __device__ __forceinline__ void flush_claims(const P& p, int knext, Claims& cl) 
   __syncthreads();
   int32_t* Q = p.queue[knext % 3];
   for (int i = threadIdx.x; i < nq; i += kClaimBlock)
-    if (bfsdev::in_range(p.status, bfsdev::kSiteQueue, (long long)cl.qbase + i, p.n)) Q[cl.qbase + i] = cl.cq[i];
+    if (bfsdev::in_range(p.status, bfsdev::kSiteQueue, (long long)cl.qbase + i, p.n)) Q[cl.qbase + i] = cl.queue()[i];
   int64_t* dst = p.chunks[knext & 1];
   for (int it = threadIdx.x; it < nch_total; it += kClaimBlock) {
     int lo = 0, hi = nbig - 1;  // the first entry whose inclusive prefix exceeds it
@@ -201,10 +209,11 @@ __device__ __forceinline__ void flush_claims(const P& p, int knext, Claims& cl) 
 // same level also use: the level took 0.81 ms instead of 0.44 ms.  Called by
 // every thread of the CTA at a point where the whole CTA is converged.
 template <typename P>
-__device__ __forceinline__ void flush_claims_if_full(const P& p, int knext, Claims& cl, int qroom, int bigroom) {
+__device__ __forceinline__ void flush_claims_if_full(const P& p, int knext, Claims& cl, int qroom, int bigroom,
+                                                     int room = kQBuf) {
   __syncthreads();
-  if (cl.qn > kQBuf - qroom || cl.nbig > kBigBuf - bigroom) {  // the same on every thread after the barrier
-    flush_claims(p, knext, cl);
+  if (cl.qn > room - qroom || cl.nbig > kBigBuf - bigroom) {  // the same on every thread after the barrier
+    flush_claims(p, knext, cl, room);
     __syncthreads();  // thread 0's reset of the counts lands before any thread claims again
   }
 }

@@ -150,19 +150,19 @@ __device__ __forceinline__ void acc_vertex(Acc& a, long long deg) {
 
 // Bookkeeping of a vertex claimed for level knext (the caller already set nxt).
 __device__ __forceinline__ void claim_topdown(const LoopParams& p, int knext, int w, long long deg, Acc& acc,
-                                              Claims& cl) {
+                                              Claims& cl, int room) {
   p.level[w] = knext;
-  cta_enqueue(p, knext, cl, w);
+  cta_enqueue(p, knext, cl, w, room);
   acc_vertex(acc, deg);
   if (deg > p.chunk_deg) push_chunks_cta(p, knext, cl, w, deg);
 }
 
 // Top-down visits of up to N edges (u[i] -> w[i]) in phase k (w[i] < 0: none).
 // Each kind of load is issued for all of them before any is used: a visit is a
-// chain of three dependent round trips to L2 or DRAM.
+// chain of three dependent round trips to L2 or DRAM.  room: see cta_enqueue.
 template <int N>
 __device__ __forceinline__ void td_visit(const LoopParams& p, const uint32_t* cur, uint32_t* nxt, int k,
-                                         const int (&u)[N], const int (&w)[N], Acc& acc, Claims& cl) {
+                                         const int (&u)[N], const int (&w)[N], Acc& acc, Claims& cl, int room = kQBuf) {
   uint32_t reached[N], nw[N];
 #pragma unroll
   for (int i = 0; i < N; ++i) {
@@ -198,16 +198,16 @@ __device__ __forceinline__ void td_visit(const LoopParams& p, const uint32_t* cu
   for (int i = 0; i < N; ++i) {
     if (mine[i]) {
       if (p.claim_by_parent) atomicOr(&nxt[w[i] >> 5], 1u << (w[i] & 31));
-      claim_topdown(p, k + 1, w[i], deg[i], acc, cl);
+      claim_topdown(p, k + 1, w[i], deg[i], acc, cl, room);
     }
   }
 }
 
 // One edge.
 __device__ __forceinline__ void td_visit(const LoopParams& p, const uint32_t* cur, uint32_t* nxt, int k, int u, int w,
-                                         Acc& acc, Claims& cl) {
+                                         Acc& acc, Claims& cl, int room = kQBuf) {
   const int u1[1] = {u}, w1[1] = {w};
-  td_visit<1>(p, cur, nxt, k, u1, w1, acc, cl);
+  td_visit<1>(p, cur, nxt, k, u1, w1, acc, cl, room);
 }
 
 // 64-bit warp sum.
@@ -223,7 +223,7 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
 // End of a phase: the CTA's counter contributions, its buffered queue entries
 // and its buffered chunk items go to level knext with one atomic each.
 template <typename S>
-__device__ __forceinline__ void end_phase(const LoopParams& p, int knext, Acc& acc, S& sm) {
+__device__ __forceinline__ void end_phase(const LoopParams& p, int knext, Acc& acc, S& sm, int room = kQBuf) {
   const bool mine = (acc.b0 | acc.b1 | acc.b2) != 0;
   if (__syncthreads_or(mine)) {
     // n < 2^31 vertices in all: a warp's counts fit 32 bits
@@ -246,11 +246,12 @@ __device__ __forceinline__ void end_phase(const LoopParams& p, int knext, Acc& a
       sm.acc[0] = sm.acc[1] = sm.acc[2] = sm.acc[3] = 0;
     }
   }
-  flush_claims(p, knext, sm.cl);
+  flush_claims(p, knext, sm.cl, room);
   acc = Acc{};
 }
 
-struct Smem {
+// The CTA's state; the phases' area follows it in shared memory, behind the claim buffer.
+struct __align__(64) Smem {
   float4 mlp_y;  // outputs of the selector network
   LevelCtr ctr;  // counters of the level to expand, fetched by thread 0 at the barrier before it
   int owner;
@@ -259,7 +260,6 @@ struct Smem {
   int warp_tmp[kWarps + 1];
   unsigned long long acc[4];
   Claims cl;
-  unsigned long long next_item;  // top-down: the next chunk item of this CTA
 };
 
 // ---------------- top-down phase ----------------
@@ -339,6 +339,16 @@ struct FirstRow {
   long long b = 0, e = 0;
 };
 
+// The thread and warp variants leave the phases' area free, and their claim buffer
+// goes on into it: without a barrier in their loops, which a row of 1,024 edges
+// would hold up, they cannot empty it on the way.  Six roots at scale 25, edgefactor 4,
+// per root: thread 15.2 -> 11.9 ms, warp 13.1 -> 8.8 (14.0 and 11.9 with a buffer of
+// 6,144 entries, which took L1 from every phase).
+constexpr int kLongQ = 15040;  // entries (checked below)
+__device__ __forceinline__ int claim_room(int variant) {
+  return variant == BFS_VARIANT_TD_THREAD || variant == BFS_VARIANT_TD_WARP ? kLongQ : kQBuf;
+}
+
 __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned count, unsigned nchunks,
                               const FirstRow& first, Smem& sm, FlatSmem& fl, Acc& acc, unsigned G) {
   const uint32_t* cur = p.bits[k % 3];
@@ -350,7 +360,7 @@ __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned 
   // item the CTA makes room in its buffers for the item's claims
   const int64_t* items = p.chunks[k & 1];
   for (unsigned ci = blockIdx.x; ci < nchunks; ci += G) {
-    flush_claims_if_full(p, k + 1, sm.cl, kChunkEdges, kBigBuf / 2);
+    flush_claims_if_full(p, k + 1, sm.cl, kChunkEdges, kBigBuf / 2, claim_room(variant));
     const int64_t it = items[ci];
     const int v = (int)(it >> 32);
     const long long c = it & 0xffffffffll;
@@ -360,7 +370,7 @@ __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned 
     static_assert(kChunkEdges == 2 * kBlock, "two visits per thread and chunk");
     const int us[2] = {b + tid < e ? v : -1, b + kBlock + tid < e ? v : -1};
     const int ws[2] = {us[0] >= 0 ? __ldg(&p.adj[b + tid]) : 0, us[1] >= 0 ? __ldg(&p.adj[b + kBlock + tid]) : 0};
-    td_visit<2>(p, cur, nxt, k, us, ws, acc, sm.cl);
+    td_visit<2>(p, cur, nxt, k, us, ws, acc, sm.cl, claim_room(variant));
   }
 
   // frontier entry i goes to CTA i % G, so that small frontiers spread over the SMs
@@ -371,7 +381,7 @@ __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned 
       atomicOr(&p.vis[u >> 5], 1u << (u & 31));
       const long long b = __ldg(&p.off[u]), e = __ldg(&p.off[u + 1]);
       if (e - b > p.chunk_deg) continue;
-      for (long long j = b; j < e; ++j) td_visit(p, cur, nxt, k, u, __ldg(&p.adj[j]), acc, sm.cl);
+      for (long long j = b; j < e; ++j) td_visit(p, cur, nxt, k, u, __ldg(&p.adj[j]), acc, sm.cl, kLongQ);
     }
   } else if (variant == BFS_VARIANT_TD_WARP) {
     const long long gwarps = gthreads / 32;
@@ -384,7 +394,8 @@ __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned 
       }
       if (lane == 0) atomicOr(&p.vis[row.u >> 5], 1u << (row.u & 31));
       if (row.e - row.b <= p.chunk_deg)
-        for (long long j = row.b + lane; j < row.e; j += 32) td_visit(p, cur, nxt, k, row.u, __ldg(&p.adj[j]), acc, sm.cl);
+        for (long long j = row.b + lane; j < row.e; j += 32)
+          td_visit(p, cur, nxt, k, row.u, __ldg(&p.adj[j]), acc, sm.cl, kLongQ);
       row.u = -1;
     }
   } else {  // BFS_VARIANT_TD_BINNED
@@ -1004,6 +1015,8 @@ __device__ __forceinline__ int heuristic_variant(const LoopParams& p, int prev_v
 constexpr size_t kFlatBytes = (sizeof(FlatSmem) + 15) / 16 * 16;
 // the largest phase's area, without and with the tiled phase
 constexpr size_t kPhaseBytes = std::max(sizeof(PullSmem), kFlatBytes);
+static_assert(offsetof(Smem, cl) + offsetof(Claims, cq) + kLongQ * sizeof(int) <= sizeof(Smem) + kPhaseBytes,
+              "the long claim buffer ends with the phases' area");
 constexpr size_t kMlpBytes = (sizeof(float) * BFS_MLP_PARAMS + 15) / 16 * 16;
 static_assert(kPhaseBytes >= kMlpBytes + sizeof(bfsdev::MlpScratch), "the network fits the phases' area");
 constexpr size_t kTiledBytes = std::max(kPhaseBytes, kFlatBytes + sizeof(uint32_t) * 3 * kTileWordsMax);
@@ -1032,11 +1045,12 @@ struct FetchMlp {
 // pick the tiled variant, and the other runs do without the network's code.
 template <bool kTiles, bool kLearned>
 __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
-  __shared__ Smem sm;
   // dynamic shared memory: one area that the phases use in turn (PullSmem, or
   // FlatSmem and the tiled phase's 3 * kTileWordsMax words), and between phases
   // the selector network's parameters
-  extern __shared__ __align__(16) unsigned char s_dyn[];
+  extern __shared__ __align__(64) unsigned char s_all[];
+  Smem& sm = *reinterpret_cast<Smem*>(s_all);
+  unsigned char* const s_dyn = s_all + sizeof(Smem);
   FlatSmem& s_flat = *reinterpret_cast<FlatSmem*>(s_dyn);
   uint32_t* s_tile = reinterpret_cast<uint32_t*>(s_dyn + kFlatBytes);
   PullSmem& s_pull = *reinterpret_cast<PullSmem*>(s_dyn);
@@ -1234,7 +1248,7 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
         flat_phase(p, k, count, sm, s_flat, acc, G);
       else topdown_phase(p, k, variant, count, nchunks, first, sm, s_flat, acc, G);
       PHASE_TS(k, 3);
-      end_phase(p, k + 1, acc, sm);
+      end_phase(p, k + 1, acc, sm, claim_room(variant));
     }
     PHASE_TS(k, 4);
     PHASE_ARRIVAL(k);
@@ -1414,7 +1428,7 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
     p.t_ncb = ts->ncb;
   }
 
-  const size_t dyn_smem = p.t_jc ? kTiledBytes : kPhaseBytes;
+  const size_t dyn_smem = sizeof(Smem) + (p.t_jc ? kTiledBytes : kPhaseBytes);
   const void* const kernels[] = {(const void*)level_loop_kernel<false, false>, (const void*)level_loop_kernel<true, false>,
                                  (const void*)level_loop_kernel<false, true>};
   const void* kernel = kernels[p.mlp ? 2 : p.t_jc ? 1 : 0];
@@ -1425,7 +1439,8 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
     if (di.device < 0 || di.device >= 64) return fail(BFS_ERR_UNSUPPORTED, "device ordinal out of range");
     if (!configured[di.device]) {
       for (const void* f : kernels)
-        BFS_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTiledBytes));
+        BFS_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)(sizeof(Smem) + kTiledBytes)));
       configured[di.device] = true;
     }
   }
