@@ -460,8 +460,10 @@ __global__ void __launch_bounds__(kMetaThreads) row_meta_kernel(const int64_t* _
 
 // Probe records of the rows with entries (out non-null): one warp per bitmap
 // word, packed in id order; and the chunk items of rows longer than kChunkEdges,
-// in any order.
-__global__ void row_records_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
+// in any order.  A row outside [0, nnz) (a malformed CSR, taken without
+// validation) gives a record without entries: creating a graph reads no entry
+// that is not there.
+__global__ void row_records_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ adj, long long nnz,
                                    const uint32_t* __restrict__ dead, const uint32_t* __restrict__ rank,
                                    long long nwords, int4* __restrict__ out, int64_t* __restrict__ big,
                                    unsigned long long* big_count) {
@@ -471,9 +473,11 @@ __global__ void row_records_kernel(const int64_t* __restrict__ off, const int32_
     const uint32_t live = ~dead[w];  // the bits past n are dead
     if (!((live >> lane) & 1u)) continue;
     const long long v = w * 32 + lane, b = off[v], e = off[v + 1], d = e - b;
-    if (out)
+    if (out) {
+      const bool in = b >= 0 && e <= nnz;
       out[(long long)rank[w] + __popc(live & bfsdev::lanemask_lt())] =
-          make_int4((int)d, adj[e - 1], d > 1 ? adj[e - 2] : 0, d > 2 ? adj[e - 3] : 0);
+          make_int4((int)d, in ? adj[e - 1] : 0, in && d > 1 ? adj[e - 2] : 0, in && d > 2 ? adj[e - 3] : 0);
+    }
     if (d > kChunkEdges) {
       const unsigned long long nch = (unsigned long long)((d + kChunkEdges - 1) / kChunkEdges);
       const unsigned long long pos = atomicAdd(big_count, nch);
@@ -613,7 +617,7 @@ int build_row_tables(const int64_t* d_off, const int32_t* d_adj, int32_t n, int6
   // the pull works without probe records, only slower: a graph that leaves no room for them does without
   if (dev_alloc((void**)&t.probe, sizeof(int4) * (size_t)std::max(1ull, rep.nlive), "probe records") != BFS_OK)
     t.probe = nullptr;
-  row_records_kernel<<<di.sm_count * 8, 256, 0, s>>>(d_off, d_adj, t.dead, t.rank, nwords, t.probe, t.big, &d_rep->nkeys);
+  row_records_kernel<<<di.sm_count * 8, 256, 0, s>>>(d_off, d_adj, nnz, t.dead, t.rank, nwords, t.probe, t.big, &d_rep->nkeys);
   err = cudaGetLastError();
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);
   if (err != cudaSuccess) return give_up(cuda_fail(err, "row tables"));
