@@ -38,6 +38,7 @@
 #include <mutex>
 #include <climits>
 #include <cstdio>
+#include <type_traits>
 
 #include "device_common.cuh"
 #include "internal.h"
@@ -250,7 +251,7 @@ __device__ __forceinline__ void end_phase(const LoopParams& p, int knext, Acc& a
   acc = Acc{};
 }
 
-// The CTA's state; the phases' area follows it in shared memory, behind the claim buffer.
+// The CTA's state.  With kLong the phases' area follows it in shared memory, behind the claim buffer.
 struct __align__(64) Smem {
   float4 mlp_y;  // outputs of the selector network
   LevelCtr ctr;  // counters of the level to expand, fetched by thread 0 at the barrier before it
@@ -339,28 +340,29 @@ struct FirstRow {
   long long b = 0, e = 0;
 };
 
-// The thread and warp variants leave the phases' area free, and their claim buffer
-// goes on into it: without a barrier in their loops, which a row of 1,024 edges
-// would hold up, they cannot empty it on the way.  Six roots at scale 25, edgefactor 4,
-// per root: thread 15.2 -> 11.9 ms, warp 13.1 -> 8.8 (14.0 and 11.9 with a buffer of
-// 6,144 entries, which took L1 from every phase).
+// kLong: the claim buffer of the thread and warp variants goes on into the phases'
+// area, which they leave free: without a barrier in their loops, which a row of
+// 1,024 edges would hold up, they cannot empty it on the way.
 constexpr int kLongQ = 15040;  // entries (checked below)
+template <bool kLong>
 __device__ __forceinline__ int claim_room(int variant) {
-  return variant == BFS_VARIANT_TD_THREAD || variant == BFS_VARIANT_TD_WARP ? kLongQ : kQBuf;
+  return kLong && (variant == BFS_VARIANT_TD_THREAD || variant == BFS_VARIANT_TD_WARP) ? kLongQ : kQBuf;
 }
 
+template <bool kLong>
 __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned count, unsigned nchunks,
                               const FirstRow& first, Smem& sm, FlatSmem& fl, Acc& acc, unsigned G) {
   const uint32_t* cur = p.bits[k % 3];
   uint32_t* nxt = p.bits[(k + 1) % 3];
   const int32_t* Q = p.queue[k % 3];
   const int tid = threadIdx.x, lane = tid & 31;
+  constexpr int kRoom = kLong ? kLongQ : kQBuf;  // of the thread and warp variants
 
   // chunk items of high-degree frontier vertices: one CTA per item; before each
   // item the CTA makes room in its buffers for the item's claims
   const int64_t* items = p.chunks[k & 1];
   for (unsigned ci = blockIdx.x; ci < nchunks; ci += G) {
-    flush_claims_if_full(p, k + 1, sm.cl, kChunkEdges, kBigBuf / 2, claim_room(variant));
+    flush_claims_if_full(p, k + 1, sm.cl, kChunkEdges, kBigBuf / 2);
     const int64_t it = items[ci];
     const int v = (int)(it >> 32);
     const long long c = it & 0xffffffffll;
@@ -370,8 +372,10 @@ __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned 
     static_assert(kChunkEdges == 2 * kBlock, "two visits per thread and chunk");
     const int us[2] = {b + tid < e ? v : -1, b + kBlock + tid < e ? v : -1};
     const int ws[2] = {us[0] >= 0 ? __ldg(&p.adj[b + tid]) : 0, us[1] >= 0 ? __ldg(&p.adj[b + kBlock + tid]) : 0};
-    td_visit<2>(p, cur, nxt, k, us, ws, acc, sm.cl, claim_room(variant));
+    td_visit<2>(p, cur, nxt, k, us, ws, acc, sm.cl);
   }
+  // the items' claims, for which there was room in kQBuf, come before any claim past it
+  if (kLong && nchunks) __syncthreads();
 
   // frontier entry i goes to CTA i % G, so that small frontiers spread over the SMs
   const long long gthreads = (long long)G * kBlock;
@@ -381,7 +385,7 @@ __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned 
       atomicOr(&p.vis[u >> 5], 1u << (u & 31));
       const long long b = __ldg(&p.off[u]), e = __ldg(&p.off[u + 1]);
       if (e - b > p.chunk_deg) continue;
-      for (long long j = b; j < e; ++j) td_visit(p, cur, nxt, k, u, __ldg(&p.adj[j]), acc, sm.cl, kLongQ);
+      for (long long j = b; j < e; ++j) td_visit(p, cur, nxt, k, u, __ldg(&p.adj[j]), acc, sm.cl, kRoom);
     }
   } else if (variant == BFS_VARIANT_TD_WARP) {
     const long long gwarps = gthreads / 32;
@@ -395,7 +399,7 @@ __device__ void topdown_phase(const LoopParams& p, int k, int variant, unsigned 
       if (lane == 0) atomicOr(&p.vis[row.u >> 5], 1u << (row.u & 31));
       if (row.e - row.b <= p.chunk_deg)
         for (long long j = row.b + lane; j < row.e; j += 32)
-          td_visit(p, cur, nxt, k, row.u, __ldg(&p.adj[j]), acc, sm.cl, kLongQ);
+          td_visit(p, cur, nxt, k, row.u, __ldg(&p.adj[j]), acc, sm.cl, kRoom);
       row.u = -1;
     }
   } else {  // BFS_VARIANT_TD_BINNED
@@ -1043,14 +1047,22 @@ struct FetchMlp {
 // code alone made the other phases 5 % slower.
 // kLearned: the selector network may choose the variants.  Learned runs never
 // pick the tiled variant, and the other runs do without the network's code.
-template <bool kTiles, bool kLearned>
+// kLong: see topdown_phase; for forced and scheduled runs, which may run a large level
+// by threads or warps.  The heuristic runs only levels of at most 32 edges a warp that
+// way, and the network's choices at large levels are others.  Six roots on 2^27 edges,
+// every level by threads and by warps, ms per root: edgefactor 4 15.2 -> 11.1 and 13.1 ->
+// 7.6, 8 7.9 -> 7.8 and 6.5 -> 6.1, 16 6.7 -> 6.6 and 4.5 (with a buffer of 6,144 entries in
+// every instance, which took L1 from every phase, edgefactor 4 took 14.0 and 11.9).
+template <bool kTiles, bool kLearned, bool kLong>
 __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
   // dynamic shared memory: one area that the phases use in turn (PullSmem, or
   // FlatSmem and the tiled phase's 3 * kTileWordsMax words), and between phases
   // the selector network's parameters
   extern __shared__ __align__(64) unsigned char s_all[];
-  Smem& sm = *reinterpret_cast<Smem*>(s_all);
-  unsigned char* const s_dyn = s_all + sizeof(Smem);
+  // kLong: the CTA's state lies in front of the phases' area, so that its claim buffer can go on into it
+  __shared__ std::conditional_t<kLong, char, Smem> s_state;
+  Smem& sm = *reinterpret_cast<Smem*>(kLong ? s_all : reinterpret_cast<unsigned char*>(&s_state));
+  unsigned char* const s_dyn = kLong ? s_all + sizeof(Smem) : s_all;
   FlatSmem& s_flat = *reinterpret_cast<FlatSmem*>(s_dyn);
   uint32_t* s_tile = reinterpret_cast<uint32_t*>(s_dyn + kFlatBytes);
   PullSmem& s_pull = *reinterpret_cast<PullSmem*>(s_dyn);
@@ -1246,9 +1258,9 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
       // the degree-binned variant deals a small frontier's edges out flat
       else if (variant == BFS_VARIANT_TD_BINNED && count <= (unsigned)kFlatRows && edges <= p.flat_visits * pthreads)
         flat_phase(p, k, count, sm, s_flat, acc, G);
-      else topdown_phase(p, k, variant, count, nchunks, first, sm, s_flat, acc, G);
+      else topdown_phase<kLong>(p, k, variant, count, nchunks, first, sm, s_flat, acc, G);
       PHASE_TS(k, 3);
-      end_phase(p, k + 1, acc, sm, claim_room(variant));
+      end_phase(p, k + 1, acc, sm, claim_room<kLong>(variant));
     }
     PHASE_TS(k, 4);
     PHASE_ARRIVAL(k);
@@ -1428,10 +1440,16 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
     p.t_ncb = ts->ncb;
   }
 
-  const size_t dyn_smem = sizeof(Smem) + (p.t_jc ? kTiledBytes : kPhaseBytes);
-  const void* const kernels[] = {(const void*)level_loop_kernel<false, false>, (const void*)level_loop_kernel<true, false>,
-                                 (const void*)level_loop_kernel<false, true>};
-  const void* kernel = kernels[p.mlp ? 2 : p.t_jc ? 1 : 0];
+  // The long claim buffer (kLong) pays where a level can overfill the short ones of all CTAs together: below twice
+  // their entries (2.6 M vertices) it gained nothing (2.1 M, edgefactor 64: 5.4 and 2.7 ms with either) and cost
+  // narrow levels 0.5 % (grid 128^3, all by warps: 2.660 and 2.675 ms).
+  const bool picked = r.selector == BFS_SELECT_FORCED || r.selector == BFS_SELECT_SCHEDULE;
+  const bool long_buffer = p.t_jc || (picked && g->n > 2ll * (2 * di.sm_count) * kQBuf);
+  const size_t dyn_smem = (p.t_jc ? kTiledBytes : kPhaseBytes) + (long_buffer ? sizeof(Smem) : 0);
+  const void* const kernels[] = {
+      (const void*)level_loop_kernel<false, false, false>, (const void*)level_loop_kernel<false, false, true>,
+      (const void*)level_loop_kernel<true, false, true>, (const void*)level_loop_kernel<false, true, false>};
+  const void* kernel = kernels[p.mlp ? 3 : p.t_jc ? 2 : long_buffer ? 1 : 0];
   {  // the attribute belongs to the current device: set it once per device
     static std::mutex mu;
     static bool configured[64] = {};

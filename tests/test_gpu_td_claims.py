@@ -37,12 +37,14 @@ def check(g, want_parent, want_level):
         name = bfs.VARIANT_NAMES[variant]
         assert torch.equal(level, want_level), name
         assert torch.equal(parent, want_parent), name
-        assert opts.edges == g.n - 1 and opts.nlevels == 3, name
+        assert opts.edges == int((want_level > 0).sum()) and opts.nlevels == 3, name
     g.destroy()
 
 
 @pytest.mark.parametrize("children", edges((BUFFER, LONG)))
-def test_claims_at_the_ends_of_the_buffers(children):
+@pytest.mark.parametrize("large", [False, True])
+def test_claims_at_the_ends_of_the_buffers(children, large):
+    """large: with isolated vertices up to a size whose forced runs have the long buffer."""
     require_cuda()
     ctas = 2 * torch.cuda.get_device_properties(0).multi_processor_count
     rows = WARPS * ctas
@@ -50,8 +52,10 @@ def test_claims_at_the_ends_of_the_buffers(children):
     inner = torch.arange(1, rows + 1, dtype=torch.int32, device="cuda")
     leaves = torch.arange(rows + 1, n, dtype=torch.int32, device="cuda")
     of = inner.repeat_interleave(children)
-    g = bfs.bfs_graph_create_from_edges(torch.cat([torch.zeros_like(inner), of]), torch.cat([inner, leaves]), n)
-    check(g, want_parent_of(inner, of), level_of(inner, of))
+    more = max(0, 3000000 - n) if large else 0
+    g = bfs.bfs_graph_create_from_edges(torch.cat([torch.zeros_like(inner), of]), torch.cat([inner, leaves]), n + more)
+    none = torch.full((more,), -1, dtype=torch.int32, device="cuda")
+    check(g, torch.cat([want_parent_of(inner, of), none]), torch.cat([level_of(inner, of), none]))
 
 
 def test_chunked_rows_beside_overflowing_ones():
