@@ -22,8 +22,8 @@
 //   top-down : every frontier row ORs its bits into F_{k+1} of unreached
 //              neighbours and offers itself as their parent with atomicMax
 //              for each new root bit (every frontier neighbour offers, so the
-//              largest id wins); the first writer of a root bit writes the
-//              level, the first writer of any bit enqueues the neighbour.
+//              largest id wins); the first writer of any bit enqueues the
+//              neighbour.
 //              Rows above kChunkEdges entries are split into chunk items.
 // Output rows are root-major: level[r * n + v], parent[r * n + v].  During
 // the traversal the parents go to vertex-major scratch (sp[v][r], one row of
@@ -325,8 +325,8 @@ __device__ __forceinline__ void td_visit(const BatchParams& p, const Word* Fc, W
 
 // Pull over one kChunkEdges-entry chunk [rb, re) of a long row of v by one warp;
 // chunks of the same row combine through atomicMax on the parents and atomicOr
-// on F_{k+1}, whose first setter of a root bit writes that root's level, and
-// whose first setter of any bit claims v for the queue.
+// on F_{k+1}, whose first setter of any bit claims v for the queue (the level
+// goes to the planes when v is expanded, as everywhere).
 template <typename Word>
 __device__ __forceinline__ void pull_chunk(const BatchParams& p, const Word* Fc, Word* Fn, int knext, int v,
                                            long long rb, long long re, uint64_t need, int lane, Claims& cl,

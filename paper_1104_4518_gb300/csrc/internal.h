@@ -173,9 +173,11 @@ bfs_tuning effective_tuning(const bfs_graph* g);
 // mode 0: undirected (both arcs of every edge), 1: arcs src -> dst, 2: arcs dst -> src.
 int build_csr_from_edges(const int32_t* d_src, const int32_t* d_dst, int64_t m, int32_t n, int mode,
                          cudaStream_t s, int64_t** d_off, int32_t** d_adj, int64_t* nnz);
-// Stable least-significant-digit radix sort of N 64-bit keys on bits
-// [lo_bit, hi_bit); alt is scratch of N keys; *sorted is whichever of the two
-// buffers holds the result.  Synchronises s.
+// Least-significant-digit radix sort of N 64-bit keys on bits [lo_bit, hi_bit);
+// alt is scratch of N keys; *sorted is whichever of the two buffers holds the
+// result.  Stable when lo_bit > 0.  With lo_bit == 0 keys must have no bits at or
+// above hi_bit: keys that agree in all sorted bits are then the same key, and the
+// first pass does not keep their order.  Synchronises s.
 int radix_sort_u64(uint64_t* keys, uint64_t* alt, long long N, int lo_bit, int hi_bit, cudaStream_t s,
                    uint64_t** sorted);
 // Exclusive prefix sum of N uint32 values into int64 out; *total receives the sum.

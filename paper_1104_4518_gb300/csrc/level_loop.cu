@@ -218,11 +218,9 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
   return v;
 }
 
-// End of a phase for one CTA: adds its counters into level knext's slot and
-// moves its buffered next-frontier vertices to the global queue with a single
-// atomic.  CTAs that claimed nothing skip all of it.
 // End of a phase: the CTA's counter contributions, its buffered queue entries
-// and its buffered chunk items go to level knext with one atomic each.
+// and its buffered chunk items go to level knext with one atomic each.  CTAs that
+// claimed nothing skip all of it.  room: see cta_enqueue.
 template <typename S>
 __device__ __forceinline__ void end_phase(const LoopParams& p, int knext, Acc& acc, S& sm, int room = kQBuf) {
   const bool mine = (acc.b0 | acc.b1 | acc.b2) != 0;
@@ -1475,7 +1473,9 @@ int launch_level_loop(const RunRequest& r, cudaStream_t s) {
   // the parents no longer sit in L2 its result comes from DRAM (scale 26, 7 M edges: 425 -> 496 us).
   p.claim_by_parent = 4ll * g->n <= (di.l2_bytes > 0 ? di.l2_bytes : (1ll << 27)) / 2;
   // 32 parts of a ragged batch, 0.9 M edges: flat 28 us, by rows and chunks 55 us; at scale 26, 2.1 M edges, the
-  // chunks' two visits in flight win (171 us against 223)
+  // chunks' two visits in flight win (171 us against 223).  Whole traversals feel it by 1 or 2 % at most: 16 against 4,
+  // us per root over 32 roots, edgefactor 16, scale 20 72.1 and 73.0, 22 127.2 and 127.6, 24 419.5 and 420.8, 25 794
+  // and 794, 26 1,489.5 and 1,488.5; 32 ragged parts 417 and 436; against it scale 24 with edgefactor 64, 513 and 509
   p.flat_visits = p.claim_by_parent ? 16 : 4;
   // one chunk per resident warp while a lane per word allows it (see pull_phase)
   const long long grid_warps = (long long)grid * kWarps;

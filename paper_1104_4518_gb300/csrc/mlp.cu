@@ -505,7 +505,7 @@ int bfs_selector_save(const char* path) {
 int bfs_level_features(int32_t n, int64_t nnz, int32_t k, int64_t frontier_count, int64_t frontier_edges,
                        int64_t unvisited_count, int64_t unvisited_edges, const int64_t* bin_count, float* out12) {
   if (!bin_count || !out12) return fail(BFS_ERR_INVALID_ARG, "bfs_level_features: NULL pointer");
-  // the float32 expressions of the in-loop selector (bfsdev::level_features)
+  // the float32 expressions of the in-loop selector (bfsdev::warp_level_features)
   float rn = 0.0f, re = 0.0f;
   bfsint::graph_feature_constants(n, nnz, &out12[0], &out12[1], &rn, &re);
   const float c = (float)frontier_count, d = (float)frontier_edges;

@@ -1,4 +1,8 @@
-// Stable least-significant-digit radix sort of 64-bit keys.
+// Least-significant-digit radix sort of 64-bit keys, in the manner of the
+// published one-sweep method (Adinets and Merrill, 2022): one read for all
+// digit histograms, one read and one write per pass, the tiles of a pass linked
+// by a chained scan with look-back (Merrill and Garland, 2016).  The order of
+// equal digits is kept, except by a pass on bit 0 (see launch_sort_passes).
 //
 // All digit histograms are taken in one read of the keys (by the caller, who
 // often makes the keys anyway), and each pass then reads and writes every key

@@ -128,9 +128,10 @@ SortScratch sort_scratch_at(void* block, long long cap);
 
 // Digit histograms of keys[0, N) into sc.hist.
 int launch_sort_hist(const uint64_t* keys, long long N, const SortPlan& plan, const SortScratch& sc, cudaStream_t s);
-// The passes of a stable sort of *d_n keys (at most cap; cap itself when d_n is
-// null), whose histograms sc.hist holds.  Keys sorted from bit 0 on have no bits
-// above the sorted ones, so that equal keys are alike.  Nothing is waited for.  Returns the
+// The passes of a sort of *d_n keys (at most cap; cap itself when d_n is null),
+// whose histograms sc.hist holds.  Stable unless it starts at bit 0: keys sorted
+// from there on must have no bits above the sorted ones, so that equal keys are
+// alike and the first pass need not keep their order.  Nothing is waited for.  Returns the
 // buffer that will hold the result; *status receives BFS_ERR_TIMEOUT when a
 // wait ran out.
 uint64_t* launch_sort_passes(uint64_t* keys, uint64_t* alt, long long cap, const unsigned long long* d_n,
