@@ -44,7 +44,7 @@ int current_device_info(DeviceInfo* out);
 // ---------------- level counters (device) ----------------
 // One slot per level in a ring of kCtrRing: filled while the frontier of that
 // level is built, read after the grid barrier that ends the phase.
-constexpr int kCtrRing = 8;
+constexpr int kCtrRing = 64;
 struct __align__(64) LevelCtr {
   unsigned int count;             // frontier vertices (also the queue tail)
   unsigned int chunks;            // chunk items of high-degree frontier vertices

@@ -14,7 +14,7 @@
 //   vis  = visited bitmap; during phase k it holds levels <= k-1 (and possibly k),
 //          so "reached" is tested as (vis | cur)
 //   queue[k % 3]              f_k as a list; queue[(k + 1) % 3] receives f_{k+1}
-//   ctr[k % 8]                counters of f_k (size, degree sum, degree bins)
+//   ctr[k % 64]               counters of f_k (size, degree sum, degree bins)
 //
 // Variants (identical results):
 //   top-down (thread / warp / degree-binned): for u in f_k and every neighbour w
@@ -1142,6 +1142,7 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
     }
   }
   if (blockIdx.x == 0) {
+    static_assert(kCtrRing * sizeof(LevelCtr) / 8 <= kBlock, "one word of the ring per thread");
     if (tid < kCtrRing * (int)(sizeof(LevelCtr) / 8)) reinterpret_cast<unsigned long long*>(p.ctr)[tid] = 0ull;
     __syncthreads();
     if (single && tid == 0) {
@@ -1205,14 +1206,19 @@ __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
     // at its barrier, which halves the barrier's arrivals and the CTAs that
     // contend for the level's few claims.  The other CTAs still choose the
     // variant (the next level's choice depends on it) and wait at the barrier.
-    const unsigned G = (edges <= p.narrow_edges && nblocks >= 2) ? (nblocks + 1) / 2 : nblocks;
+    // A CTA that does not arrive may fall behind the others, which must not clear the
+    // counters that it has yet to read: every kAllArrive-th level is everyone's.
+    constexpr int kAllArrive = 32, kClearAhead = 4;
+    static_assert(kAllArrive + kClearAhead < kCtrRing, "no slot is cleared before the last CTA has read it");
+    const bool narrow = edges <= p.narrow_edges && nblocks >= 2 && k % kAllArrive != kAllArrive - 1;
+    const unsigned G = narrow ? (nblocks + 1) / 2 : nblocks;
     const bool part = blockIdx.x < G;
     const long long pthreads = (long long)G * kBlock;
 
     // recycle: counters of level k+4, bitmap of level k-1 (stores only; they
     // drain while the selector runs)
     if (blockIdx.x == 0 && tid < (int)(sizeof(LevelCtr) / 8))
-      reinterpret_cast<unsigned long long*>(&p.ctr[(k + 4) % kCtrRing])[tid] = 0ull;
+      reinterpret_cast<unsigned long long*>(&p.ctr[(k + kClearAhead) % kCtrRing])[tid] = 0ull;
     if (k >= 1 && part) {
       uint32_t* clr = p.bits[(k + 2) % 3];
       if (sparse_clr) {
