@@ -1049,7 +1049,7 @@ struct FetchMlp {
 // by threads or warps.  The heuristic runs only levels of at most 32 edges a warp that
 // way, and the network's choices at large levels are others.  Six roots on 2^27 edges,
 // every level by threads and by warps, ms per root: edgefactor 4 15.2 -> 11.1 and 13.1 ->
-// 7.6, 8 7.9 -> 7.8 and 6.5 -> 6.1, 16 6.7 -> 6.6 and 4.5 (with a buffer of 6,144 entries in
+// 7.6, 8 7.9 -> 7.8 and 6.5 -> 6.0, 16 6.7 and 4.5 as before (with a buffer of 6,144 entries in
 // every instance, which took L1 from every phase, edgefactor 4 took 14.0 and 11.9).
 template <bool kTiles, bool kLearned, bool kLong>
 __global__ void __launch_bounds__(kBlock, 2) level_loop_kernel(LoopParams p) {
