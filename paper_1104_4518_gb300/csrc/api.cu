@@ -146,6 +146,7 @@ int dev_alloc(void** p, size_t bytes, const char* what) {
     }
   }
   cudaError_t e = cudaMalloc(p, need);
+  if (here.context == 0) here.context = current_context();  // the thread's first call made it current
   if (e == cudaErrorMemoryAllocation) {  // give back what the cache holds and try once more
     cudaGetLastError();
     for (void* q : take_idle(here, std::chrono::steady_clock::duration::zero())) cudaFree(q);
@@ -158,7 +159,6 @@ int dev_alloc(void** p, size_t bytes, const char* what) {
                 std::string("device allocation of ") + std::to_string(bytes) + " bytes for " + what + " failed: " +
                     cudaGetErrorString(e));
   }
-  if (here.context == 0) here.context = current_context();  // the thread's first call made it current
   std::lock_guard<std::mutex> lk(g_mem_mu);
   g_mem_used[*p] = {need, here.device, here.context};
   return BFS_OK;

@@ -3,7 +3,8 @@
 // copies and fills happen at once, kernels are recorded and not run.  Every
 // call that allocates, frees, fills, copies, launches or waits goes to a log
 // with its pointer, size and stream; allocations and device synchronisations
-// can be made to fail.  fake_* are the test's own entry points.
+// can be made to fail, and fills and copies on a captured stream are only
+// recorded.  fake_* are the test's own entry points.
 #include <cuda_runtime_api.h>
 #include <sys/mman.h>
 
@@ -30,7 +31,8 @@ size_t reported_total = (size_t)64 << 30;                       // what cudaMemG
 long long mallocs_left = -1;  // allocations that still succeed (negative: all)
 cudaError_t sync_error = cudaSuccess;
 int device = 0;
-unsigned long long context = 1;
+unsigned long long context = 1;  // 0: none is current yet; the next allocation makes one
+cudaStream_t captured = nullptr;  // the stream being captured
 thread_local struct { dim3 grid, block; size_t smem; void* stream; } config;
 
 void note(const char* what, const void* p = nullptr, size_t bytes = 0, void* stream = nullptr) {
@@ -51,6 +53,7 @@ FAKE void fake_set_mallocs_left(long long n) { mallocs_left = n; }
 FAKE void fake_sync_error(int e) { sync_error = (cudaError_t)e; }
 FAKE void fake_set_device(int d) { device = d; }
 FAKE void fake_set_context(unsigned long long id) { context = id; }
+FAKE void fake_set_captured(void* s) { captured = (cudaStream_t)s; }
 FAKE void fake_set_total(size_t b) { total_bytes = b; }
 FAKE void fake_set_reported_total(size_t b) { reported_total = b; }
 FAKE size_t fake_live_bytes() {
@@ -63,6 +66,7 @@ FAKE size_t fake_live_bytes() {
 CUDA cudaMalloc(void** p, size_t bytes) {
   std::lock_guard<std::recursive_mutex> lk(mu);
   *p = nullptr;
+  if (context == 0) context = 1;
   if (mallocs_left == 0 || live_bytes + bytes > total_bytes) {
     note("malloc failed", nullptr, bytes);
     return cudaErrorMemoryAllocation;
@@ -93,10 +97,12 @@ CUDA cudaFreeHost(void* p) { return free(p), cudaSuccess; }
 CUDA cudaMemGetInfo(size_t* f, size_t* t) { return *f = total_bytes - live_bytes, *t = reported_total, cudaSuccess; }
 namespace {
 cudaError_t fill(void* p, int v, size_t n, void* s) {
+  if (s && s == captured) return note("recorded", p, n, s), cudaSuccess;
   if (n && !p) return note("memset failed", p, n, s), cudaErrorInvalidValue;
   return memset(p, v, n), note("memset", p, n, s), cudaSuccess;
 }
 cudaError_t copy(void* d, const void* from, size_t n, void* s) {
+  if (s && s == captured) return note("recorded", d, n, s), cudaSuccess;
   if (n && (!d || !from)) return note("memcpy failed", d, n, s), cudaErrorInvalidValue;
   return memcpy(d, from, n), note("memcpy", d, n, s), cudaSuccess;
 }
@@ -106,7 +112,13 @@ CUDA cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t s) { return fill(p, 
 CUDA cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { return copy(d, s, n, nullptr); }
 CUDA cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t st) { return copy(d, s, n, st); }
 CUDA cudaDeviceSynchronize() { return note("device sync"), sync_error; }
-CUDA cudaStreamSynchronize(cudaStream_t s) { return note("stream sync", nullptr, 0, s), cudaSuccess; }
+CUDA cudaStreamSynchronize(cudaStream_t s) {
+  if (s && s == captured) return cudaErrorStreamCaptureUnsupported;
+  return note("stream sync", nullptr, 0, s), cudaSuccess;
+}
+CUDA cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* st) {
+  return *st = s && s == captured ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone, cudaSuccess;
+}
 CUDA cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return *s = (cudaStream_t)malloc(1), cudaSuccess; }
 CUDA cudaStreamDestroy(cudaStream_t s) { return free(s), cudaSuccess; }
 CUDA cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
@@ -117,7 +129,7 @@ CUDA cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 CUDA cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 CUDA cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { return *ms = 1.0f, cudaSuccess; }
 CUDA cudaGetDevice(int* d) { return *d = device, cudaSuccess; }
-CUDA cudaSetDevice(int d) { return device = d, cudaSuccess; }
+CUDA cudaSetDevice(int d) { return device = d, note("set device"), cudaSuccess; }
 CUDA cudaGetLastError() { return cudaSuccess; }
 extern "C" __attribute__((visibility("default"))) const char* cudaGetErrorString(cudaError_t) { return "fake error"; }
 extern "C" __attribute__((visibility("default"))) const char* cudaGetErrorName(cudaError_t) { return "fakeError"; }

@@ -96,6 +96,17 @@ def test_a_failed_allocation_takes_the_idle_blocks_first(lib):
     assert log[at + 1] == "free" and "malloc" in log[at:]
 
 
+def test_a_failed_first_allocation_of_a_thread_takes_the_idle_blocks_too(lib):
+    """No context is current in a thread before its first call; the allocation makes it so, and then the idle blocks
+    can be told to be its own."""
+    cycle(lib, 20 * N)
+    lib.c.fake_set_total(ctypes.c_size_t(400000))
+    lib.c.fake_set_context(ctypes.c_ulonglong(0))
+    log = whats(lib.taken(lambda: lib.graph(20 * N)))
+    at = log.index("malloc failed")
+    assert log[at + 1] == "free" and "malloc" in log[at:]
+
+
 def test_release_with_another_device_current(lib):
     """A block of another device is not idle after a wait for the current one; and a device gets its own blocks only."""
     g = lib.graph(N)
