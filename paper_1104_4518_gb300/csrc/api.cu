@@ -692,13 +692,15 @@ int bfs_memory_trim(void) {
   BFS_CUDA_TRY(cudaGetDevice(&current));
   cudaError_t err = cudaSuccess;
   for (int d : devices) {
-    cudaError_t e = cudaSetDevice(d);
+    // cudaSetDevice would replace a current context that is not the device's primary one; cudaFree(nullptr) leaves it,
+    // and makes the primary one current in a thread without any
+    cudaError_t e = d == current ? cudaFree(nullptr) : cudaSetDevice(d);
     if (e == cudaSuccess)
       for (void* p : take_idle(Here{}, std::chrono::steady_clock::duration::zero()))
         if (cudaError_t f = cudaFree(p); f != cudaSuccess) e = f;
+    if (d != current && cudaSetDevice(current) != cudaSuccess && e == cudaSuccess) e = cudaErrorInvalidDevice;
     if (e != cudaSuccess) err = e;
   }
-  if (!devices.empty() && cudaSetDevice(current) != cudaSuccess && err == cudaSuccess) err = cudaErrorInvalidDevice;
   return err == cudaSuccess ? BFS_OK : cuda_fail(err, "bfs_memory_trim");
 }
 

@@ -31,7 +31,7 @@ size_t reported_total = (size_t)64 << 30;                       // what cudaMemG
 long long mallocs_left = -1;  // allocations that still succeed (negative: all)
 cudaError_t sync_error = cudaSuccess;
 int device = 0;
-unsigned long long context = 1;  // 0: none is current yet; the next allocation makes one
+unsigned long long context = 1;  // 0: none is current yet; the next allocation or release makes one
 cudaStream_t captured = nullptr;  // the stream being captured
 thread_local struct { dim3 grid, block; size_t smem; void* stream; } config;
 
@@ -83,6 +83,7 @@ CUDA cudaMalloc(void** p, size_t bytes) {
 }
 CUDA cudaFree(void* p) {
   std::lock_guard<std::recursive_mutex> lk(mu);
+  if (context == 0) context = 1;
   if (!p) return cudaSuccess;
   auto it = live.find(p);
   if (it == live.end()) return note("free failed", p), cudaErrorInvalidValue;

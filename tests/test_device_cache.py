@@ -107,6 +107,16 @@ def test_a_failed_first_allocation_of_a_thread_takes_the_idle_blocks_too(lib):
     assert log[at + 1] == "free" and "malloc" in log[at:]
 
 
+def test_request_leaves_the_current_context_alone(lib):
+    """With all idle blocks on the current device there is no need to make another context current."""
+    cycle(lib)
+    log = lib.taken(lambda: lib.c.bfs_memory_trim())
+    assert "set device" not in whats(log) and lib.c.fake_live_bytes() == 0
+    cycle(lib)
+    lib.c.fake_set_context(ctypes.c_ulonglong(0))  # in a thread that has made no call yet
+    assert lib.c.bfs_memory_trim() == 0 and lib.c.fake_live_bytes() == 0
+
+
 def test_release_with_another_device_current(lib):
     """A block of another device is not idle after a wait for the current one; and a device gets its own blocks only."""
     g = lib.graph(N)
