@@ -186,6 +186,20 @@ void dev_free(void* p) {
   trim_device_cache(here);
 }
 
+SetupStream::SetupStream(cudaStream_t s) : stream_(s) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  status_ = cudaStreamIsCapturing(s, &capture);
+  if (status_ != cudaSuccess || capture == cudaStreamCaptureStatusNone) return;
+  status_ = cudaStreamCreateWithFlags(&stream_, cudaStreamNonBlocking);
+  own_ = status_ == cudaSuccess;
+}
+
+SetupStream::~SetupStream() {
+  if (own_) cudaStreamDestroy(stream_);
+}
+
+cudaError_t SetupStream::done(bool finish) { return own_ || finish ? cudaStreamSynchronize(stream_) : cudaSuccess; }
+
 int current_device_info(DeviceInfo* out) {
   static thread_local DeviceInfo cache[64];
   int dev = 0;
@@ -281,9 +295,12 @@ int get_workspace(bfs_graph* g, cudaStream_t s, Workspace** out) {
   }
   if (!rc) {
     // on s: a non-blocking stream would not wait for fills on the default stream
-    cudaError_t e = cudaMemsetAsync(w->barrier, 0, 2 * sizeof(bfsdev::GridBarrier), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w->status, 0, sizeof(int) * 4, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w->ctr, 0, sizeof(LevelCtr) * kCtrRing, s);
+    SetupStream setup(s);
+    cudaError_t e = setup.status();
+    if (e == cudaSuccess) e = cudaMemsetAsync(w->barrier, 0, 2 * sizeof(bfsdev::GridBarrier), setup);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w->status, 0, sizeof(int) * 4, setup);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w->ctr, 0, sizeof(LevelCtr) * kCtrRing, setup);
+    if (e == cudaSuccess) e = setup.done(false);
     if (e != cudaSuccess) rc = cuda_fail(e, "workspace initialisation");
   }
   if (rc) {

@@ -32,6 +32,26 @@ int dev_alloc(void** p, size_t bytes, const char* what);
 // Waits for the device, then releases a block (null: nothing) to the library's cache or to the driver.
 void dev_free(void* p);
 
+// The stream for work that later launches of any capture or none rely on: the
+// caller's, or while that is being captured, when work on it would only be
+// recorded, one of its own.
+class SetupStream {
+ public:
+  explicit SetupStream(cudaStream_t s);
+  ~SetupStream();
+  SetupStream(const SetupStream&) = delete;
+  SetupStream& operator=(const SetupStream&) = delete;
+  operator cudaStream_t() const { return stream_; }
+  cudaError_t status() const { return status_; }
+  // Orders the work before what is launched on the caller's stream next; `finish` waits for it in any case.
+  cudaError_t done(bool finish);
+
+ private:
+  cudaStream_t stream_;
+  bool own_ = false;
+  cudaError_t status_;
+};
+
 // ---------------- device properties ----------------
 struct DeviceInfo {
   int device = -1;

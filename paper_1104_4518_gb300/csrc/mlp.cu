@@ -367,8 +367,10 @@ const float* learned_params_device(cudaStream_t s) {
     float* p = nullptr;
     if (dev_alloc((void**)&p, sizeof(float) * BFS_MLP_PARAMS, "selector parameters") != BFS_OK) return nullptr;
     // there before any stream reads them: a pageable copy may still be on its way when the call returns
-    if (cudaMemcpyAsync(p, warp.data(), sizeof(float) * BFS_MLP_PARAMS, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess) {
+    SetupStream setup(s);
+    if (setup.status() != cudaSuccess ||
+        cudaMemcpyAsync(p, warp.data(), sizeof(float) * BFS_MLP_PARAMS, cudaMemcpyHostToDevice, setup) != cudaSuccess ||
+        setup.done(true) != cudaSuccess) {
       dev_free(p);
       return nullptr;
     }

@@ -107,3 +107,20 @@ def test_copying_the_rows_out_waits_for_the_copies(lib):
     copies = [i for i, e in enumerate(log) if e.what == "memcpy"]
     assert len(copies) == 2
     assert any(e.what == "stream sync" and e.stream == log[copies[-1]].stream for e in log[copies[-1]:])
+
+
+def test_first_run_on_a_captured_stream(lib):
+    """Work on a captured stream happens when the graph is launched, if ever; what a workspace and the selector's
+    parameters start from has to be there for every later run as well."""
+    import paper_1104_4518_gb300 as bfs
+    g = lib.graph()
+    assert lib.c.bfs_selector_set_params((ctypes.c_float * bfs.BFS_MLP_PARAMS)()) == 0
+    o = bfs.bfs_opts(selector=bfs.BFS_SELECT_LEARNED)
+    lib.c.fake_set_captured(ctypes.c_void_p(S))
+    log = lib.taken(lambda: setattr(lib, "rc", lib.run(g, 100, S, ctypes.byref(o))))
+    lib.c.fake_set_captured(None)
+    assert lib.rc == 0, lib.c.bfs_last_error()
+    done = [(i, e) for i, e in enumerate(log) if e.what in ("memset", "memcpy")]
+    assert {16, 128 * 2} <= {e.bytes for _, e in done} and 4 * bfs.BFS_MLP_PARAMS in {e.bytes for _, e in done}
+    for i, e in done:
+        assert e.stream != S and any(x.what == "stream sync" and x.stream == e.stream for x in log[i:])
